@@ -75,6 +75,13 @@ struct lqcd_ctx {
   int tc_stop_after;         // injected stall of the next tensor-core launch (-1: none)
   int inner_gs_passes;       // Gram-Schmidt passes of the reduced-precision inner Arnoldi (0 = by storage)
   int probe_depth;           // full applications of P per probe in the hopping traces (0 = by cost)
+  // converted links of the fixed-point FP64 operator (workspace WS_FX_LINKS): the gauge field they were
+  // made from in the running call (nullptr: none), the depth of nested scopes that keep them, and
+  // the end of their last use with its stream (a later call on another stream waits for it)
+  const void *fx_src;
+  int fx_depth;
+  cudaEvent_t fx_event;
+  cudaStream_t fx_event_stream;
   int inner_window;          // Lanczos window of Hermitian mixed-precision inner cycles (0 = full Gram-Schmidt)
   // even/odd reduced context (lqcd_ctx_create_evenodd): fields hold the even sites only (V above is
   // half the lattice), the operator is hat M = 1 - kappa^2 P_eo P_oe, eo_dims the full extents
@@ -130,7 +137,7 @@ enum WsSlot {
   WS_PARTIAL = 0, WS_SCAL, WS_TMP0, WS_TMP1, WS_TMP2, WS_TMP3, WS_BASIS, WS_HESS, WS_COEF,
   WS_BASIS2, WS_TMP4, WS_TMP5, WS_EST0, WS_EST1, WS_EST2, WS_PROBE,
   WS_MIX_U, WS_MIX_V, WS_MIX_R32, WS_MIX_E32, WS_MIX_R, WS_MIX_S, WS_COUNT, WS_TUNE, WS_SPEC, WS_NBLK, WS_TC_STAT, WS_TC_B, WS_TC_PART, WS_TC_D,
-  WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_NSLOTS
+  WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_FX_LINKS, WS_FX_FIELD, WS_NSLOTS
 };
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr);
 void graph_cache_clear(lqcd_ctx *ctx);
@@ -144,6 +151,31 @@ lqcd_status graph_cached(lqcd_ctx *ctx, const std::string &key, lqcd_status (*en
 // sides and up to max_nvec basis vectors (so graph capture never grows a buffer).
 lqcd_status blas_reserve(lqcd_ctx *ctx, long long n, int nrhs, int max_nvec);
 lqcd_status host_stage(lqcd_ctx *ctx, size_t bytes, double **ptr);
+
+// Converted links of the fixed-point FP64 operator (fxhop.cuh).  fx_links gives those of U: converted now,
+// or earlier in the same outermost FxScope (one library call, during which the caller's gauge field does
+// not change; nothing is kept beyond it).  use = false: the caller runs the plain FP64 stencil, which
+// needs no workspace (a stream under the caller's capture, or no memory for the workspace).
+namespace fx { struct Links; struct Field; }
+lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use);
+// workspace for up to chunk fields of S sites in that form (use as above), and the conversion into it
+lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *chunk, bool *use);
+lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs);
+void fx_done(lqcd_ctx *ctx);   // records the end of a use (outside scopes; a scope does it at its end)
+struct FxScope {
+  lqcd_ctx *ctx;
+  explicit FxScope(lqcd_ctx *c) : ctx(c) {
+    if (ctx->fx_depth++ == 0) ctx->fx_src = nullptr;
+  }
+  ~FxScope() {
+    if (--ctx->fx_depth == 0) {
+      if (ctx->fx_src) fx_done(ctx);
+      ctx->fx_src = nullptr;
+    }
+  }
+  FxScope(const FxScope &) = delete;
+  FxScope &operator=(const FxScope &) = delete;
+};
 
 // ----- complex helpers (device) -----------------------------------------------------------
 __host__ __device__ __forceinline__ double2 cmake(double r, double i) { return make_double2(r, i); }

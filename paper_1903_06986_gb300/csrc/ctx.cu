@@ -221,6 +221,10 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
   c->inner_gs_passes = 0;
   c->probe_depth = 0;
   c->inner_window = 0;
+  c->fx_src = nullptr;
+  c->fx_depth = 0;
+  c->fx_event = nullptr;
+  c->fx_event_stream = nullptr;
   c->eo = 0;
   for (int i = 0; i < 4; ++i) c->eo_dims[i] = dims[i];
   c->cap_stream = nullptr;
@@ -246,6 +250,10 @@ lqcd_status lqcd_ctx_destroy(lqcd_ctx *ctx) {
   for (void *p : ctx->ws_ptr)
     if (p) cudaFree(p);
   if (ctx->host_pinned) cudaFreeHost(ctx->host_pinned);
+  if (ctx->fx_event) {
+    cudaEventSynchronize(ctx->fx_event);
+    cudaEventDestroy(ctx->fx_event);
+  }
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
   delete ctx;
   return LQCD_OK;

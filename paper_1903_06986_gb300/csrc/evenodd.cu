@@ -14,9 +14,12 @@
 // dims (Lx/2, Ly, Lz, Lt), so its field length 12 V/2 is what every level-1/2 kernel and Krylov
 // solver of the library already works with; its Wilson operator is hat M (two hopping launches
 // through a workspace odd field), taking the full links [mu][V][3][3].
+#include <algorithm>
 #include <complex>
+#include <type_traits>
 
 #include "common.cuh"
+#include "fxhop.cuh"
 #include "spin.cuh"
 
 using cd = std::complex<double>;
@@ -116,6 +119,36 @@ __global__ void __launch_bounds__(128) eo_hop_kernel(const double2 *__restrict__
     for (int c = 0; c < 3; ++c) store_c(dst + 3 * a + c, o[a][c]);
 }
 
+// The FP64 form of the same on the fixed-point hopping term (fxhop.cuh); one site and right-hand side
+// per thread, right-hand side blockIdx.x % nrhs; f holds the integers of in
+constexpr int EO_FX_BS = 128;
+struct EoTorus : fx::Torus {
+  __device__ __forceinline__ EoTorus(int lx, int ly, int lz, int lt, int i, int par) : fx::Torus(lx >> 1, ly, lz, lt, i) {
+    Lx = lx;
+    x = 2 * x + ((y + z + t + par) & 1);
+    s = x + Lx * (y + Ly * (z + Lz * t));
+  }
+};
+template <int FL, int SPLIT>
+__global__ void __launch_bounds__(EO_FX_BS, 4) eo_hop_fx_kernel(const double2 *__restrict__ U, fx::Links L, fx::Field f,
+                                                                const double2 *__restrict__ in,
+                                                                const double2 *__restrict__ self,
+                                                                double2 *__restrict__ out, double coef, int Lx, int Ly,
+                                                                int Lz, int Lt, int Vh, int nrhs, int par) {
+  __shared__ __align__(16) char sm[fx::SMEM_BYTES<SPLIT>];
+  const long long r = blockIdx.x % nrhs;
+  const int i0 = (blockIdx.x / nrhs) * (EO_FX_BS / SPLIT) + threadIdx.x % (EO_FX_BS / SPLIT);
+  const int i = min(i0, Vh - 1);
+  const EoTorus nb(Lx, Ly, Lz, Lt, i, par);
+  const long long V = 2LL * Vh, S = (FL & EO_IN_FULL) ? V : Vh, Ss = (FL & EO_SELF_FULL) ? V : Vh,
+                  So = (FL & EO_OUT_FULL) ? V : Vh;
+  fx::run<SPLIT, !(FL & EO_IN_FULL)>(sm, U, L, V, nb.s, (const fx::Torus &)nb, f, (int)r, S, in + r * S * 12,
+                                     (FL & EO_HOP_G5) != 0, (FL & EO_SELF) ? self + r * Ss * 12 : nullptr,
+                                     (FL & EO_SELF_FULL) ? nb.s : i, (FL & EO_SELF_G5) != 0, coef,
+                                     (FL & EO_LEFT_G5) != 0, out + r * So * 12,
+                                     i0 >= Vh ? -1 : (FL & EO_OUT_FULL) ? nb.s : i);
+}
+
 // full field <-> (even, odd) compact fields; either compact pointer may be NULL (not copied)
 template <bool SPLIT>
 __global__ void eo_copy_kernel(double2 *__restrict__ full, double2 *__restrict__ ev, double2 *__restrict__ od, int Lx,
@@ -162,14 +195,40 @@ __global__ void eo_pair_kernel(const double2 *__restrict__ ve, const double2 *__
 template <typename R, int FL>
 lqcd_status hop_launch(lqcd_ctx *ctx, const double2 *U, const double2 *in, const double2 *self, double2 *out,
                        double coef, int nrhs, int par) {
+  const int *d = ctx->eo_dims;
+  // compulsory bytes: the input half read, the output half written (plus the added half), links once
+  const double bytes = (2.0 + ((FL & EO_SELF) ? 1.0 : 0.0)) * nrhs * ctx->V * 12 * 16.0 + 36.0 * 2 * ctx->V * 16.0;
+  if constexpr (std::is_same<R, double>::value) {
+    fx::Links L;
+    fx::Field f;
+    bool use;
+    int chunk;
+    const long long S = (FL & EO_IN_FULL) ? 2LL * ctx->V : ctx->V;
+    const long long So = (FL & EO_OUT_FULL) ? 2LL * ctx->V : ctx->V, Ss = (FL & EO_SELF_FULL) ? 2LL * ctx->V : ctx->V;
+    LQCD_TRY(fx_links(ctx, U, &L, &use));
+    if (use) LQCD_TRY(fx_field(ctx, S, nrhs, &f, &chunk, &use));
+    if (use) {
+      for (int r0 = 0; r0 < nrhs; r0 += chunk) {
+        const int nr = std::min(chunk, nrhs - r0);
+        const double2 *src = in + 12 * S * r0;
+        LQCD_TRY(fx_convert(ctx, src, f, S, nr));
+        const bool split = fx::use_split(ctx->V, nr, ctx->sms);
+        kbegin(ctx);
+        (split ? eo_hop_fx_kernel<FL, 4> : eo_hop_fx_kernel<FL, 1>)
+            <<<(unsigned)((long long)ceil_div(ctx->V, split ? 32 : EO_FX_BS) * nr), EO_FX_BS, 0, ctx->stream>>>(
+                U, L, f, src, self ? self + 12 * Ss * r0 : nullptr, out + 12 * So * r0, coef, d[0], d[1], d[2], d[3],
+                ctx->V, nr, par);
+        LQCD_TRY(launch_check_bytes(ctx, "eo_hop_fx_kernel", K_WILSON, (double)ctx->V * nr, bytes * nr / nrhs));
+      }
+      if (ctx->fx_depth == 0) fx_done(ctx);
+      return LQCD_OK;
+    }
+  }
   int bs = 128;
   while (bs > 32 && (long long)ceil_div(ctx->V, bs) * nrhs < 2LL * ctx->sms) bs /= 2;
-  const int *d = ctx->eo_dims;
   kbegin(ctx);
   eo_hop_kernel<R, FL><<<dim3(ceil_div(ctx->V, bs), nrhs), bs, 0, ctx->stream>>>(U, in, self, out, coef, d[0], d[1],
                                                                                d[2], d[3], ctx->V, par);
-  // compulsory bytes: the input half read, the output half written (plus the added half), links once
-  const double bytes = (2.0 + ((FL & EO_SELF) ? 1.0 : 0.0)) * nrhs * ctx->V * 12 * 16.0 + 36.0 * 2 * ctx->V * 16.0;
   return launch_check_bytes(ctx, "eo_hop_kernel", K_WILSON, (double)ctx->V * nrhs, bytes);
 }
 
@@ -195,6 +254,7 @@ lqcd_status check_nrhs(lqcd_ctx *ctx, int nrhs, const char *what) {
 template <typename R>
 lqcd_status eo_schur_launch_t(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out,
                               int nrhs, int flags) {
+  FxScope scope(ctx);   // two hopping launches, one conversion of the links
   double2 *tmp;
   LQCD_TRY(ws_get(ctx, WS_EO, sizeof(double2) * (size_t)nrhs * ctx->N, (void **)&tmp));
   const double k2 = -kappa * kappa;

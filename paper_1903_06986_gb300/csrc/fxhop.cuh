@@ -1,0 +1,468 @@
+// The hopping term of the FP64 Wilson operator in block fixed point on the integer pipes.
+//
+// What bounds the plain form: an SM issues two FP64 operations per clock and the stencil needs
+// about 860 per (site, right-hand side): 430 clocks, 6.6 ms for ten fields of 24^3 x 32, against
+// 0.3 ms of HBM traffic.  The same SM issues 64 32 x 32 -> 64-bit integer multiply-adds per clock
+// (measured: 59 mad.wide.s32 against 1.7 to 2 DFMA), so the stencil runs on integers:
+//   * fx_convert_kernel turns a field into integers once per application: a real x of a site whose
+//     largest real has biased exponent X becomes q = x 2^(1082 - X), |q| < 2^60 (the mantissa
+//     shifted by X - exponent; all 53 bits survive down to 2^-7 of the site's largest entry).
+//     Converting the half spinor of each direction inside the stencil (tried) costs 96 conversions
+//     of 15 instructions per site, and the two FP64 operations of each projection;
+//   * links become q_u = u 2^(1082 - X_u), once per call (fx_links_kernel);
+//   * spin projections are 64-bit additions; a half spinor is shifted right by E - X_u - X - 1 to the
+//     exponent E >= X_u + X + 2 that all eight directions of the thread share, leaving |h| < 2^60;
+//   * both factors are split as hi 2^32 + lo with signed lo: a product needs hi hi and
+//     (hi lo + lo hi) / 2^32, three mad.wide; lo lo / 2^64 is below half the unit that is kept.  Six
+//     products are summed exactly (|hi hi| sum < 2^59, |mixed| sum < 2^63), the mixed sum enters by
+//     its high word (one mad.wide), and the eight directions are added as 64-bit integers (< 2^62).
+// FP64 arithmetic is left with the last p - kappa acc (24 conversions, 24 DFMA).
+// Error: the kept unit is 2^-56 of (largest link entry x largest half spinor entry around the site),
+// below the roundings of the FP64 chain it replaces (tests/test_gpu_fxhop.py compares both with
+// extended precision).
+// Sites or links with a NaN, an Inf, or a scale near the ends of the exponent range carry the exponent
+// FX_BAD; the threads that meet one run the plain FP64 stencil.
+//
+// Layout: blocks of 32 sites, [block][component][site of the block] with 16 bytes each (components: the
+// 12 of a field; 9 entries of each of the four links), so that a warp reads 512 contiguous bytes and
+// one address serves all components; the canonical layout (192 bytes per site) would cost 32 cache
+// lines per load.  The canonical side goes through a warp-private shared buffer with 208 bytes per
+// site (conflict-free) in memory order.
+#pragma once
+
+#include "spin.cuh"
+
+namespace fx {
+
+using spin::Cx;
+using spin::mk;
+
+struct Links {
+  const int4 *q;   // [site / 32][mu 4][entry 9][site % 32]: (re hi, re lo, im hi, im lo)
+  const int *ex;   // [mu 4][site]: biased exponent X_u of the link's largest real, or FX_BAD
+};
+struct Field {
+  longlong2 *q;    // [right-hand side][site / 32][component 12][site % 32]
+  int *ex;         // [right-hand side][site]: X, or FX_BAD
+};
+__host__ __device__ __forceinline__ long long blocks32(long long S) { return (S + 31) >> 5; }
+// first component of site s in an array with per components per site
+__device__ __forceinline__ long long slot(int s, int per) { return (long long)(s >> 5) * (32 * per) + (s & 31); }
+constexpr int FX_BAD = 1 << 20;       // exponent that sends the thread to the FP64 stencil
+constexpr int FX_MINX = 64;           // X of a block of zeros (and the least a shift may start from)
+constexpr int FX_MIN_FIELD = 400, FX_MIN_LINK = 700;   // smaller non-zero blocks are FX_BAD
+constexpr int SITE_BYTES = 208;       // 192 + 16: lanes of a quarter warp fall on distinct banks
+constexpr int WARP_BYTES = 32 * SITE_BYTES;
+
+__device__ __forceinline__ unsigned long long shr64(unsigned long long a, int n) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));  // shifts above 63 give 0
+  return r;
+}
+__device__ __forceinline__ long long sar64(long long a, int n) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
+  return r;
+}
+// acc + a b: this form becomes one multiply-add; inline mad.wide.s32 becomes two instructions, and the
+// plain C++ product in between
+__device__ __forceinline__ long long madw(long long acc, int a, int b) {
+  long long p;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+  return acc + p;
+}
+
+// mantissa of x left aligned in 64 bits.  Zeros and denormals have exponent field 0, so that a shift
+// by base - exponent >= 64 (FX_MINX) takes their (wrong) implicit one out.
+__device__ __forceinline__ unsigned long long mantissa(double x) {
+  return (((unsigned long long)((__double2hiint(x) & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x)) << 11;
+}
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+// x -> trunc(x 2^(1086 - base)), base = X + 4 for 60 bits
+__device__ __forceinline__ long long fixed(double x, int base) {
+  const long long s = __double2hiint(x) >> 31;
+  return ((long long)shr64(mantissa(x), base - exponent(x)) ^ s) - s;
+}
+// q = hi 2^32 + lo with lo in [-2^31, 2^31)
+__device__ __forceinline__ void split(long long q, int &hi, int &lo) {
+  lo = (int)q;
+  hi = (int)(q >> 32) + (int)((unsigned)lo >> 31);
+}
+
+__device__ __forceinline__ void cp_async16(unsigned sa, const void *g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(g) : "memory");
+}
+__device__ __forceinline__ void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// Warp-private staging of 32 site blocks (12 double2 each): chunk i = lane + 32 j of the 384 belongs to
+// site i / 12, component i % 12; 96 chunks are 8 sites, so three (site, component) pairs serve all j.
+struct Stage {
+  int lane;
+  int site[3], comp[3];
+  unsigned sm;      // shared address of the warp's buffer
+  char *smp;
+  __device__ __forceinline__ void init(char *warp_smem) {
+    lane = threadIdx.x & 31;
+    smp = warp_smem;
+    sm = (unsigned)__cvta_generic_to_shared(warp_smem);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int i = lane + 32 * r;
+      site[r] = i / 12;
+      comp[r] = i - 12 * site[r];
+    }
+  }
+  // copy the 192-byte blocks of the lanes' sites m (each lane names its own) into the buffer
+  // (SPLIT = 4: warp part of the four that share the sites copies a quarter)
+  template <int SPLIT = 1>
+  __device__ __forceinline__ void load(const double2 *src, int m, int part = 0) const {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int j = 0; j < 4 / SPLIT; ++j) {
+        const int q = SPLIT == 1 ? j : part;
+        const int ms = __shfl_sync(0xffffffffu, m, site[r] + 8 * q);
+        cp_async16(sm + (site[r] + 8 * q) * SITE_BYTES + comp[r] * 16,
+                   src + (long long)ms * 12 + comp[r]);
+      }
+    commit();
+  }
+  // write the blocks of the buffer to the lanes' sites m of dst; lanes with m < 0 write nothing
+  template <int SPLIT = 1>
+  __device__ __forceinline__ void store(double2 *dst, int m, int part = 0) const {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int j = 0; j < 4 / SPLIT; ++j) {
+        const int q = SPLIT == 1 ? j : part;
+        const int ms = __shfl_sync(0xffffffffu, m, site[r] + 8 * q);
+        if (ms >= 0)
+          dst[(long long)ms * 12 + comp[r]] =
+              *(const double2 *)(smp + (site[r] + 8 * q) * SITE_BYTES + comp[r] * 16);
+      }
+  }
+  __device__ __forceinline__ double2 *mine() const {
+    return (double2 *)(smp + lane * SITE_BYTES);
+  }
+};
+
+struct Acc {
+  long long v[4][3][2];   // [spin][colour][re, im], unit 2^(E - 2101)
+  int E;
+  bool bad;
+};
+
+__device__ __forceinline__ void add2(long long a[2], long long re, long long im) { a[0] += re; a[1] += im; }
+
+// Adds direction d (2 mu: x + mu, 2 mu + 1: x - mu) to A: q: the field's integers at the neighbour, of
+// which the half spinor is shifted by sh; u: the link of direction mu; pu, pl: component offsets of
+// the upper and lower spin pair (exchanged: -gamma_5 times the field).  d is a run-time value, the
+// same in all threads: the loop over the directions stays rolled, since eight unrolled copies (100 kB
+// of instructions) missed the instruction cache on one issue in six.
+__device__ __forceinline__ void direction(int d, const longlong2 *__restrict__ q, int pu, int pl, int sh,
+                                          const int4 *__restrict__ u, Acc &A) {
+  const int mu = d >> 1, bwd = d & 1;
+  // half spinor (table at the head of spin.cuh), shifted and split; the t projection is 2 p of one pair
+  longlong2 h[2][3];
+  if (mu == 3) {
+    sh -= 1;
+    const longlong2 *p = q + (bwd ? pu : pl);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      h[0][c] = __ldg(p + c * 32);
+      h[1][c] = __ldg(p + (3 + c) * 32);
+    }
+  } else {
+    const longlong2 *p = q + pu, *w0 = q + pl + (mu == 2 ? 0 : 96), *w1 = q + pl + (mu == 2 ? 96 : 0);
+    longlong2 w[2][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      h[0][c] = __ldg(p + c * 32);
+      h[1][c] = __ldg(p + (3 + c) * 32);
+      w[0][c] = __ldg(w0 + c * 32);
+      w[1][c] = __ldg(w1 + c * 32);
+    }
+    // (h0, h1) += phases (i, i), (1, -1), (i, -i) of x, y, z, the negatives backward
+    switch (d) {
+#define LQCD_FX_CASE(D, X0, Y0, X1, Y1)                                     \
+  case D:                                                                   \
+    _Pragma("unroll") for (int c = 0; c < 3; ++c) {                         \
+      h[0][c].x += X0; h[0][c].y += Y0; h[1][c].x += X1; h[1][c].y += Y1;   \
+    }                                                                       \
+    break;
+      LQCD_FX_CASE(0, -w[0][c].y, w[0][c].x, -w[1][c].y, w[1][c].x)
+      LQCD_FX_CASE(1, w[0][c].y, -w[0][c].x, w[1][c].y, -w[1][c].x)
+      LQCD_FX_CASE(2, w[0][c].x, w[0][c].y, -w[1][c].x, -w[1][c].y)
+      LQCD_FX_CASE(3, -w[0][c].x, -w[0][c].y, w[1][c].x, w[1][c].y)
+      LQCD_FX_CASE(4, -w[0][c].y, w[0][c].x, w[1][c].y, -w[1][c].x)
+      default:
+      LQCD_FX_CASE(5, w[0][c].y, -w[0][c].x, -w[1][c].y, w[1][c].x)
+#undef LQCD_FX_CASE
+    }
+  }
+  int hi[2][3][2], lo[2][3][2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      split(sar64(h[k][c].x, sh), hi[k][c][0], lo[k][c][0]);
+      split(sar64(h[k][c].y, sh), hi[k][c][1], lo[k][c][1]);
+    }
+  // o_a = sum_b U_ab h_b (forward) or conj(U_ba) h_b (backward)
+  long long o[2][3][2];
+  const int4 *um = u + mu * 288;
+  const int ea = bwd ? 32 : 96, eb = bwd ? 96 : 32, cs = bwd ? -1 : 1;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    long long hh[2][2], md[2][2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        hh[k][z] = 0;
+        md[k][z] = 1ll << 31;   // rounds to the high word
+      }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 v = __ldg(um + a * ea + b * eb);
+      // (re, im) += (v_re, +-v_im) (h_re, h_im); v is the factor that is negated, since its lo is
+      // never -2^31 (fx_links_kernel)
+      const int ih = v.z * cs, il = v.w * cs, nh = -ih, nl = -il;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int rh = hi[k][b][0], rl = lo[k][b][0], mh = hi[k][b][1], ml = lo[k][b][1];
+        hh[k][0] = madw(hh[k][0], v.x, rh);
+        md[k][0] = madw(md[k][0], v.x, rl);
+        md[k][0] = madw(md[k][0], v.y, rh);
+        hh[k][0] = madw(hh[k][0], nh, mh);
+        md[k][0] = madw(md[k][0], nh, ml);
+        md[k][0] = madw(md[k][0], nl, mh);
+        hh[k][1] = madw(hh[k][1], v.x, mh);
+        md[k][1] = madw(md[k][1], v.x, ml);
+        md[k][1] = madw(md[k][1], v.y, mh);
+        hh[k][1] = madw(hh[k][1], ih, rh);
+        md[k][1] = madw(md[k][1], ih, rl);
+        md[k][1] = madw(md[k][1], il, rh);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) o[k][a][z] = madw(hh[k][z], (int)(md[k][z] >> 32), 1);
+  }
+  if (d != 6) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      add2(A.v[0][c], o[0][c][0], o[0][c][1]);
+      add2(A.v[1][c], o[1][c][0], o[1][c][1]);
+    }
+  }
+  // the lower pair is the upper one (exchanged for x and y) times the conjugate phases
+  switch (d) {
+#define LQCD_FX_CASE(D, X2, Y2, X3, Y3)                                                           \
+  case D:                                                                                         \
+    _Pragma("unroll") for (int c = 0; c < 3; ++c) {                                               \
+      const long long *o0 = o[0][c], *o1 = o[1][c];                                               \
+      add2(A.v[2][c], X2, Y2);                                                                    \
+      add2(A.v[3][c], X3, Y3);                                                                    \
+    }                                                                                             \
+    break;
+    LQCD_FX_CASE(0, o1[1], -o1[0], o0[1], -o0[0])
+    LQCD_FX_CASE(1, -o1[1], o1[0], -o0[1], o0[0])
+    LQCD_FX_CASE(2, -o1[0], -o1[1], o0[0], o0[1])
+    LQCD_FX_CASE(3, o1[0], o1[1], -o0[0], -o0[1])
+    LQCD_FX_CASE(4, o0[1], -o0[0], -o1[1], o1[0])
+    LQCD_FX_CASE(5, -o0[1], o0[0], o1[1], -o1[0])
+    LQCD_FX_CASE(6, o0[0], o0[1], o1[0], o1[1])
+#undef LQCD_FX_CASE
+    default: break;
+  }
+}
+
+// A = sum over the directions d0 .. d1 - 1 of the hopping term at link-lattice site s for right-hand side
+// r of the field f (S sites), at the exponent E of all eight; with g5 the spins are read exchanged, which is -gamma_5 times the field
+// (finish flips the sign).  nbr(d): link-lattice index of the neighbour; COMPACT: the field holds one
+// parity (index = neighbour >> 1).
+template <bool COMPACT, typename Nbr>
+__device__ __forceinline__ void hop(const Field &f, int r, long long S, bool g5, const Links &L, long long VL, int s,
+                                    const Nbr &nbr, int d0, int d1, Acc &A) {
+  const longlong2 *q = f.q + (long long)r * blocks32(S) * 384;
+  const int *ex = f.ex + (long long)r * S;
+  A.E = 0;
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    const int n = nbr(d);
+    A.E = max(A.E, __ldg(ex + (COMPACT ? n >> 1 : n)) + __ldg(L.ex + (d >> 1) * VL + ((d & 1) ? n : s)) + 2);
+  }
+  A.bad = A.E > 2900;   // FX_BAD among them, or kappa 2^(E - 2101) without room to the end of the range
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) A.v[a][c][0] = A.v[a][c][1] = 0;
+#pragma unroll 1
+  for (int d = d0; d < d1; ++d) {
+    const int n = nbr(d), m = COMPACT ? n >> 1 : n, l = (d & 1) ? n : s;
+    const int X = __ldg(ex + m) + __ldg(L.ex + (d >> 1) * VL + l);
+    direction(d, q + slot(m, 12), g5 ? 192 : 0, g5 ? 0 : 192, A.E - X - 1, L.q + slot(l, 36), A);
+  }
+}
+
+// The same sum in FP64 (bad threads), with the factor -gamma_5 that g5 stands for
+template <bool COMPACT, typename Nbr>
+__device__ __noinline__ void hop_fp64(const double2 *U, const double2 *src, long long VL, int s, bool g5, Nbr nbr,
+                                      double2 *out) {
+  using namespace spin;
+  Cx<double> acc[4][3], p[4][3], u[9];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc[a][c] = mk<double>(0.0, 0.0);
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d) {
+    const int n = nbr(d);
+    load_spinor<double, false>(src + 12LL * (COMPACT ? n >> 1 : n), p);
+    if (g5) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const Cx<double> v = p[a][c];
+          p[a][c] = p[a + 2][c];
+          p[a + 2][c] = v;
+        }
+    }
+    load_link<double>(U, (d >> 1) * VL + ((d & 1) ? n : s), u);
+    switch (d) {
+      case 0: term_fwd<double, 0>(p, u, acc); break;
+      case 1: term_bwd<double, 0>(p, u, acc); break;
+      case 2: term_fwd<double, 1>(p, u, acc); break;
+      case 3: term_bwd<double, 1>(p, u, acc); break;
+      case 4: term_fwd<double, 2>(p, u, acc); break;
+      case 5: term_bwd<double, 2>(p, u, acc); break;
+      case 6: term_fwd<double, 3>(p, u, acc); break;
+      default: term_bwd<double, 3>(p, u, acc); break;
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[3 * a + c] = make_double2(acc[a][c].x, acc[a][c].y);
+}
+
+// Neighbours of a site on a periodic Lx x Ly x Lz x Lt lattice
+struct Torus {
+  int Lx, Ly, Lz, Lt, x, y, z, t, s;
+  __device__ __forceinline__ Torus(int lx, int ly, int lz, int lt, int site) : Lx(lx), Ly(ly), Lz(lz), Lt(lt), s(site) {
+    x = s % Lx;
+    int q = s / Lx;
+    y = q % Ly;
+    q /= Ly;
+    z = q % Lz;
+    t = q / Lz;
+  }
+  __device__ __forceinline__ int operator()(int d) const {
+    switch (d) {
+      case 0: return x + 1 == Lx ? s - (Lx - 1) : s + 1;
+      case 1: return x == 0 ? s + (Lx - 1) : s - 1;
+      case 2: return y + 1 == Ly ? s - (Ly - 1) * Lx : s + Lx;
+      case 3: return y == 0 ? s + (Ly - 1) * Lx : s - Lx;
+      case 4: return z + 1 == Lz ? s - (Lz - 1) * Lx * Ly : s + Lx * Ly;
+      case 5: return z == 0 ? s + (Lz - 1) * Lx * Ly : s - Lx * Ly;
+      case 6: return t + 1 == Lt ? s - (Lt - 1) * Lx * Ly * Lz : s + Lx * Ly * Lz;
+      default: return t == 0 ? s + (Lt - 1) * Lx * Ly * Lz : s - Lx * Ly * Lz;
+    }
+  }
+};
+
+// Shared bytes of a block of 128 threads in run
+template <int SPLIT> constexpr int SMEM_BYTES = SPLIT == 1 ? 4 * WARP_BYTES : WARP_BYTES + 4 * 24 * 32 * 8;
+
+// One application for this thread: out[out_i] = self[self_i] + coef * hopping term (self may be NULL; the
+// gamma_5 flags: on the hopping input, on self, on the result).  src: the canonical field f was
+// converted from.  A lane with out_i < 0 (its site repeats another's) helps and stores nothing.
+// SPLIT = 1: one thread per site.  SPLIT = 4, for fields that leave most of the chip idle: the four
+// warps of a block share 32 sites, warp w adds the two directions of mu = w and finishes spin w; the
+// sums are integers at one exponent, so both forms give the same bits.
+template <int SPLIT, bool COMPACT, typename Nbr>
+__device__ __forceinline__ void run(char *smem, const double2 *U, const Links &L, long long VL, int s, const Nbr &nbr,
+                                    const Field &f, int r, long long S, const double2 *src, bool g5,
+                                    const double2 *self, int self_i, bool self_g5, double coef, bool left_g5,
+                                    double2 *out, int out_i) {
+  const int warp = threadIdx.x >> 5;
+  Stage st;
+  st.init(smem + (SPLIT == 1 ? warp * WARP_BYTES : 0));
+  if (self) st.load<SPLIT>(self, self_i, warp);
+  Acc A;
+  hop<COMPACT>(f, r, S, g5, L, VL, s, nbr, SPLIT == 1 ? 0 : 2 * warp, SPLIT == 1 ? 8 : 2 * warp + 2, A);
+  // E is above 1100 unless every block was zero (FX_MIN_FIELD, FX_MIN_LINK); the exchanged spins of g5
+  // are -gamma_5 times the field
+  const double sc = g5 ? -coef : coef;
+  const double k = A.E > 1080 ? sc * __hiloint2double((A.E - 2101 + 1023) << 20, 0) : 0.0;
+  double2 *m = st.mine();
+  if constexpr (SPLIT == 1) {
+    double2 p[12];
+    wait_all();
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 12; ++i)
+      p[i] = !self ? make_double2(0.0, 0.0) : self_g5 ? make_double2(-m[(i + 6) % 12].x, -m[(i + 6) % 12].y) : m[i];
+    __syncwarp();
+    if (!A.bad) {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) {
+        p[i].x = fma(k, (double)A.v[i / 3][i % 3][0], p[i].x);
+        p[i].y = fma(k, (double)A.v[i / 3][i % 3][1], p[i].y);
+      }
+    } else {
+      hop_fp64<COMPACT>(U, src, VL, s, g5, nbr, m);
+#pragma unroll
+      for (int i = 0; i < 12; ++i) p[i] = make_double2(fma(sc, m[i].x, p[i].x), fma(sc, m[i].y, p[i].y));
+    }
+#pragma unroll
+    for (int i = 0; i < 12; ++i) m[i] = left_g5 ? make_double2(-p[(i + 6) % 12].x, -p[(i + 6) % 12].y) : p[i];
+    __syncwarp();
+    st.store<SPLIT>(out, out_i);
+  } else {
+    long long *red = (long long *)(smem + WARP_BYTES);   // [warp][real 24][lane 32]
+#pragma unroll
+    for (int i = 0; i < 24; ++i) red[(warp * 24 + i) * 32 + st.lane] = A.v[i / 6][i / 2 % 3][i & 1];
+    wait_all();
+    __syncthreads();
+    double2 p[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int i = 3 * warp + c;
+      p[c] = !self ? make_double2(0.0, 0.0) : self_g5 ? make_double2(-m[(i + 6) % 12].x, -m[(i + 6) % 12].y) : m[i];
+      long long re = 0, im = 0;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        re += red[(w * 24 + 2 * i) * 32 + st.lane];
+        im += red[(w * 24 + 2 * i + 1) * 32 + st.lane];
+      }
+      if (!A.bad) p[c] = make_double2(fma(k, (double)re, p[c].x), fma(k, (double)im, p[c].y));
+    }
+    if (A.bad) {
+      double2 full[12];
+      hop_fp64<COMPACT>(U, src, VL, s, g5, nbr, full);
+#pragma unroll
+      for (int i = 0; i < 12; ++i)
+        if (i / 3 == warp) p[i % 3] = make_double2(fma(sc, full[i].x, p[i % 3].x), fma(sc, full[i].y, p[i % 3].y));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int i = 3 * warp + c;
+      m[left_g5 ? (i + 6) % 12 : i] = left_g5 ? make_double2(-p[c].x, -p[c].y) : p[c];
+    }
+    __syncthreads();
+    st.store<SPLIT>(out, out_i, warp);
+  }
+}
+
+// Blocks of 128 threads for n sites per right-hand side; the split form up to 8 warps per SM of the plain
+// one, measured on 8^3 x 16 with 1 and 4 right-hand sides (256 and 1024 warps of 152 SMs)
+inline bool use_split(long long n, int nrhs, int sms) { return blocks32(n) * nrhs <= 8LL * sms; }
+
+}  // namespace fx

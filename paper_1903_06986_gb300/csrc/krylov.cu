@@ -25,6 +25,7 @@
 
 #include "common.cuh"
 #include "dense.h"
+#include "fxhop.cuh"
 
 using dense::cd;
 using dense::Mat;
@@ -88,6 +89,7 @@ template <typename S, typename Derived> struct PolyApply {
   lqcd_status reserve(lqcd_ctx *ctx, int nrhs) {
     Derived &d = static_cast<Derived &>(*this);
     LQCD_TRY(eo_reserve(ctx, nrhs));
+    if constexpr (std::is_same<S, double2>::value) LQCD_TRY(d.reserve_fx(ctx, nrhs));
     if (d.pp.degree == 0) return LQCD_OK;
     const size_t bytes = sizeof(S) * (size_t)nrhs * ctx->N;
     LQCD_TRY(ws_get(ctx, WS_POLY1, bytes, &d.pp.t1));
@@ -103,6 +105,16 @@ template <> struct OpT<double2> : PolyApply<double2, OpT<double2>> {
   unsigned long long g5mask;    // OP_MASKED: right-hand side r uses M gamma_5 when bit r is set
   Poly pp;
   OpT() = default;
+  // converts the links and sizes the workspace before a graph of applications is captured
+  lqcd_status reserve_fx(lqcd_ctx *ctx, int nrhs) const {
+    fx::Links L;
+    fx::Field f;
+    bool use;
+    int chunk;
+    if (prec != LQCD_PREC_F64) return LQCD_OK;
+    LQCD_TRY(fx_links(ctx, U, &L, &use));
+    return use ? fx_field(ctx, ctx->V, nrhs, &f, &chunk, &use) : LQCD_OK;
+  }
   OpT(const double2 *U_, double kappa_, int flags_, int prec_, unsigned long long g5mask_)
       : U(U_), kappa(kappa_), flags(flags_), prec(prec_), g5mask(g5mask_) {}
   lqcd_status apply_base(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs) const {
@@ -1063,6 +1075,7 @@ lqcd_status set_poly(lqcd_ctx *ctx, Op &op, const lqcd_krylov_opts *o, int nrhs)
 
 lqcd_status proj_core_entry(lqcd_ctx *ctx, const double *links, double kappa, const lqcd_defl *defl, const double2 *b,
                             double2 *x, int nrhs, const lqcd_krylov_opts *o, lqcd_solve_info *info) {
+  FxScope scope(ctx);
   const int sys = defl->hermitian ? LQCD_SYS_MG5 : o->system;
   Op op{(const double2 *)links, kappa, sys == LQCD_SYS_MG5 ? LQCD_APPLY_G5R : LQCD_APPLY_M, LQCD_PREC_F64, 0ull};
   LQCD_TRY(set_poly(ctx, op, o, nrhs));
@@ -1078,6 +1091,7 @@ lqcd_status proj_core_entry(lqcd_ctx *ctx, const double *links, double kappa, co
 // Rayleigh-Ritz pairs serve deflation).  b2 holds the same source twice; x2 receives both solutions.
 lqcd_status special_solves(lqcd_ctx *ctx, const double *links, double kappa, const double2 *b2, double2 *x2,
                            const lqcd_krylov_opts *o, lqcd_solve_info *info, lqcd_defl **defl_m, lqcd_defl **defl_h) {
+  FxScope scope(ctx);
   Op op{(const double2 *)links, kappa, OP_MASKED, LQCD_PREC_F64, 2ull};
   std::vector<lqcd_defl *> defls;
   const lqcd_status st = gmresdr_core(ctx, op, b2, x2, 2, o, std::vector<char>{0, 1}, info, &defls);
@@ -1091,6 +1105,7 @@ lqcd_status gmresdr_entry(lqcd_ctx *ctx, const double *links, double kappa, cons
   if (!ctx) return LQCD_ERR_INVALID_ARG;
   if (!links || !b || !x || !opts) return set_err(ctx, LQCD_ERR_INVALID_ARG, "NULL argument");
   if (defl_out) *defl_out = nullptr;
+  FxScope scope(ctx);
   const int sys = hermitian ? LQCD_SYS_MG5 : opts->system;
   if (sys != LQCD_SYS_M && sys != LQCD_SYS_MG5) return set_err(ctx, LQCD_ERR_INVALID_ARG, "bad system %d", sys);
   if (opts->prec != LQCD_PREC_F64 && opts->prec != LQCD_PREC_F32)

@@ -526,6 +526,7 @@ static lqcd_status scaled_acc(lqcd_ctx *ctx, const double2 *x, double2 *y, cd a,
 // out = sum_k c_k (kappa P)^k eta   (c == NULL: all ones)
 static lqcd_status hop_series_dev(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *eta, double2 *out,
                                   int nrhs, int K, const cd *c) {
+  FxScope scope(ctx);
   const long long n = (long long)nrhs * ctx->N;
   double2 *t0, *t1;
   LQCD_TRY(ws_get(ctx, WS_TMP2, sizeof(double2) * (size_t)n, (void **)&t0));
@@ -546,6 +547,7 @@ static lqcd_status hop_series_dev(lqcd_ctx *ctx, const double2 *U, double kappa,
 // out = sum_j a_j M^j eta
 static lqcd_status poly_apply_dev(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *eta, double2 *out,
                                   int nrhs, int n, const cd *a) {
+  FxScope scope(ctx);
   const long long len = (long long)nrhs * ctx->N;
   double2 *t0, *t1;
   LQCD_TRY(ws_get(ctx, WS_TMP2, sizeof(double2) * (size_t)len, (void **)&t0));
@@ -600,6 +602,7 @@ static lqcd_status deflate_dev(lqcd_ctx *ctx, const lqcd_defl *defl, const doubl
 // Min-Res coefficients: QR (classical Gram-Schmidt twice) of v = (M b, .., M^{n+1} b)
 static lqcd_status poly_coeffs_dev(lqcd_ctx *ctx, const double2 *U, double kappa, uint64_t seed, int n,
                                    std::vector<cd> &a, int flags = LQCD_APPLY_M) {
+  FxScope scope(ctx);
   const long long N = ctx->N;
   double2 *Q, *b, *h;
   double *nrm;
@@ -648,6 +651,7 @@ static lqcd_status poly_coeffs_dev(lqcd_ctx *ctx, const double2 *U, double kappa
 
 // t[(k * 9 + op) * Lt + t] for k < K
 static lqcd_status hop_traces_dev(lqcd_ctx *ctx, const double2 *U, double kappa, int K, std::vector<cd> &tr) {
+  FxScope scope(ctx);
   const int *d = ctx->dims;
   const int Lt = d[3];
   const long long N = ctx->N;
@@ -1064,6 +1068,7 @@ lqcd_status eo_noise_solve(lqcd_loop *L, const double2 *U, const double2 *eta, d
                            lqcd_solve_info *info) {
   lqcd_ctx *ctx = L->ctx, *ce = L->ce;
   ce->stream = ctx->stream;
+  FxScope scope_e(ce);
   const long long Ne = ce->N, N = ctx->N;
   double2 *be, *xe, *ye;
   LQCD_TRY(ws_get(ce, WS_NBLK, sizeof(double2) * (size_t)nb * Ne * 3, (void **)&be));
@@ -1212,6 +1217,7 @@ lqcd_status loop_finish_setup(lqcd_loop *L, const double2 *U, const double *link
 lqcd_status loop_noises(lqcd_loop *L, const double *links, uint32_t first0, int count, std::vector<cd> &per_noise_t,
                         lqcd_noise_info *info) {
   lqcd_ctx *ctx = L->ctx;
+  FxScope scope(ctx);
   const lqcd_est_opts *o = &L->o;
   const double kappa = L->kappa;
   const double2 *U = (const double2 *)links;

@@ -17,7 +17,10 @@
 //   mu = t:  1 - g = diag(0,0,2,2): only the lower pair, (2 p2, 2 p3)
 //            1 + g = diag(2,2,0,0): only the upper pair, (2 p0, 2 p1)
 // gamma_5 = -[[0, 1], [1, 0]] in this basis: (g5 p) = (-p2, -p3, -p0, -p1).
+#include <algorithm>
+
 #include "common.cuh"
+#include "fxhop.cuh"
 #include "spin.cuh"
 
 namespace {
@@ -137,13 +140,195 @@ lqcd_status launch_mode(lqcd_ctx *ctx, const S *U, double kappa, const S *in, S 
   return launch_check_bytes(ctx, "wilson_kernel", K_WILSON, (double)ctx->V * nrhs, bytes);
 }
 
+// FP64 links [mu][site][3][3] -> the chunk-major limbs and exponents of fx::Links
+__global__ void __launch_bounds__(128) fx_links_kernel(const double2 *__restrict__ U, int4 *__restrict__ q,
+                                                       int *__restrict__ ex, int VL) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int mu = blockIdx.y;
+  if (s >= VL) return;
+  const double2 *u = U + ((long long)mu * VL + s) * 9;
+  double2 v[9];
+  int mx = 0;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    v[e] = __ldg(u + e);
+    mx = max(mx, max(fx::abs_hi(v[e].x), fx::abs_hi(v[e].y)));
+  }
+  const int X = max(mx >> 20, fx::FX_MINX);
+  ex[(long long)mu * VL + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_LINK) ? fx::FX_BAD : X;
+  int4 *o = q + fx::slot(s, 36) + mu * 9 * 32;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    int4 w;
+    fx::split(fx::fixed(v[e].x, 4 + X), w.x, w.y);
+    fx::split(fx::fixed(v[e].y, 4 + X), w.z, w.w);
+    w.w = max(w.w, -0x7fffffff);   // fx::direction negates the imaginary part
+    o[e * 32] = w;
+  }
+}
+
+// nrhs canonical FP64 fields of S sites -> fx::Field.  Bound by HBM (192 bytes read and 196 written per
+// site); 32 sites of one right-hand side per warp, staged in memory order
+constexpr int FX_BS = 128;
+__global__ void __launch_bounds__(FX_BS) fx_convert_kernel(const double2 *__restrict__ in, fx::Field f, int S,
+                                                           int nrhs) {
+  __shared__ __align__(16) char sm[FX_BS / 32 * fx::WARP_BYTES];
+  const int r = blockIdx.x % nrhs;
+  const int s0 = (blockIdx.x / nrhs) * FX_BS + threadIdx.x, s = min(s0, S - 1);
+  fx::Stage st;
+  st.init(sm + (threadIdx.x >> 5) * fx::WARP_BYTES);
+  st.load(in + (long long)r * S * 12, s);
+  fx::wait_all();
+  __syncwarp();
+  if (s0 >= S) return;
+  double2 v[12];
+  int mx = 0;
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    v[c] = st.mine()[c];
+    mx = max(mx, max(fx::abs_hi(v[c].x), fx::abs_hi(v[c].y)));
+  }
+  const int X = max(mx >> 20, fx::FX_MINX);
+  f.ex[(long long)r * S + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_FIELD) ? fx::FX_BAD : X;
+  longlong2 *o = f.q + (long long)r * fx::blocks32(S) * 384 + fx::slot(s, 12);
+#pragma unroll
+  for (int c = 0; c < 12; ++c) o[c * 32] = make_longlong2(fx::fixed(v[c].x, 4 + X), fx::fixed(v[c].y, 4 + X));
+}
+
+// FP64 operator: M, M g5 (bit r of g5mask for the masked form), M^dag or P for right-hand side r =
+// blockIdx.x % nrhs (fastest, so that the links of one site block are shared through L2).
+// Four blocks per SM (128 registers): ten fields of 24^3 x 32 in 1.63 ms, 1.71 ms with three and 1.79 ms
+// with five; the integer multiply-adds alone (1824 per site, 32 per clock and SM) take 0.86 ms.
+enum { FX_G5IN = 1, FX_G5LEFT = 2, FX_HOP = 4, FX_MASK = 8 };
+template <int SPLIT>
+__global__ void __launch_bounds__(FX_BS, 4) wilson_fx_kernel(const double2 *__restrict__ U, fx::Links L, fx::Field f,
+                                                             const double2 *__restrict__ in, double2 *__restrict__ out,
+                                                             double kappa, int Lx, int Ly, int Lz, int Lt, int V,
+                                                             int nrhs, int mode, unsigned long long g5mask) {
+  __shared__ __align__(16) char sm[fx::SMEM_BYTES<SPLIT>];
+  const int r = blockIdx.x % nrhs;
+  const int s0 = (blockIdx.x / nrhs) * (FX_BS / SPLIT) + threadIdx.x % (FX_BS / SPLIT);
+  const int s = min(s0, V - 1);
+  const double2 *src = in + (long long)r * V * 12;
+  const bool g5 = (mode & FX_MASK) ? ((g5mask >> r) & 1ull) != 0 : (mode & FX_G5IN) != 0;
+  const bool hop = (mode & FX_HOP) != 0;
+  const fx::Torus nb(Lx, Ly, Lz, Lt, s);
+  fx::run<SPLIT, false>(sm, U, L, V, s, nb, f, r, V, src, g5, hop ? nullptr : src, s, g5, hop ? 1.0 : -kappa,
+                        (mode & FX_G5LEFT) != 0, out + (long long)r * V * 12, s0 < V ? s : -1);
+}
+
+lqcd_status fx_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out, int nrhs,
+                      int flags, unsigned long long g5mask) {
+  int mode = 0;
+  switch (flags) {
+    case LQCD_APPLY_M: break;
+    case LQCD_APPLY_G5R: mode = FX_G5IN; break;
+    case LQCD_APPLY_DAG: mode = FX_G5IN | FX_G5LEFT; break;
+    case LQCD_APPLY_HOP: mode = FX_HOP; break;
+    case 4: mode = FX_MASK; break;
+    default: return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply: unknown flags %d", flags);
+  }
+  fx::Links L;
+  fx::Field f;
+  bool use;
+  int chunk;
+  LQCD_TRY(fx_links(ctx, U, &L, &use));
+  if (use) LQCD_TRY(fx_field(ctx, ctx->V, nrhs, &f, &chunk, &use));
+  if (!use) return launch_mode<double, double2>(ctx, U, kappa, in, out, nrhs, flags, g5mask);
+  const int *d = ctx->dims;
+  for (int r0 = 0; r0 < nrhs; r0 += chunk) {
+    const int nr = std::min(chunk, nrhs - r0);
+    const double2 *src = in + (long long)r0 * ctx->N;
+    LQCD_TRY(fx_convert(ctx, src, f, ctx->V, nr));
+    const bool split = fx::use_split(ctx->V, nr, ctx->sms);
+    kbegin(ctx);
+    (split ? wilson_fx_kernel<4> : wilson_fx_kernel<1>)
+        <<<(unsigned)((long long)ceil_div(ctx->V, split ? 32 : FX_BS) * nr), FX_BS, 0, ctx->stream>>>(
+            U, L, f, src, out + (long long)r0 * ctx->N, kappa, d[0], d[1], d[2], d[3], ctx->V, nr, mode,
+            flags == 4 ? g5mask >> r0 : 0ull);
+    // compulsory bytes: each field read and written once, the links once
+    const double bytes = 2.0 * nr * ctx->V * 12 * 16 + 36.0 * ctx->V * 16;
+    LQCD_TRY(launch_check_bytes(ctx, "wilson_fx_kernel", K_WILSON, (double)ctx->V * nr, bytes));
+  }
+  if (ctx->fx_depth == 0) fx_done(ctx);
+  return LQCD_OK;
+}
+
 }  // namespace
+
+lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use) {
+  const int VL = ctx->eo ? 2 * ctx->V : ctx->V;
+  const size_t n = (size_t)4 * VL, qbytes = (size_t)fx::blocks32(VL) * 32 * 36 * sizeof(int4), bytes = qbytes + n * sizeof(int);
+  *use = true;
+  const bool have = ctx->fx_depth > 0 && ctx->fx_src == U;   // converted earlier in this call
+  if (!have) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      *use = false;
+      return LQCD_OK;
+    }
+    if (ctx->fx_event && ctx->fx_event_stream != ctx->stream)
+      LQCD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->fx_event, 0));
+  }
+  char *p;
+  const lqcd_status st = ws_get(ctx, WS_FX_LINKS, bytes, (void **)&p);
+  if (st == LQCD_ERR_OOM) {
+    ctx->err.clear();
+    *use = false;
+    return LQCD_OK;
+  }
+  LQCD_TRY(st);
+  L->q = (const int4 *)p;
+  L->ex = (const int *)(p + qbytes);
+  if (have) return LQCD_OK;
+  kbegin(ctx);
+  fx_links_kernel<<<dim3(ceil_div(VL, 128), 4), 128, 0, ctx->stream>>>(U, (int4 *)p, (int *)(p + qbytes), VL);
+  LQCD_TRY(launch_check_bytes(ctx, "fx_links_kernel", K_BLAS1, (double)n * 9, (double)n * (9 * 32 + 4)));
+  if (ctx->fx_depth > 0) ctx->fx_src = U;
+  return LQCD_OK;
+}
+
+lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *chunk, bool *use) {
+  // at most 1 GiB of integers: 12 fields of 24^3 x 32, enough that the links (0.25 GB there) count
+  // little, and a bounded share of the memory beside a Krylov basis or hundreds of eigenvectors.
+  // Blocks are numbered 32-bit within a chunk: (S / FX_BS + 1) x chunk < 2^31 for all S <= 2^28.
+  const size_t qper = (size_t)fx::blocks32(S) * 32 * 12 * sizeof(longlong2), per = qper + S * sizeof(int);
+  *chunk = (int)std::max<long long>(1, std::min<long long>(nrhs, (1ll << 30) / (long long)per));
+  char *p;
+  const lqcd_status st = ws_get(ctx, WS_FX_FIELD, *chunk * per, (void **)&p);
+  *use = st != LQCD_ERR_OOM;
+  if (!*use) {
+    ctx->err.clear();
+    return LQCD_OK;
+  }
+  f->q = (longlong2 *)p;
+  f->ex = (int *)(p + *chunk * qper);
+  return st;
+}
+
+lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs) {
+  kbegin(ctx);
+  fx_convert_kernel<<<(unsigned)((long long)ceil_div(S, FX_BS) * nrhs), FX_BS, 0, ctx->stream>>>(in, f, (int)S, nrhs);
+  return launch_check_bytes(ctx, "fx_convert_kernel", K_BLAS1, 12.0 * S * nrhs, 388.0 * S * nrhs);
+}
+
+void fx_done(lqcd_ctx *ctx) {
+  if (!ctx->fx_event && cudaEventCreateWithFlags(&ctx->fx_event, cudaEventDisableTiming) != cudaSuccess) {
+    ctx->fx_event = nullptr;
+    cudaGetLastError();
+    cudaStreamSynchronize(ctx->stream);   // no event to wait for later: the use ends here
+    return;
+  }
+  cudaEventRecord(ctx->fx_event, ctx->stream);
+  ctx->fx_event_stream = ctx->stream;
+}
 
 lqcd_status wilson_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out, int nrhs,
                           int prec, int flags) {
   if (nrhs <= 0 || nrhs > 65535) return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply: nrhs %d out of range", nrhs);
   if (ctx->eo) return eo_schur_launch(ctx, U, kappa, in, out, nrhs, prec, flags);
-  if (prec == LQCD_PREC_F64) return launch_mode<double, double2>(ctx, U, kappa, in, out, nrhs, flags);
+  if (prec == LQCD_PREC_F64) return fx_launch(ctx, U, kappa, in, out, nrhs, flags, 0ull);
   if (prec == LQCD_PREC_F32) return launch_mode<float, double2>(ctx, U, kappa, in, out, nrhs, flags);
   return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply: unknown precision %d", prec);
 }
@@ -152,7 +337,7 @@ lqcd_status wilson_launch_masked(lqcd_ctx *ctx, const double2 *U, double kappa, 
                                  int nrhs, unsigned long long g5mask) {
   if (nrhs <= 0 || nrhs > 64) return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson (masked): nrhs %d out of range", nrhs);
   LQCD_TRY(require_full(ctx, "wilson (masked)"));
-  return launch_mode<double, double2>(ctx, U, kappa, in, out, nrhs, 4, g5mask);
+  return fx_launch(ctx, U, kappa, in, out, nrhs, 4, g5mask);
 }
 
 lqcd_status wilson_launch_f32(lqcd_ctx *ctx, const float2 *U, double kappa, const float2 *in, float2 *out, int nrhs,
