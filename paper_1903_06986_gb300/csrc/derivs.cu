@@ -42,108 +42,143 @@ __constant__ double c_lambda[8][9][2] = {
     {{0.57735026918962576, 0}, {0, 0}, {0, 0}, {0, 0}, {0.57735026918962576, 0}, {0, 0}, {0, 0}, {0, 0},
      {-1.1547005383792515, 0}}};
 
-__device__ __forceinline__ void zero4(Cx<double> a[4][3]) {
+// Half spinors of direction MU: (1 - g_MU) p (SIGN = -1) and (1 + g_MU) p (SIGN = +1) are rank two, an upper
+// pair h = p_k + phase p_lower and a lower pair that repeats it (table at the head of spin.cuh); a product
+// over all four spins of such a spinor with any q is the product of the two upper pairs.  In the t
+// direction h is the surviving pair, and the product takes a factor 2 (see link_grad_kernel).
+template <int MU, int SIGN>
+__device__ __forceinline__ void half(const double2 *p, Cx<double> h[2][3]) {
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a[s][c] = mk<double>(0.0, 0.0);
-}
-
-// (1 + g_mu) p as a full spinor, through the backward term with the unit colour matrix
-template <int MU>
-__device__ __forceinline__ void proj_plus(const Cx<double> p[4][3], Cx<double> o[4][3]) {
-  Cx<double> one[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) one[i] = mk<double>((i % 4 == 0) ? 1.0 : 0.0, 0.0);
-  zero4(o);
-  term_bwd<double, MU>(p, one, o);
-}
-
-template <int MU>
-__device__ __forceinline__ void proj_minus(const Cx<double> p[4][3], Cx<double> o[4][3]) {
-  Cx<double> one[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) one[i] = mk<double>((i % 4 == 0) ? 1.0 : 0.0, 0.0);
-  zero4(o);
-  term_fwd<double, MU>(p, one, o);
-}
-
-template <int MU>
-__device__ void link_terms(const Cx<double> u[9], const Cx<double> zs[4][3], const Cx<double> zf[4][3],
-                           const Cx<double> xs[4][3], const Cx<double> xf[4][3], Cx<double> B[9], Cx<double> dU[9],
-                           Cx<double> dUc[9]) {
-  Cx<double> w1[4][3], pm[4][3], v2[4][3];
-  // w1 = (1 - g) U x(s+mu); pm = (1 - g) x(s+mu); v2 = (1 + g) x(s)
-  zero4(w1);
-  term_fwd<double, MU>(xf, u, w1);
-  proj_minus<MU>(xf, pm);
-  proj_plus<MU>(xs, v2);
-#pragma unroll
-  for (int sp = 0; sp < 4; ++sp) {
-    // q = U z(s+mu) for this spin
-    Cx<double> q[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        re = fma(u[3 * a + b].x, zf[sp][b].x, re);
-        re = fma(-u[3 * a + b].y, zf[sp][b].y, re);
-        im = fma(u[3 * a + b].x, zf[sp][b].y, im);
-        im = fma(u[3 * a + b].y, zf[sp][b].x, im);
-      }
-      q[a] = mk<double>(re, im);
+  for (int c = 0; c < 3; ++c) {
+    if (MU == 3) {
+      const int k = SIGN < 0 ? 6 : 0;
+      h[0][c] = load_c<double>(p + k + c);
+      h[1][c] = load_c<double>(p + k + 3 + c);
+    } else {
+      Cx<double> p0 = load_c<double>(p + c), p1 = load_c<double>(p + 3 + c), p2 = load_c<double>(p + 6 + c),
+                 p3 = load_c<double>(p + 9 + c);
+      Cx<double> a = MU == 0 ? ti(p3) : MU == 1 ? p3 : ti(p2);
+      Cx<double> b = MU == 0 ? ti(p2) : MU == 1 ? neg(p2) : neg(ti(p3));
+      h[0][c] = SIGN < 0 ? p0 + a : p0 - a;
+      h[1][c] = SIGN < 0 ? p1 + b : p1 - b;
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        // B[c][d] += w1_c conj(z_d) - v2_c conj(q_d)
-        const Cx<double> a1 = w1[sp][c], z = zs[sp][d], v = v2[sp][c], qq = q[d];
-        B[3 * c + d].x += a1.x * z.x + a1.y * z.y - (v.x * qq.x + v.y * qq.y);
-        B[3 * c + d].y += a1.y * z.x - a1.x * z.y - (v.y * qq.x - v.x * qq.y);
-        // dU[c][d] += conj(z_c) pm_d ;  dUc[c][d] += conj(z(s+mu)_d) v2_c
-        const Cx<double> zc = zs[sp][c], pmd = pm[sp][d], zfd = zf[sp][d], vc = v2[sp][c];
-        dU[3 * c + d].x += zc.x * pmd.x + zc.y * pmd.y;
-        dU[3 * c + d].y += zc.x * pmd.y - zc.y * pmd.x;
-        dUc[3 * c + d].x += zfd.x * vc.x + zfd.y * vc.y;
-        dUc[3 * c + d].y += zfd.x * vc.y - zfd.y * vc.x;
-      }
   }
 }
+// m[c][d] += sum_k conj(a_k[c]) b_k[d]
+__device__ __forceinline__ void outer(const Cx<double> a[2][3], const Cx<double> b[2][3], Cx<double> m[9]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        Cx<double> &o = m[3 * c + d];
+        o.x = fma(a[k][c].x, b[k][d].x, o.x);
+        o.x = fma(a[k][c].y, b[k][d].y, o.x);
+        o.y = fma(a[k][c].x, b[k][d].y, o.y);
+        o.y = fma(-a[k][c].y, b[k][d].x, o.y);
+      }
+}
+// one right-hand side's share of D[c][d] = sum_spin conj(z(s)_c) [(1 - g) x(s+mu)]_d and
+// Dc[d][c] = sum_spin conj(z(s+mu)_d) [(1 + g) x(s)]_c
+template <int MU>
+__device__ __forceinline__ void link_terms(const double2 *z, const double2 *x, int s, int sf, Cx<double> D[9],
+                                           Cx<double> Dc[9]) {
+  Cx<double> a[2][3], b[2][3];
+  half<MU, -1>(z + 12LL * s, a);
+  half<MU, -1>(x + 12LL * sf, b);
+  outer(a, b, D);
+  half<MU, 1>(z + 12LL * sf, a);
+  half<MU, 1>(x + 12LL * s, b);
+  outer(a, b, Dc);
+}
 
-// One thread per (site, direction): accumulates scale * sum over right-hand sides into grad
-// (dT/dw_a, 8 per link) and, when given, into gU = dT/dU* + conj(dT/dU) (torch convention for Re T).
-__global__ void link_grad_kernel(const double2 *__restrict__ U, double kappa, const double2 *__restrict__ z,
-                                 const double2 *__restrict__ x, int nrhs, double scale, int Lx, int Ly, int Lz, int Lt,
-                                 double2 *__restrict__ grad, double2 *__restrict__ gU) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+// One thread per (site, direction) and group of right-hand sides: accumulates scale * sum over right-hand
+// sides into grad (dT/dw_a, 8 per link) and, when given, into gU = dT/dU* + conj(dT/dU) (torch
+// convention for Re T).
+// Bound by FP64 issue (two operations per clock and SM).  Per right-hand side only the two colour
+// matrices D and Dc are summed, from half spinors: 192 operations per link (144 in the outer products,
+// 48 in the projections).  The link enters once at the end, B = U D^T - Dc^T U^dag.  Forming U x, U z and
+// B for every right-hand side on all four spins took about 1000: 6.24 ms for 16 right-hand sides of
+// 12^3 x 24 before, 1.08 ms now (0.87 ms of FP64 issue).
+// G > 1: the block's 128 threads are 32 sites x G = 4 groups of right-hand sides, summed through shared
+// memory in a fixed order.
+template <int G>
+__global__ void __launch_bounds__(128) link_grad_kernel(const double2 *__restrict__ U, double kappa,
+                                                        const double2 *__restrict__ z, const double2 *__restrict__ x,
+                                                        int nrhs, double scale, int Lx, int Ly, int Lz, int Lt,
+                                                        double2 *__restrict__ grad, double2 *__restrict__ gU) {
+  const int grp = G == 1 ? 0 : threadIdx.x >> 5;
+  const int s0 = G == 1 ? blockIdx.x * 128 + threadIdx.x : blockIdx.x * 32 + (threadIdx.x & 31);
   const int mu = blockIdx.y;
   const int V = Lx * Ly * Lz * Lt;
-  if (s >= V) return;
+  const int s = min(s0, V - 1);
   const int xx = s % Lx, y = (s / Lx) % Ly, zz = (s / (Lx * Ly)) % Lz, t = s / (Lx * Ly * Lz);
   int sf;
   if (mu == 0) sf = (xx + 1 == Lx) ? s - (Lx - 1) : s + 1;
   else if (mu == 1) sf = (y + 1 == Ly) ? s - (Ly - 1) * Lx : s + Lx;
   else if (mu == 2) sf = (zz + 1 == Lz) ? s - (Lz - 1) * Lx * Ly : s + Lx * Ly;
   else sf = (t + 1 == Lt) ? s - (Lt - 1) * Lx * Ly * Lz : s + Lx * Ly * Lz;
-  Cx<double> u[9];
-  load_link<double>(U, (long long)mu * V + s, u);
-  Cx<double> B[9], dU[9], dUc[9];
+  Cx<double> D[9], Dc[9];
 #pragma unroll
-  for (int i = 0; i < 9; ++i) B[i] = dU[i] = dUc[i] = mk<double>(0.0, 0.0);
-  for (int r = 0; r < nrhs; ++r) {
+  for (int i = 0; i < 9; ++i) D[i] = Dc[i] = mk<double>(0.0, 0.0);
+  for (int r = grp; r < nrhs; r += G) {
     const long long off = (long long)r * V * 12;
-    Cx<double> zs[4][3], zf[4][3], xs[4][3], xf[4][3];
-    load_spinor<double, false>(z + off + 12LL * s, zs);
-    load_spinor<double, false>(z + off + 12LL * sf, zf);
-    load_spinor<double, false>(x + off + 12LL * s, xs);
-    load_spinor<double, false>(x + off + 12LL * sf, xf);
-    if (mu == 0) link_terms<0>(u, zs, zf, xs, xf, B, dU, dUc);
-    if (mu == 1) link_terms<1>(u, zs, zf, xs, xf, B, dU, dUc);
-    if (mu == 2) link_terms<2>(u, zs, zf, xs, xf, B, dU, dUc);
-    if (mu == 3) link_terms<3>(u, zs, zf, xs, xf, B, dU, dUc);
+    if (mu == 0) link_terms<0>(z + off, x + off, s, sf, D, Dc);
+    if (mu == 1) link_terms<1>(z + off, x + off, s, sf, D, Dc);
+    if (mu == 2) link_terms<2>(z + off, x + off, s, sf, D, Dc);
+    if (mu == 3) link_terms<3>(z + off, x + off, s, sf, D, Dc);
   }
+  if constexpr (G > 1) {
+    __shared__ double2 red[G - 1][18][32];
+    const int lane = threadIdx.x & 31;
+    if (grp > 0) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        red[grp - 1][i][lane] = make_double2(D[i].x, D[i].y);
+        red[grp - 1][9 + i][lane] = make_double2(Dc[i].x, Dc[i].y);
+      }
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int g = 0; g < G - 1; ++g)
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const double2 a = red[g][i][lane], b = red[g][9 + i][lane];
+        D[i].x += a.x; D[i].y += a.y;
+        Dc[i].x += b.x; Dc[i].y += b.y;
+      }
+  }
+  if (s0 >= V) return;
+  if (mu == 3) {   // (1 -+ g_t) is twice the projector on a pair
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      D[i].x *= 2.0; D[i].y *= 2.0;
+      Dc[i].x *= 2.0; Dc[i].y *= 2.0;
+    }
+  }
+  Cx<double> u[9], B[9];
+  load_link<double>(U, (long long)mu * V + s, u);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      double re = 0.0, im = 0.0;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const Cx<double> p = u[3 * c + b], q = D[3 * d + b], v = Dc[3 * b + c], w = u[3 * d + b];
+        re = fma(p.x, q.x, re);
+        re = fma(-p.y, q.y, re);
+        im = fma(p.x, q.y, im);
+        im = fma(p.y, q.x, im);
+        re = fma(-v.x, w.x, re);
+        re = fma(-v.y, w.y, re);
+        im = fma(v.x, w.y, im);
+        im = fma(-v.y, w.x, im);
+      }
+      B[3 * c + d] = mk<double>(re, im);
+    }
   // dT/dw_a = (i kappa / 2) tr(lambda_a B)
   double2 *g = grad + ((long long)mu * V + s) * 8;
 #pragma unroll
@@ -168,13 +203,15 @@ __global__ void link_grad_kernel(const double2 *__restrict__ U, double kappa, co
   if (gU) {
     double2 *o = gU + ((long long)mu * V + s) * 9;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      // dT/dU* + conj(dT/dU), both carrying kappa
-      double2 v = o[i];
-      v.x += scale * kappa * (dUc[i].x + dU[i].x);
-      v.y += scale * kappa * (dUc[i].y - dU[i].y);
-      o[i] = v;
-    }
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        // dT/dU* + conj(dT/dU) = Dc^T + conj(D), both carrying kappa
+        double2 v = o[3 * c + d];
+        v.x += scale * kappa * (Dc[3 * d + c].x + D[3 * c + d].x);
+        v.y += scale * kappa * (Dc[3 * d + c].y - D[3 * c + d].y);
+        o[3 * c + d] = v;
+      }
   }
 }
 
@@ -187,9 +224,11 @@ double now_s() {
 lqcd_status link_grad_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *z, const double2 *x,
                              int nrhs, double scale, double2 *grad, double2 *gU) {
   const int *d = ctx->dims;
+  // four groups of right-hand sides per block while one thread per link leaves fewer than 16 warps per SM
+  const bool split = nrhs >= 4 && (long long)ceil_div(ctx->V, 32) * 4 < 16LL * ctx->sms;
   kbegin(ctx);
-  link_grad_kernel<<<dim3(ceil_div(ctx->V, 128), 4), 128, 0, ctx->stream>>>(U, kappa, z, x, nrhs, scale, d[0], d[1],
-                                                                          d[2], d[3], grad, gU);
+  (split ? link_grad_kernel<4> : link_grad_kernel<1>)<<<dim3(ceil_div(ctx->V, split ? 32 : 128), 4), 128, 0, ctx->stream>>>(
+      U, kappa, z, x, nrhs, scale, d[0], d[1], d[2], d[3], grad, gU);
   return launch_check(ctx, "link_grad_kernel", K_CONTRACT, (double)ctx->V * 4 * nrhs);
 }
 

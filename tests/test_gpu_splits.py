@@ -1,0 +1,41 @@
+"""Launch forms that depend on sizes, where they can go wrong: right-hand sides split over a block in the
+link gradient."""
+import numpy as np
+import pytest
+
+from oracle import derivs as Dv, lattice as L
+from paper_1903_06986_gb300 import lqcd, synth
+from tests.gpu_util import context, dev, host, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+def fields(dims, n, seed):
+    r = np.random.default_rng(seed)
+    shp = L.field_shape(dims, (n,))
+    return r.standard_normal(shp) + 1j * r.standard_normal(shp)
+
+
+@pytest.mark.parametrize("dims,n", [((3, 2, 4, 4), 1), ((3, 2, 4, 4), 4), ((2, 3, 5, 2), 7), ((4, 4, 4, 3), 5)])
+def test_link_grad_groups(dims, n):
+    """n = 1: one thread per link; else four groups of right-hand sides, the last ones short."""
+    ctx = context(dims)
+    U, x, z = synth.su3_links(dims, 0.5, 3), fields(dims, n, 1), fields(dims, n, 2)
+    g, gl = lqcd.link_grad(ctx, dev(U), 0.137, dev(z), dev(x), scale=0.5)
+    ref = 0.5 * sum(Dv.link_gradient(U, 0.137, x[r], z[r]) for r in range(n))
+    assert rel_err(host(g), ref) < 1e-12
+    dU = sum(Dv.link_matrix_derivatives(U, 0.137, x[r], z[r])[0] for r in range(n))
+    dUc = sum(Dv.link_matrix_derivatives(U, 0.137, x[r], z[r])[1] for r in range(n))
+    assert rel_err(host(gl), 0.5 * (dUc + dU.conj())) < 1e-12
+
+
+def test_link_grad_one_call_is_the_sum_of_single_ones():
+    """20736 sites: one thread per link with every right-hand side in it, against n calls of one."""
+    dims, n = (12, 12, 12, 12), 5
+    ctx = context(dims)
+    Ud, x, z = dev(synth.su3_links(dims, 0.4323, 4)), dev(fields(dims, n, 5)), dev(fields(dims, n, 6))
+    g, gl = lqcd.link_grad(ctx, Ud, 0.137, z, x)
+    parts = [lqcd.link_grad(ctx, Ud, 0.137, z[r:r + 1].contiguous(), x[r:r + 1].contiguous()) for r in range(n)]
+    for got, i in ((g, 0), (gl, 1)):
+        want = sum(host(p[i]) for p in parts)
+        assert rel_err(host(got), want) < 1e-14
