@@ -1,9 +1,9 @@
 """Launch forms that depend on sizes, where they can go wrong: right-hand sides split over a block in the
-link gradient."""
+link gradient, chunks of a timeslice in the contraction."""
 import numpy as np
 import pytest
 
-from oracle import derivs as Dv, lattice as L
+from oracle import derivs as Dv, lattice as L, operators as O
 from paper_1903_06986_gb300 import lqcd, synth
 from tests.gpu_util import context, dev, host, rel_err
 
@@ -39,3 +39,13 @@ def test_link_grad_one_call_is_the_sum_of_single_ones():
     for got, i in ((g, 0), (gl, 1)):
         want = sum(host(p[i]) for p in parts)
         assert rel_err(host(got), want) < 1e-14
+
+
+@pytest.mark.parametrize("dims,n", [((9, 7, 11, 3), 2), ((16, 16, 8, 2), 1), ((5, 3, 2, 6), 40)])
+def test_contract_chunks(dims, n):
+    """Ragged chunks of a timeslice (the last one short), several chunks with few pairs, one with many."""
+    ctx = context(dims)
+    U, eta, w = synth.su3_links(dims, 0.5, 7), fields(dims, n, 8), fields(dims, n, 9)
+    got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
+    ref = O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
+    assert rel_err(got, ref) < 1e-13
