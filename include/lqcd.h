@@ -338,7 +338,9 @@ lqcd_status lqcd_poly_coeffs(lqcd_ctx *ctx, const double *links, double kappa, u
  * Meet in the middle (Sec. 5.1 add-back): P is applied to the whole probe field only up to a depth
  * h (lqcd_set_probe_depth; by default the h with the fewest site updates, e.g. 2 of the 6 orders at
  * K = 7 with 512 classes); each higher order k is evaluated only within K - k hops of the class
- * members, where the contraction and the later orders read it.  The result is the same trace. */
+ * members, where the contraction and the later orders read it.  The result is the same trace.
+ * Where every extent exceeds K and K <= 9, and no depth is fixed, no probe is applied to the lattice at
+ * all: every column of P^k is followed from its source within min(k, K - k) hops. */
 lqcd_status lqcd_hop_traces(lqcd_ctx *ctx, const double *links, double kappa, int K, double *t);
 
 /* Full-lattice applications of P per probe in lqcd_hop_traces and in the setup of loop estimates:
@@ -347,7 +349,7 @@ lqcd_status lqcd_hop_traces(lqcd_ctx *ctx, const double *links, double kappa, in
  * minimise the site updates (default).  LQCD_ERR_INVALID_ARG for values outside 0..64. */
 lqcd_status lqcd_set_probe_depth(lqcd_ctx *ctx, int depth);
 
-/* The depth lqcd_hop_traces uses (host only; needs no GPU and no context): for an Lx x Ly x Lz x Lt
+/* The depth lqcd_hop_traces uses when it probes (host only; needs no GPU and no context): for an Lx x Ly x Lz x Lt
  * torus (dims[0..3], each in 2..1024), K terms and a fixed depth as lqcd_set_probe_depth sets it
  * (0 = by cost), *depth receives the number of full applications of P per probe.
  * LQCD_ERR_INVALID_ARG for bad arguments. */

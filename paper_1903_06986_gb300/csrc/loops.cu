@@ -19,6 +19,7 @@
 
 #include "common.cuh"
 #include "dense.h"
+#include "fxhop.cuh"
 #include "spin.cuh"
 
 using dense::cd;
@@ -481,6 +482,180 @@ static int probe_depth(const lqcd_ctx *ctx, const Colouring &col, int K) {
   return probe_depth_for(ctx->probe_depth, col, K);
 }
 
+// ---- hopping traces site by site ----------------------------------------------------------------
+// While every extent exceeds K, no walk of the trace winds around the torus, and a column of P^k (a unit
+// source at one site and component) is read only at the source and its neighbours.  A walk from the
+// source that comes back there is within min(k, max(1, K - k)) hops after k steps, so order k is needed
+// on that ball alone, and there only on the sites of parity k (all others are zero): 8, 33, 96, 33, 8, 1
+// sites for K = 7, 179 of them instead of the 3 applications to the whole lattice that a probe of 512
+// classes takes (24,000 site updates per class member of 8^3 x 16, against 2864).  One block follows
+// G components of one source in shared memory: order k overwrites the sites of its own parity and reads
+// those of the other, a neighbour outside order k - 1's ball counts as zero, and nothing but the links
+// is read from global memory.
+// Bound by FP64 issue: about 670 of the 1432 neighbour terms are non-zero (a site on the rim of a growing
+// ball has one to three), 54 clocks each per SM: 12 ms of the 33.4 ms measured on 8^3 x 16, K = 7
+// (189 ms by probing with the fixed-point operator, 295 ms with the FP64 one).
+constexpr int TB_THREADS = 128, TB_SITE = 208;   // shared bytes per (site, component): see fxhop.cuh
+constexpr int TB_MAXR = 4, TB_MAXK = 2 * TB_MAXR + 1;
+struct BallTable {
+  int n;                     // sites of the ball
+  int base[2];               // first site of each parity; within one, by distance from the source
+  int cnt[TB_MAXK];          // sites of parity k within min(k, max(1, K - k)) hops, per order k
+};
+
+__device__ __forceinline__ void sm_spinor(const double2 *p, Cx<double> s[4][3]) {
+#pragma unroll
+  for (int i = 0; i < 12; ++i) s[i / 3][i % 3] = mk<double>(p[i].x, p[i].y);
+}
+
+// part[(k * 10 + q) * nx + i], source x0 + i, 1 <= k < K: q = 0..4 the local densities (even k), 5 + mu the
+// second point-split term and, for mu < 3, the first one too (odd k), q = 9 the first term of mu = t,
+// which belongs to the timeslice before the source's; point-split terms without kappa
+__global__ void __launch_bounds__(TB_THREADS, 2) trace_ball_kernel(const double2 *__restrict__ U, int K, int G,
+                                                                   BallTable bt, const char4 *__restrict__ off,
+                                                                   const short *__restrict__ nbt, int x0, int nx, int Lx,
+                                                                   int Ly, int Lz, int Lt,
+                                                                   double2 *__restrict__ part) {
+  extern __shared__ __align__(16) char sm[];
+  __shared__ double2 res[TB_MAXK][10];
+  const long long V = (long long)Lx * Ly * Lz * Lt;
+  const int m = x0 + blockIdx.x;
+  const int mx = m % Lx, my = (m / Lx) % Ly, mz = (m / (Lx * Ly)) % Lz, mt = m / (Lx * Ly * Lz);
+  auto at = [&](int b, int g) { return (double2 *)(sm + (b * G + g) * TB_SITE); };
+  auto wrap = [](int v, int L) { return v < 0 ? v + L : v >= L ? v - L : v; };
+  for (int i = threadIdx.x; i < TB_MAXK * 10; i += TB_THREADS) res[i / 10][i % 10] = make_double2(0.0, 0.0);
+  for (int c0 = 0; c0 < 12; c0 += G) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < 12 * G; i += TB_THREADS)
+      at(bt.base[0], i / 12)[i % 12] = make_double2(i % 12 == c0 + i / 12 ? 1.0 : 0.0, 0.0);
+    __syncthreads();
+    for (int k = 1; k < K; ++k) {
+      const int own = bt.base[k & 1], other = bt.base[(k - 1) & 1], live = bt.cnt[k - 1];
+      for (int it = threadIdx.x; it < bt.cnt[k] * G; it += TB_THREADS) {
+        const int b = own + it / G, g = it % G;
+        const char4 o = off[b];
+        const int x = wrap(mx + o.x, Lx), y = wrap(my + o.y, Ly), z = wrap(mz + o.z, Lz), t = wrap(mt + o.w, Lt);
+        const int s = x + Lx * (y + Ly * (z + Lz * t));
+        const fx::Torus nb(Lx, Ly, Lz, Lt, s);
+        Cx<double> acc[4][3], p[4][3], u[9];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) acc[a][c] = mk<double>(0.0, 0.0);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+          const int j = nbt[b * 8 + d];
+          if (j < 0 || j - other >= live) continue;
+          sm_spinor(at(j, g), p);
+          load_link<double>(U, (d >> 1) * V + ((d & 1) ? nb(d) : s), u);
+          if (d == 0) term_fwd<double, 0>(p, u, acc);
+          if (d == 1) term_bwd<double, 0>(p, u, acc);
+          if (d == 2) term_fwd<double, 1>(p, u, acc);
+          if (d == 3) term_bwd<double, 1>(p, u, acc);
+          if (d == 4) term_fwd<double, 2>(p, u, acc);
+          if (d == 5) term_bwd<double, 2>(p, u, acc);
+          if (d == 6) term_fwd<double, 3>(p, u, acc);
+          if (d == 7) term_bwd<double, 3>(p, u, acc);
+        }
+        double2 *dst = at(b, g);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) dst[i] = make_double2(acc[i / 3][i % 3].x, acc[i / 3][i % 3].y);
+      }
+      __syncthreads();
+      // contraction by the first warp: G lanes per task (local operator, or direction and term); the
+      // next order writes only sites of the other parity
+      if (threadIdx.x < 32) {
+        const int g = threadIdx.x % G, task = threadIdx.x / G, comp = c0 + g;
+        Cx<double> v = mk<double>(0.0, 0.0);
+        if (task < 8) {
+          if ((k & 1) == 0) {
+            Cx<double> w[4][3], gw[4][3];
+            if (task < 5) {
+              sm_spinor(at(bt.base[0], g), w);
+              if (task == 0) v = pick(w, comp);
+              if (task == 1) { gamma_apply<0>(w, gw); v = pick(gw, comp); }
+              if (task == 2) { gamma_apply<1>(w, gw); v = pick(gw, comp); }
+              if (task == 3) { gamma_apply<2>(w, gw); v = pick(gw, comp); }
+              if (task == 4) { gamma_apply<3>(w, gw); v = pick(gw, comp); }
+            }
+          } else {
+            // the source is the first site of parity 0; its neighbours are nbt[base[0]]
+            const int mu = task & 3, first = task >> 2;   // first: base site m - mu
+            const fx::Torus nb(Lx, Ly, Lz, Lt, m);
+            const int d = 2 * mu + first;
+            Cx<double> w[4][3], a[4][3], u[9];
+            sm_spinor(at(nbt[bt.base[0] * 8 + d], g), w);
+            load_link<double>(U, mu * V + (first ? nb(d) : m), u);
+            zero_sp<0>(a);
+            if (d == 0) term_fwd<double, 0>(w, u, a);
+            if (d == 1) term_bwd<double, 0>(w, u, a);
+            if (d == 2) term_fwd<double, 1>(w, u, a);
+            if (d == 3) term_bwd<double, 1>(w, u, a);
+            if (d == 4) term_fwd<double, 2>(w, u, a);
+            if (d == 5) term_bwd<double, 2>(w, u, a);
+            if (d == 6) term_fwd<double, 3>(w, u, a);
+            if (d == 7) term_bwd<double, 3>(w, u, a);
+            v = pick(a, comp);
+            if (!first) v = neg(v);
+          }
+        }
+        for (int h = 1; h < G; h <<= 1) {
+          v.x += __shfl_xor_sync(0xffffffffu, v.x, h);
+          v.y += __shfl_xor_sync(0xffffffffu, v.y, h);
+        }
+        // the two point-split terms of mu < 3 are added on the lane of the second one
+        const double ox = __shfl_down_sync(0xffffffffu, v.x, 4 * G % 32), oy = __shfl_down_sync(0xffffffffu, v.y, 4 * G % 32);
+        if (g == 0 && task < 8) {
+          int q = -1;
+          if ((k & 1) == 0) {
+            if (task < 5) q = task;
+          } else if (task < 4) {
+            q = 5 + task;
+            if (task < 3) { v.x += ox; v.y += oy; }
+          } else if (task == 7) {
+            q = 9;
+          }
+          if (q >= 0) {
+            res[k][q].x += v.x;
+            res[k][q].y += v.y;
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < K * 10; i += TB_THREADS) part[(long long)i * nx + blockIdx.x] = res[i / 10][i % 10];
+}
+
+// out[q * Lt + t0 + blockIdx.y] = sum over the Vs sources of slice blockIdx.y of part row q (fixed order)
+__global__ void __launch_bounds__(256) trace_sum_kernel(const double2 *__restrict__ part, int Vs, int nx, int t0, int Lt,
+                                                        double2 *__restrict__ out) {
+  const double2 *p = part + (long long)blockIdx.x * nx + (long long)blockIdx.y * Vs;
+  KSum re, im;
+  re.init();
+  im.init();
+  for (int i = threadIdx.x; i < Vs; i += 256) {
+    re.add(p[i].x);
+    im.add(p[i].y);
+  }
+  __shared__ double2 red[256];
+  red[threadIdx.x] = make_double2(re.value(), im.value());
+  __syncthreads();
+  for (int h = 128; h > 0; h >>= 1) {
+    if (threadIdx.x < h) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + h]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) out[(long long)blockIdx.x * Lt + t0 + blockIdx.y] = red[0];
+}
+
+// Whether the traces of K terms are followed site by site: no winding walk, and the ball in shared memory
+static bool trace_local(const int *d, int K) {
+  if (K < 2 || K / 2 > TB_MAXR || K > TB_MAXK) return false;
+  for (int i = 0; i < 4; ++i)
+    if (d[i] <= K) return false;
+  return true;
+}
+
 template <typename T>
 lqcd_status download_v(lqcd_ctx *ctx, const void *dev, std::vector<T> &h, size_t count) {
   h.resize(count);
@@ -696,10 +871,85 @@ static lqcd_status poly_coeffs_dev(lqcd_ctx *ctx, const double2 *U, double kappa
   return LQCD_OK;
 }
 
+// The traces site by site (trace_ball_kernel); tr as in hop_traces_dev
+static lqcd_status hop_traces_local(lqcd_ctx *ctx, const double2 *U, double kappa, int K, std::vector<cd> &tr) {
+  const int *d = ctx->dims;
+  const int Lt = d[3], Vs = d[0] * d[1] * d[2];
+  // the ball of radius K / 2, by parity and distance, and the neighbours of its sites in it
+  const std::vector<char4> ball = taxicab_ball(std::max(1, K / 2));
+  auto dist = [](const char4 &o) { return std::abs(o.x) + std::abs(o.y) + std::abs(o.z) + std::abs(o.w); };
+  std::vector<char4> sites = ball;
+  std::stable_sort(sites.begin(), sites.end(), [&](const char4 &a, const char4 &b) {
+    const int da = dist(a), db = dist(b);
+    return (da & 1) != (db & 1) ? (da & 1) < (db & 1) : da < db;
+  });
+  BallTable bt{};
+  bt.n = (int)sites.size();
+  bt.base[0] = 0;
+  while (bt.base[1] < bt.n && (dist(sites[bt.base[1]]) & 1) == 0) ++bt.base[1];
+  for (int k = 0; k < K; ++k) {
+    const int r = k == 0 ? 0 : std::min(k, completion_radius(K, k));
+    for (int i = bt.base[k & 1]; i < bt.n && ((dist(sites[i]) ^ k) & 1) == 0 && dist(sites[i]) <= r; ++i) ++bt.cnt[k];
+  }
+  std::vector<short> nb(8 * sites.size(), -1);
+  for (int i = 0; i < bt.n; ++i)
+    for (int e = 0; e < 8; ++e) {
+      char4 o = sites[i];
+      const int sg = (e & 1) ? -1 : 1;
+      if (e / 2 == 0) o.x += sg;
+      if (e / 2 == 1) o.y += sg;
+      if (e / 2 == 2) o.z += sg;
+      if (e / 2 == 3) o.w += sg;
+      for (int j = 0; j < bt.n; ++j)
+        if (sites[j].x == o.x && sites[j].y == o.y && sites[j].z == o.z && sites[j].w == o.w) nb[8 * i + e] = (short)j;
+    }
+  // four components per block while two blocks fit an SM (radius 3: 105 KB each), else two (radius 4: 130 KB)
+  const int G = bt.n <= 129 ? 4 : 2;
+  const int smem = bt.n * G * TB_SITE;
+  const size_t tab = sizeof(char4) * sites.size();
+  char *td;
+  LQCD_TRY(ws_get(ctx, WS_PROBE_OFF, tab + sizeof(short) * nb.size(), (void **)&td));
+  LQCD_CUDA(ctx, cudaMemcpyAsync(td, sites.data(), tab, cudaMemcpyHostToDevice, ctx->stream));
+  LQCD_CUDA(ctx, cudaMemcpyAsync(td + tab, nb.data(), sizeof(short) * nb.size(), cudaMemcpyHostToDevice, ctx->stream));
+  // whole timeslices per launch, 256 MiB of per-source results at most
+  const int nt = (int)std::max<long long>(1, std::min<long long>(Lt, (256ll << 20) / ((long long)K * 160 * Vs)));
+  double2 *part, *out;
+  LQCD_TRY(ws_get(ctx, WS_PROBE, sizeof(double2) * (size_t)K * 10 * nt * Vs, (void **)&part));
+  LQCD_TRY(ws_get(ctx, WS_EST0, sizeof(double2) * (size_t)K * 10 * Lt, (void **)&out));
+  LQCD_CUDA(ctx, cudaFuncSetAttribute(trace_ball_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  for (int t0 = 0; t0 < Lt; t0 += nt) {
+    const int n = std::min(nt, Lt - t0), nx = n * Vs;
+    kbegin(ctx);
+    trace_ball_kernel<<<nx, TB_THREADS, smem, ctx->stream>>>(U, K, G, bt, (const char4 *)td, (const short *)(td + tab),
+                                                            t0 * Vs, nx, d[0], d[1], d[2], d[3], part);
+    LQCD_TRY(launch_check(ctx, "trace_ball_kernel", K_PROBE, 12.0 * nx));
+    kbegin(ctx);
+    trace_sum_kernel<<<dim3(K * 10, n), 256, 0, ctx->stream>>>(part, Vs, nx, t0, Lt, out);
+    LQCD_TRY(launch_check(ctx, "trace_sum_kernel", K_PROBE, 0.0));
+  }
+  std::vector<double2> h;
+  LQCD_TRY(download_v(ctx, out, h, (size_t)K * 10 * Lt));
+  tr.assign((size_t)K * 9 * Lt, cd(0.0, 0.0));
+  for (int t = 0; t < Lt; ++t) tr[t] = 12.0 * Vs;   // order 0: the identity
+  for (int k = 1; k < K; ++k)
+    for (int q = 0; q < 9; ++q)
+      for (int t = 0; t < Lt; ++t) {
+        cd v(h[((size_t)k * 10 + q) * Lt + t].x, h[((size_t)k * 10 + q) * Lt + t].y);
+        if (q == 8) {
+          const double2 a = h[((size_t)k * 10 + 9) * Lt + (t + 1) % Lt];
+          v += cd(a.x, a.y);
+        }
+        tr[((size_t)k * 9 + q) * Lt + t] = q >= 5 ? kappa * v : v;
+      }
+  return LQCD_OK;
+}
+
 // t[(k * 9 + op) * Lt + t] for k < K
 static lqcd_status hop_traces_dev(lqcd_ctx *ctx, const double2 *U, double kappa, int K, std::vector<cd> &tr) {
-  FxScope scope(ctx);
   const int *d = ctx->dims;
+  // a depth that the caller fixed is one of the probing form
+  if (ctx->probe_depth == 0 && trace_local(d, K)) return hop_traces_local(ctx, U, kappa, K, tr);
+  FxScope scope(ctx);
   const int Lt = d[3];
   const long long N = ctx->N;
   const Colouring col = choose_colouring(d, K);

@@ -1,9 +1,9 @@
 """Launch forms that depend on sizes, where they can go wrong: right-hand sides split over a block in the
-link gradient, chunks of a timeslice in the contraction."""
+link gradient, chunks of a timeslice in the contraction, hopping traces by site."""
 import numpy as np
 import pytest
 
-from oracle import derivs as Dv, lattice as L, operators as O
+from oracle import derivs as Dv, lattice as L, operators as O, subtract as S
 from paper_1903_06986_gb300 import lqcd, synth
 from tests.gpu_util import context, dev, host, rel_err
 
@@ -49,3 +49,27 @@ def test_contract_chunks(dims, n):
     got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
     ref = O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
     assert rel_err(got, ref) < 1e-13
+
+
+@pytest.mark.parametrize("dims,K", [((3, 3, 3, 3), 2), ((4, 5, 4, 6), 3), ((5, 5, 6, 5), 4), ((6, 8, 6, 7), 5),
+                                    ((7, 7, 7, 8), 6), ((8, 8, 8, 9), 7), ((9, 9, 9, 10), 8)])
+def test_hop_traces_by_site(dims, K):
+    """Extents just above K (no walk of the trace winds) and odd ones: source by source against the
+    probing form with every order a full application, order by order."""
+    ctx = context(dims)
+    Ud = dev(synth.su3_links(dims, 0.5, 11))
+    got = ctx.hop_traces(Ud, 0.13, K)
+    ctx.set_probe_depth(max(1, K - 1))
+    want = ctx.hop_traces(Ud, 0.13, K)
+    # order k sums V terms of size up to 8^k / ... : relative to the largest entry of the order, or to the
+    # rounding of the 12 V unit terms where the order vanishes
+    for k in range(K):
+        scale = max(np.abs(want[k]).max(), 12.0 * np.prod(dims[:3]) * 2.0 ** k)
+        assert np.abs(got[k] - want[k]).max() <= 1e-13 * scale, k
+
+
+def test_hop_traces_by_site_against_the_oracle():
+    dims, K = (4, 4, 5, 4), 3
+    ctx = context(dims)
+    U = synth.su3_links(dims, 0.5, 12)
+    assert rel_err(ctx.hop_traces(dev(U), 0.13, K), O.per_t(S.hop_traces(U, 0.13, K, dims))) < 1e-13
