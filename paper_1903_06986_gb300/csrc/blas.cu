@@ -384,11 +384,11 @@ __global__ void __launch_bounds__(BT) multiaxpy_vec_kernel(const SV *__restrict_
   *reinterpret_cast<uint4 *>(wp) = raw;
 }
 
-constexpr int CT = 8;           // output columns per pass in combine
+constexpr int COMB_CT = 8;      // most output columns per pass in combine
 constexpr int COMB_MAXV = 256;  // basis vectors of one combine (coefficient tile in shared memory)
 // out_c^r = fac * sum_i V_i^r C[(i * ncol + c) * nrhs + r]; a tile of CT columns of coefficients for
 // this right-hand side is staged in shared memory per pass.
-template <typename SV, typename SO>
+template <typename SV, typename SO, int CT>
 __global__ void __launch_bounds__(BT) combine_kernel(const SV *__restrict__ V, long long vstride,
                                                      long long vrs, int nvec, const double2 *__restrict__ Cf,
                                                      int ncol, double fac, SO *__restrict__ out, long long ostride,
@@ -703,7 +703,7 @@ lqcd_status blas_g5(lqcd_ctx *ctx, const double2 *x, double2 *y, int nrhs) {
 }
 
 // per-right-hand-side arrival counters of the single-launch reductions (zeroed once, left at zero)
-static lqcd_status reduction_counters(lqcd_ctx *ctx, int nrhs, unsigned **c) {
+lqcd_status reduction_counters(lqcd_ctx *ctx, int nrhs, unsigned **c) {
   const size_t need = sizeof(unsigned) * (size_t)std::max(nrhs, 1);
   const bool fresh = ctx->ws_size[WS_COUNT] < need;
   LQCD_TRY(ws_get(ctx, WS_COUNT, need, (void **)c));
@@ -846,8 +846,11 @@ lqcd_status blas_combine(lqcd_ctx *ctx, const SV *V, long long vstride, long lon
     combine_vec_kernel<SV, SO><<<(unsigned)((long long)ceil_div(n / kv, BT) * nrhs), BT, 0, ctx->stream>>>(
         V, vstride, vrs, nvec, C, ncol, fac, out, ostride, n, nrhs);
   } else {
-    combine_kernel<SV, SO><<<(unsigned)((long long)ceil_div(n, BT) * nrhs), BT, 0, ctx->stream>>>(
-        V, vstride, vrs, nvec, C, ncol, fac, out, ostride, n, nrhs);
+    // one column (the residual of a GMRES-Proj cycle, the HFES product) does not pay for eight: 7.8 ms with
+    // the wide form, 1.9 ms with one column, for 31 vectors of 50 right-hand sides of 8^3 x 16
+    (ncol == 1 ? combine_kernel<SV, SO, 1> : combine_kernel<SV, SO, COMB_CT>)
+        <<<(unsigned)((long long)ceil_div(n, BT) * nrhs), BT, 0, ctx->stream>>>(V, vstride, vrs, nvec, C, ncol, fac,
+                                                                               out, ostride, n, nrhs);
   }
   const double bytes = (double)sizeof(SV) * n * nvec * (vrs != 0 ? nrhs : 1) + (double)sizeof(SO) * n * ncol * nrhs;
   return launch_check_bytes(ctx, "combine_kernel", K_COMBINE, (double)n * nrhs * nvec * ncol, bytes);

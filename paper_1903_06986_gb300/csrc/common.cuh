@@ -137,7 +137,7 @@ enum WsSlot {
   WS_PARTIAL = 0, WS_SCAL, WS_TMP0, WS_TMP1, WS_TMP2, WS_TMP3, WS_BASIS, WS_HESS, WS_COEF,
   WS_BASIS2, WS_TMP4, WS_TMP5, WS_EST0, WS_EST1, WS_EST2, WS_PROBE,
   WS_MIX_U, WS_MIX_V, WS_MIX_R32, WS_MIX_E32, WS_MIX_R, WS_MIX_S, WS_COUNT, WS_TUNE, WS_SPEC, WS_NBLK, WS_TC_STAT, WS_TC_B, WS_TC_PART, WS_TC_D,
-  WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_FX_LINKS, WS_FX_FIELD, WS_NSLOTS
+  WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_FX_LINKS, WS_FX_FIELD, WS_FX_BASIS, WS_NSLOTS
 };
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr);
 void graph_cache_clear(lqcd_ctx *ctx);
@@ -161,6 +161,21 @@ lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use);
 // workspace for up to chunk fields of S sites in that form (use as above), and the conversion into it
 lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *chunk, bool *use);
 lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs);
+// FP64 operator (flags as wilson_launch, or 4 with g5mask) on nrhs fields whose integers are f; in: the
+// same fields, canonical
+lqcd_status wilson_launch_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,
+                                    double2 *out, int nrhs, int flags, unsigned long long g5mask);
+lqcd_status eo_schur_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,
+                               double2 *out, int nrhs, int flags);
+// Gram-Schmidt on the integers of a basis (fxblas.cu): field i * nrhs + r of f is basis vector i of
+// right-hand side r, V the same in canonical FP64; fields of S sites
+lqcd_status fx_blas_reserve(lqcd_ctx *ctx, long long S, int nrhs, int max_nvec);
+lqcd_status fx_multidot(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, const double2 *w, long long S, int nvec,
+                        int nrhs, double2 *h);
+lqcd_status fx_multiaxpy(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, const double2 *h, double sign, double2 *w,
+                         long long S, int nvec, int nrhs);
+// arrival counters of the single-launch reductions (zeroed once, left at zero)
+lqcd_status reduction_counters(lqcd_ctx *ctx, int n, unsigned **c);
 void fx_done(lqcd_ctx *ctx);   // records the end of a use (outside scopes; a scope does it at its end)
 struct FxScope {
   lqcd_ctx *ctx;

@@ -194,7 +194,8 @@ __global__ void eo_pair_kernel(const double2 *__restrict__ ve, const double2 *__
 
 template <typename R, int FL>
 lqcd_status hop_launch(lqcd_ctx *ctx, const double2 *U, const double2 *in, const double2 *self, double2 *out,
-                       double coef, int nrhs, int par) {
+                       double coef, int nrhs, int par, const fx::Field *pre = nullptr) {
+  // pre (FP64): the integers of in, when the caller has them
   const int *d = ctx->eo_dims;
   // compulsory bytes: the input half read, the output half written (plus the added half), links once
   const double bytes = (2.0 + ((FL & EO_SELF) ? 1.0 : 0.0)) * nrhs * ctx->V * 12 * 16.0 + 36.0 * 2 * ctx->V * 16.0;
@@ -206,12 +207,17 @@ lqcd_status hop_launch(lqcd_ctx *ctx, const double2 *U, const double2 *in, const
     const long long S = (FL & EO_IN_FULL) ? 2LL * ctx->V : ctx->V;
     const long long So = (FL & EO_OUT_FULL) ? 2LL * ctx->V : ctx->V, Ss = (FL & EO_SELF_FULL) ? 2LL * ctx->V : ctx->V;
     LQCD_TRY(fx_links(ctx, U, &L, &use));
-    if (use) LQCD_TRY(fx_field(ctx, S, nrhs, &f, &chunk, &use));
+    if (use && pre) {
+      f = *pre;
+      chunk = nrhs;
+    } else if (use) {
+      LQCD_TRY(fx_field(ctx, S, nrhs, &f, &chunk, &use));
+    }
     if (use) {
       for (int r0 = 0; r0 < nrhs; r0 += chunk) {
         const int nr = std::min(chunk, nrhs - r0);
         const double2 *src = in + 12 * S * r0;
-        LQCD_TRY(fx_convert(ctx, src, f, S, nr));
+        if (!pre) LQCD_TRY(fx_convert(ctx, src, f, S, nr));
         const bool split = fx::use_split(ctx->V, nr, ctx->sms);
         kbegin(ctx);
         (split ? eo_hop_fx_kernel<FL, 4> : eo_hop_fx_kernel<FL, 1>)
@@ -253,23 +259,23 @@ lqcd_status check_nrhs(lqcd_ctx *ctx, int nrhs, const char *what) {
 // context.  R = double (FP64) or float (FP32 arithmetic on FP64 storage).
 template <typename R>
 lqcd_status eo_schur_launch_t(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out,
-                              int nrhs, int flags) {
+                              int nrhs, int flags, const fx::Field *pre = nullptr) {
   FxScope scope(ctx);   // two hopping launches, one conversion of the links
   double2 *tmp;
   LQCD_TRY(ws_get(ctx, WS_EO, sizeof(double2) * (size_t)nrhs * ctx->N, (void **)&tmp));
   const double k2 = -kappa * kappa;
   switch (flags) {
     case LQCD_APPLY_M:
-      LQCD_TRY((hop_launch<R, 0>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1)));
+      LQCD_TRY((hop_launch<R, 0>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1, pre)));
       return hop_launch<R, EO_SELF>(ctx, U, tmp, in, out, k2, nrhs, 0);
     case LQCD_APPLY_G5R:
-      LQCD_TRY((hop_launch<R, EO_HOP_G5>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1)));
+      LQCD_TRY((hop_launch<R, EO_HOP_G5>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1, pre)));
       return hop_launch<R, EO_SELF | EO_SELF_G5>(ctx, U, tmp, in, out, k2, nrhs, 0);
     case LQCD_APPLY_DAG:
-      LQCD_TRY((hop_launch<R, EO_HOP_G5>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1)));
+      LQCD_TRY((hop_launch<R, EO_HOP_G5>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1, pre)));
       return hop_launch<R, EO_SELF | EO_SELF_G5 | EO_LEFT_G5>(ctx, U, tmp, in, out, k2, nrhs, 0);
     case LQCD_APPLY_HOP:
-      LQCD_TRY((hop_launch<R, 0>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1)));
+      LQCD_TRY((hop_launch<R, 0>(ctx, U, in, nullptr, tmp, 1.0, nrhs, 1, pre)));
       return hop_launch<R, 0>(ctx, U, tmp, nullptr, out, 1.0, nrhs, 0);
     default:
       return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply (even/odd): unknown flags %d", flags);
@@ -281,6 +287,11 @@ lqcd_status eo_schur_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const
   if (prec == LQCD_PREC_F64) return eo_schur_launch_t<double>(ctx, U, kappa, in, out, nrhs, flags);
   if (prec == LQCD_PREC_F32) return eo_schur_launch_t<float>(ctx, U, kappa, in, out, nrhs, flags);
   return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply (even/odd): precision %d not available", prec);
+}
+
+lqcd_status eo_schur_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,
+                               double2 *out, int nrhs, int flags) {
+  return eo_schur_launch_t<double>(ctx, U, kappa, in, out, nrhs, flags, &f);
 }
 
 lqcd_status eo_reserve(lqcd_ctx *ctx, int nrhs) {

@@ -121,6 +121,10 @@ template <> struct OpT<double2> : PolyApply<double2, OpT<double2>> {
     if (flags == OP_MASKED) return wilson_launch_masked(ctx, U, kappa, in, out, nrhs, g5mask);
     return wilson_launch(ctx, U, kappa, in, out, nrhs, prec, flags);
   }
+  // out = A in with the integers of in at hand (no polynomial)
+  lqcd_status apply_converted(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, double2 *out, int nrhs) const {
+    return wilson_launch_converted(ctx, U, kappa, in, f, out, nrhs, flags == OP_MASKED ? 4 : flags, g5mask);
+  }
   void append_key(std::string &k) const {
     key_add(k, U);
     key_add(k, kappa);
@@ -222,6 +226,7 @@ template <typename S> struct ArnoldiT {
   double *nrm;         // [j][r]
   int passes = 2;      // Gram-Schmidt passes per step: 2 (CGS2), or 1 (CGS) for reduced-precision bases
   int window = 0;      // > 0 (Hermitian operators only): orthogonalise against the last `window` vectors
+  fx::Field fx{nullptr, nullptr};   // FP64: integers of the (m + 1) nrhs basis vectors (arnoldi_fx), or none
 };
 
 // First basis vector step j is orthogonalised against: all of them, or the last a.window (for a
@@ -239,12 +244,68 @@ template <typename S> struct ArnoldiLaunch {
   ArnoldiT<S> *a;
   int j0;
 };
+// The same steps on the integers of the basis: each new vector is converted once, for the operator and for
+// every later inner product and update (fxblas.cu).  CGS2 over all vectors, as FP64 solves take it.
+inline lqcd_status arnoldi_enqueue_fx(Arnoldi &a, int j0) {
+  lqcd_ctx *ctx = a.ctx;
+  const long long N = a.N, vs = (long long)a.nrhs * N, V = ctx->V, fq = fx::blocks32(V) * 384 * a.nrhs, fe = V * a.nrhs;
+  if (j0 > 0) LQCD_TRY(fx_convert(ctx, a.Vb, a.fx, V, j0 * a.nrhs));   // vectors kept by a restart
+  for (int j = j0; j < a.m; ++j) {
+    double2 *vj = a.Vb + j * vs, *w = a.Vb + (j + 1) * vs;
+    const fx::Field fj{a.fx.q + j * fq, a.fx.ex + j * fe};
+    LQCD_TRY(fx_convert(ctx, vj, fj, V, a.nrhs));
+    LQCD_TRY(a.op.apply_converted(ctx, vj, fj, w, a.nrhs));
+    for (double2 *hd : {a.hd1, a.hd2}) {
+      double2 *h = hd + (long long)j * (a.m + 1) * a.nrhs;
+      LQCD_TRY(fx_multidot(ctx, a.fx, a.Vb, w, V, j + 1, a.nrhs, h));
+      LQCD_TRY(fx_multiaxpy(ctx, a.fx, a.Vb, h, -1.0, w, V, j + 1, a.nrhs));
+    }
+    LQCD_TRY(blas_norms(ctx, w, N, a.nrhs, a.nrm + (long long)j * a.nrhs));
+    LQCD_TRY(blas_invscale(ctx, w, a.nrm + (long long)j * a.nrhs, N, a.nrhs));
+  }
+  return LQCD_OK;
+}
+
+// Workspace of the integers of a cycle's basis; none (the plain kernels) for a polynomial preconditioner,
+// for the FP32 operator, where the operator itself has no integers, or where the second copy of the
+// basis would take more than a third of the free memory.
+inline lqcd_status arnoldi_fx(Arnoldi &a) {
+  lqcd_ctx *ctx = a.ctx;
+  a.fx = fx::Field{nullptr, nullptr};
+  if (a.op.pp.degree > 0 || a.op.prec != LQCD_PREC_F64 || a.passes != 2 || a.window != 0 || a.m > 512) return LQCD_OK;
+  fx::Links L;
+  bool use;
+  LQCD_TRY(fx_links(ctx, a.op.U, &L, &use));
+  if (!use) return LQCD_OK;
+  const long long V = ctx->V, cnt = (long long)(a.m + 1) * a.nrhs;
+  if ((V / 32 + 1) * cnt > 0x7fffffffLL) return LQCD_OK;
+  const size_t qb = (size_t)cnt * fx::blocks32(V) * 384 * sizeof(longlong2), bytes = qb + (size_t)cnt * V * sizeof(int);
+  if (ctx->ws_size[WS_FX_BASIS] < bytes) {
+    size_t fr = 0, total = 0;
+    LQCD_CUDA(ctx, cudaMemGetInfo(&fr, &total));
+    if (bytes > (fr + ctx->ws_size[WS_FX_BASIS]) / 3) return LQCD_OK;
+  }
+  char *p;
+  const lqcd_status st = ws_get(ctx, WS_FX_BASIS, bytes, (void **)&p);
+  if (st == LQCD_ERR_OOM) {
+    ctx->err.clear();
+    return LQCD_OK;
+  }
+  LQCD_TRY(st);
+  a.fx.q = (longlong2 *)p;
+  a.fx.ex = (int *)(p + qb);
+  return fx_blas_reserve(ctx, V, a.nrhs, a.m);
+}
+
 template <typename S>
 lqcd_status arnoldi_enqueue(void *arg) {
   ArnoldiT<S> &a = *((ArnoldiLaunch<S> *)arg)->a;
   const int j0 = ((ArnoldiLaunch<S> *)arg)->j0;
   lqcd_ctx *ctx = a.ctx;
   const long long N = a.N, vs = (long long)a.nrhs * N;
+  if constexpr (std::is_same<S, double2>::value) {
+    if (a.fx.q) return arnoldi_enqueue_fx(a, j0);
+  }
   for (int j = j0; j < a.m; ++j) {
     S *vj = a.Vb + j * vs, *w = a.Vb + (j + 1) * vs;
     LQCD_TRY(a.op.apply(ctx, vj, w, a.nrhs));
@@ -271,6 +332,7 @@ lqcd_status arnoldi_launch(ArnoldiT<S> &a, int j0) {
   if (j0 >= a.m) return LQCD_OK;
   LQCD_TRY(blas_reserve(a.ctx, a.N, a.nrhs, a.m));
   LQCD_TRY(a.op.reserve(a.ctx, a.nrhs));
+  if constexpr (std::is_same<S, double2>::value) LQCD_TRY(arnoldi_fx(a));
   std::string key("arnoldi");
   key_add(key, StoreTag<S>::value);
   a.op.append_key(key);
@@ -284,6 +346,7 @@ lqcd_status arnoldi_launch(ArnoldiT<S> &a, int j0) {
   key_add(key, j0);
   key_add(key, a.passes);
   key_add(key, a.window);
+  key_add(key, a.fx.q);
   key_add(key, a.ctx->packed_nr);
   ArnoldiLaunch<S> arg{&a, j0};
   return graph_cached(a.ctx, key, &arnoldi_enqueue<S>, &arg);

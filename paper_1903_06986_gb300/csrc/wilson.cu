@@ -217,17 +217,36 @@ __global__ void __launch_bounds__(FX_BS, 4) wilson_fx_kernel(const double2 *__re
                         (mode & FX_G5LEFT) != 0, out + (long long)r * V * 12, s0 < V ? s : -1);
 }
 
+int fx_mode(int flags) {
+  switch (flags) {
+    case LQCD_APPLY_M: return 0;
+    case LQCD_APPLY_G5R: return FX_G5IN;
+    case LQCD_APPLY_DAG: return FX_G5IN | FX_G5LEFT;
+    case LQCD_APPLY_HOP: return FX_HOP;
+    case 4: return FX_MASK;
+    default: return -1;
+  }
+}
+
+// one launch: nr fields with the integers f
+lqcd_status fx_apply(lqcd_ctx *ctx, const double2 *U, const fx::Links &L, const fx::Field &f, double kappa,
+                     const double2 *in, double2 *out, int nr, int mode, unsigned long long g5mask) {
+  const int *d = ctx->dims;
+  const bool split = fx::use_split(ctx->V, nr, ctx->sms);
+  const long long grid = (long long)ceil_div(ctx->V, split ? 32 : FX_BS) * nr;
+  if (grid > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson: grid too large");
+  kbegin(ctx);
+  (split ? wilson_fx_kernel<4> : wilson_fx_kernel<1>)<<<(unsigned)grid, FX_BS, 0, ctx->stream>>>(
+      U, L, f, in, out, kappa, d[0], d[1], d[2], d[3], ctx->V, nr, mode, g5mask);
+  // compulsory bytes: each field read and written once, the links once
+  const double bytes = 2.0 * nr * ctx->V * 12 * 16 + 36.0 * ctx->V * 16;
+  return launch_check_bytes(ctx, "wilson_fx_kernel", K_WILSON, (double)ctx->V * nr, bytes);
+}
+
 lqcd_status fx_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out, int nrhs,
                       int flags, unsigned long long g5mask) {
-  int mode = 0;
-  switch (flags) {
-    case LQCD_APPLY_M: break;
-    case LQCD_APPLY_G5R: mode = FX_G5IN; break;
-    case LQCD_APPLY_DAG: mode = FX_G5IN | FX_G5LEFT; break;
-    case LQCD_APPLY_HOP: mode = FX_HOP; break;
-    case 4: mode = FX_MASK; break;
-    default: return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply: unknown flags %d", flags);
-  }
+  const int mode = fx_mode(flags);
+  if (mode < 0) return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson_apply: unknown flags %d", flags);
   fx::Links L;
   fx::Field f;
   bool use;
@@ -235,20 +254,11 @@ lqcd_status fx_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const doubl
   LQCD_TRY(fx_links(ctx, U, &L, &use));
   if (use) LQCD_TRY(fx_field(ctx, ctx->V, nrhs, &f, &chunk, &use));
   if (!use) return launch_mode<double, double2>(ctx, U, kappa, in, out, nrhs, flags, g5mask);
-  const int *d = ctx->dims;
   for (int r0 = 0; r0 < nrhs; r0 += chunk) {
     const int nr = std::min(chunk, nrhs - r0);
     const double2 *src = in + (long long)r0 * ctx->N;
     LQCD_TRY(fx_convert(ctx, src, f, ctx->V, nr));
-    const bool split = fx::use_split(ctx->V, nr, ctx->sms);
-    kbegin(ctx);
-    (split ? wilson_fx_kernel<4> : wilson_fx_kernel<1>)
-        <<<(unsigned)((long long)ceil_div(ctx->V, split ? 32 : FX_BS) * nr), FX_BS, 0, ctx->stream>>>(
-            U, L, f, src, out + (long long)r0 * ctx->N, kappa, d[0], d[1], d[2], d[3], ctx->V, nr, mode,
-            flags == 4 ? g5mask >> r0 : 0ull);
-    // compulsory bytes: each field read and written once, the links once
-    const double bytes = 2.0 * nr * ctx->V * 12 * 16 + 36.0 * ctx->V * 16;
-    LQCD_TRY(launch_check_bytes(ctx, "wilson_fx_kernel", K_WILSON, (double)ctx->V * nr, bytes));
+    LQCD_TRY(fx_apply(ctx, U, L, f, kappa, src, out + (long long)r0 * ctx->N, nr, mode, flags == 4 ? g5mask >> r0 : 0ull));
   }
   if (ctx->fx_depth == 0) fx_done(ctx);
   return LQCD_OK;
@@ -322,6 +332,20 @@ void fx_done(lqcd_ctx *ctx) {
   }
   cudaEventRecord(ctx->fx_event, ctx->stream);
   ctx->fx_event_stream = ctx->stream;
+}
+
+lqcd_status wilson_launch_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,
+                                    double2 *out, int nrhs, int flags, unsigned long long g5mask) {
+  if (ctx->eo) return eo_schur_converted(ctx, U, kappa, in, f, out, nrhs, flags);
+  const int mode = fx_mode(flags);
+  if (mode < 0) return set_err(ctx, LQCD_ERR_INVALID_ARG, "wilson: unknown flags %d", flags);
+  fx::Links L;
+  bool use;
+  LQCD_TRY(fx_links(ctx, U, &L, &use));
+  if (!use) return launch_mode<double, double2>(ctx, U, kappa, in, out, nrhs, flags, g5mask);
+  LQCD_TRY(fx_apply(ctx, U, L, f, kappa, in, out, nrhs, mode, g5mask));
+  if (ctx->fx_depth == 0) fx_done(ctx);
+  return LQCD_OK;
 }
 
 lqcd_status wilson_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, double2 *out, int nrhs,
