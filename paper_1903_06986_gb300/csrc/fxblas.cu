@@ -194,10 +194,13 @@ __global__ void __launch_bounds__(FB, 2) fx_multidot_kernel(Field f, const doubl
 
 // w^r += sign * sum_i V_i^r h[i * nrhs + r].  Block: 32 sites of one right-hand side, warp = spin, so that a
 // thread sums three complex components.  Coefficients as 59-bit integers with one exponent each.
+// VS > 1, for fields that leave most of the chip idle: VS = 4 such groups of four warps share the sites and
+// take every fourth vector, and their integers at the one exponent are added.
 // Eight blocks per SM (64 registers): 4.8 TB/s on 50 right-hand sides of 8^3 x 16, 4.1 to 4.4 with four to
 // six; the FP64 sums ran at 1.3.
 constexpr int FAXPY_MAXV = 512;
-__global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const double2 *__restrict__ V,
+template <int VS>
+__global__ void __launch_bounds__(FB * VS, 8 / VS) fx_multiaxpy_kernel(Field f, const double2 *__restrict__ V,
                                                              const double2 *__restrict__ h, double sign,
                                                              double2 *__restrict__ w, int S, int nvec, int nrhs) {
   extern __shared__ __align__(16) char dyn[];   // coefficients int4[nvec], exponents int[nvec]
@@ -205,14 +208,14 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
   int4 *cf = (int4 *)dyn;
   int *cx = (int *)(cf + nvec);
   const int r = blockIdx.x % nrhs;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, gw = threadIdx.x >> 5, warp = gw % 4, vg = gw / 4;   // spin, vector group
   const int s0 = (blockIdx.x / nrhs) * 32 + lane, s = min(s0, S - 1);
   double2 *wr = w + (long long)r * S * 12;
   Stage st;
   st.init(sm);
-  st.load<4>(wr, s, warp);
+  if (vg == 0) st.load<4>(wr, s, warp);
   bool odd = false;   // a coefficient outside the range of the integers
-  for (int i = threadIdx.x; i < nvec; i += FB) {
+  for (int i = threadIdx.x; i < nvec; i += FB * VS) {
     const double2 a = h[(long long)i * nrhs + r];
     const int X = max(abs_hi(a.x), abs_hi(a.y)) >> 20;
     const bool zero = a.x == 0.0 && a.y == 0.0;
@@ -228,9 +231,9 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
   odd = __syncthreads_or(odd) != 0;
   const long long fq = blocks32(S) * 384;
   // the exponent of the sum: sum_i 2^(X_i) <= 2^(E + 6) with X_i = X_V + X_h, E at least their largest.
-  // Zero blocks and coefficients have no share.  Each warp looks at a quarter of the vectors.
-  __shared__ float s_tot[FB / 32][32];
-  __shared__ int s_E[FB / 32][32];
+  // Zero blocks and coefficients have no share.  Each warp looks at its share of the vectors.
+  __shared__ float s_tot[4 * VS][32];
+  __shared__ int s_E[4 * VS][32];
   int E = 0;
   float tot = 0.f;
   auto share = [](int &E, float &tot, int X, float n) {   // (E, tot) += n 2^X
@@ -243,34 +246,34 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
     }
   };
 #pragma unroll 4
-  for (int i = warp; i < nvec; i += FB / 32) {
+  for (int i = gw; i < nvec; i += 4 * VS) {
     const int xv = __ldg(f.ex + ((long long)i * nrhs + r) * S + s), xh = cx[i];
     if (xv == FX_MINX || xh == 0) continue;
     const int X = xv + xh;
     odd = odd || X > X_HIGH || X < X_LOW;
     share(E, tot, X, 1.f);
   }
-  s_E[warp][lane] = E;
-  s_tot[warp][lane] = odd ? INFINITY : tot;
+  s_E[gw][lane] = E;
+  s_tot[gw][lane] = odd ? INFINITY : tot;
   __syncthreads();
   E = 0;
   tot = 0.f;
   bool bad = false;
 #pragma unroll
-  for (int k = 0; k < FB / 32; ++k) {
+  for (int k = 0; k < 4 * VS; ++k) {
     bad = bad || isinf(s_tot[k][lane]);
     if (s_E[k][lane] > 0) share(E, tot, s_E[k][lane], s_tot[k][lane]);
   }
   E += max(0, (__float_as_int(tot) >> 23) - 127 + 1 - 6);
   double2 *m = st.mine() + 3 * warp;
-  if (!bad) {
-    long long hh[3][2], md[3][2];
+  long long hh[3][2], md[3][2];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) hh[c][0] = hh[c][1] = 0, md[c][0] = md[c][1] = 1ll << 31;
-    const longlong2 *q = f.q + (long long)r * fq + slot(s, 12) + 3 * warp * 32;
-    const int *ex = f.ex + (long long)r * S + s;
+  for (int c = 0; c < 3; ++c) hh[c][0] = hh[c][1] = 0, md[c][0] = md[c][1] = 1ll << 31;
+  if (!bad) {
+    const longlong2 *q = f.q + ((long long)vg * nrhs + r) * fq + slot(s, 12) + 3 * warp * 32;
+    const int *ex = f.ex + ((long long)vg * nrhs + r) * S + s;
 #pragma unroll 4
-    for (int i = 0; i < nvec; ++i, q += (long long)nrhs * fq, ex += (long long)nrhs * S) {
+    for (int i = vg; i < nvec; i += VS, q += (long long)VS * nrhs * fq, ex += (long long)VS * nrhs * S) {
       const int4 k = cf[i];
       const int sh = max(0, min(E - __ldg(ex) - cx[i], 63));   // out of 0..63 only where the product is 0
       const int nzh = -k.z, nzl = -k.w;
@@ -293,7 +296,7 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
         md[c][0] = madw(md[c][0], nzl, ih);
         md[c][1] = madw(md[c][1], k.w, rh);
       }
-      if ((i & 3) == 3) {   // four vectors: |md| < 2^63
+      if ((i / VS & 3) == 3) {   // four vectors: |md| < 2^63
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -303,11 +306,33 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
           }
       }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int z = 0; z < 2; ++z) hh[c][z] = madw(hh[c][z], (int)(md[c][z] >> 32), 1);
+  }
+  if constexpr (VS > 1) {
+    __shared__ long long part[VS - 1][6][FB];
+    if (vg > 0) {
+#pragma unroll
+      for (int z = 0; z < 6; ++z) part[vg - 1][z][threadIdx.x % FB] = hh[z / 2][z % 2];
+    }
+    __syncthreads();
+    if (vg == 0) {
+#pragma unroll
+      for (int g = 0; g < VS - 1; ++g)
+#pragma unroll
+        for (int z = 0; z < 6; ++z) hh[z / 2][z % 2] += part[g][z][threadIdx.x];
+    }
+  }
+  if (vg > 0) {
+    // the first group ends the sum
+  } else if (!bad) {
     // E = 0: every share was zero
     const double k = E >= X_LOW ? pow2(E - 2099) : 0.0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const long long re = madw(hh[c][0], (int)(md[c][0] >> 32), 1), im = madw(hh[c][1], (int)(md[c][1] >> 32), 1);
+      const long long re = hh[c][0], im = hh[c][1];
       const double2 o = m[c];
       m[c] = make_double2(fma((double)re, k, o.x), fma((double)im, k, o.y));
     }
@@ -323,7 +348,7 @@ __global__ void __launch_bounds__(FB, 8) fx_multiaxpy_kernel(Field f, const doub
     for (int c = 0; c < 3; ++c) m[c] = a[c];
   }
   __syncthreads();
-  st.store<4>(wr, s0 < S ? s : -1, warp);
+  if (vg == 0) st.store<4>(wr, s0 < S ? s : -1, warp);
 }
 
 // blocks per (right-hand side, vector group): about 12 blocks per SM, six resident rounds; at least one
@@ -363,7 +388,8 @@ lqcd_status fx_multiaxpy(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, co
   const long long grid = fx::blocks32(S) * nrhs;
   if (grid > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "fx_multiaxpy: grid too large");
   kbegin(ctx);
-  fx_multiaxpy_kernel<<<(unsigned)grid, FB, nvec * (sizeof(int4) + sizeof(int)), ctx->stream>>>(f, V, h, sign, w, (int)S,
-                                                                                              nvec, nrhs);
+  const int vs = grid < 4LL * ctx->sms && nvec > 1 ? 4 : 1;   // fewer than 16 warps per SM
+  (vs == 4 ? fx_multiaxpy_kernel<4> : fx_multiaxpy_kernel<1>)
+      <<<(unsigned)grid, FB * vs, nvec * (sizeof(int4) + sizeof(int)), ctx->stream>>>(f, V, h, sign, w, (int)S, nvec, nrhs);
   return launch_check_bytes(ctx, "fx_multiaxpy_kernel", K_AXPY, 12.0 * S * nrhs * nvec, 196.0 * S * nrhs * nvec + 384.0 * S * nrhs);
 }

@@ -69,7 +69,7 @@ def test_hop_traces_by_site(dims, K):
 
 
 def test_hop_traces_by_site_against_the_oracle():
-    dims, K = (4, 4, 5, 4), 3
+    dims, K = (4, 4, 4, 4), 3
     ctx = context(dims)
     U = synth.su3_links(dims, 0.5, 12)
     assert rel_err(ctx.hop_traces(dev(U), 0.13, K), O.per_t(S.hop_traces(U, 0.13, K, dims))) < 1e-13
