@@ -67,6 +67,29 @@ __device__ __forceinline__ double2 warp_sum2(double2 v) {
   return v;
 }
 
+// Sums of N doubles per lane over the warp (N = 4 or 16): the halves of the values go to the halves of the
+// lanes, so that N - 1 + log2(32 / N) additions do instead of 5 N; returns sum number
+// (lane >> (5 - log2 N)), valid in every lane.  FP64 additions cost 16 clocks per warp and SM, and the
+// 5 N form was most of a two-vector product on short vectors (45 us for eight right-hand sides of
+// 12^3 x 24 in FP16, with the launch shape of multidot_chunks 12).
+template <int N>
+__device__ __forceinline__ double warp_sums(double *v) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      const double send = up ? v[j] : v[j + n], keep = up ? v[j + n] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
 // conj(V_j[e]) w[e] summed into acc[j] over the elements e0 + t, e0 + t + BT, ... < e1 of this thread
 // (t = threadIdx.x), for the first g of the G vectors (all of them when FULL)
 template <bool FULL, int G, typename SV, typename SW, typename C>
@@ -86,6 +109,8 @@ __device__ __forceinline__ void dot_range_vec(const SV *const *vp, const SW *__r
                                               long long e1, int g, C *acc) {
   constexpr int KV = 16 / sizeof(SV);
   const long long ev = e0 + (e1 - e0) / KV * KV;
+  // four steps of a two-vector product unrolled: a thread has only some eight of them on short vectors
+#pragma unroll (G <= 2 ? 4 : 1)
   for (long long e = e0 + (long long)threadIdx.x * KV; e < ev; e += (long long)BT * KV) {
     // all G + 1 loads of this step issued before any use, so that they are in flight together
     uint4 vraw[G];
@@ -166,10 +191,17 @@ __global__ void __launch_bounds__(BT) multidot_kernel(const SV *__restrict__ V, 
     else
       dot_range<false, G>(vp, wr, e0, e1, g, acc);
   }
+  {
+    double v[2 * G];
 #pragma unroll
-  for (int j = 0; j < G; ++j) {
-    double2 v = warp_sum2(to_d2(acc[j]));
-    if (lane == 0) red[warp][j] = v;
+    for (int j = 0; j < G; ++j) {
+      const double2 a = to_d2(acc[j]);
+      v[2 * j] = a.x;
+      v[2 * j + 1] = a.y;
+    }
+    constexpr int PER = 32 / (2 * G);   // lanes that hold the same sum
+    const double sum = warp_sums<2 * G>(v);
+    if (lane % PER == 0) ((double *)red[warp])[lane / PER] = sum;
   }
   __syncthreads();
   if (threadIdx.x < g) {
@@ -199,21 +231,37 @@ __global__ void __launch_bounds__(BT) multidot_kernel(const SV *__restrict__ V, 
 }
 
 // Single-launch batched norms ||x^r||, same last-block scheme as multidot_kernel.
-template <typename S>
+template <typename S, int KV>
 __global__ void __launch_bounds__(BT) norm_kernel(const S *__restrict__ x, long long n, double fac,
                                                   double *__restrict__ partial, unsigned *__restrict__ counters,
                                                   double *__restrict__ out) {
   const int r = blockIdx.y;
   const int nb = gridDim.x;
-  const long long chunk = (n + nb - 1) / nb;
-  const long long e0 = blockIdx.x * chunk;
+  const long long chunk = ((n + nb - 1) / nb + KV - 1) / KV * KV;
+  const long long e0 = min(n, blockIdx.x * chunk);
   const long long e1 = min(n, e0 + chunk);
   const S *xr = x + r * n;
   decltype(Ar<S>().x) a = 0;
-  for (long long e = e0 + threadIdx.x; e < e1; e += BT) {
-    const Ar<S> v = ldc(xr[e]);
-    a = fma(v.x, v.x, a);
-    a = fma(v.y, v.y, a);
+  if (KV > 1) {   // 16-byte loads: x on a 16-byte boundary, n and the chunk multiples of KV
+#pragma unroll 4
+    for (long long e = e0 + (long long)threadIdx.x * KV; e < e1; e += (long long)BT * KV) {
+      S xv[KV];
+      const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(xr + e));
+      memcpy(xv, &raw, 16);
+#pragma unroll
+      for (int q = 0; q < KV; ++q) {
+        const Ar<S> v = ldc(xv[q]);
+        a = fma(v.x, v.x, a);
+        a = fma(v.y, v.y, a);
+      }
+    }
+  } else {
+#pragma unroll 4
+    for (long long e = e0 + threadIdx.x; e < e1; e += BT) {
+      const Ar<S> v = ldc(xr[e]);
+      a = fma(v.x, v.x, a);
+      a = fma(v.y, v.y, a);
+    }
   }
   double acc = (double)a;
 #pragma unroll
@@ -382,6 +430,80 @@ __global__ void __launch_bounds__(BT) multiaxpy_vec_kernel(const SV *__restrict_
   for (int q = 0; q < KV; ++q) wv[q] = stc<SW>(acc[q]);
   memcpy(&raw, wv, 16);
   *reinterpret_cast<uint4 *>(wp) = raw;
+}
+
+// The same for NV vectors (the Lanczos window) followed by the norm of the stored result, norms[r] = fac
+// ||w^r||, in one pass: block (chunk blockIdx.x, right-hand side blockIdx.y), last-block sums as in
+// norm_kernel.  Loads of two steps are in flight together.
+template <typename SV, typename SW, int NV>
+__global__ void __launch_bounds__(BT) multiaxpy_norm_kernel(const SV *__restrict__ V, long long vstride, long long vrs,
+                                                            const double2 *__restrict__ h, double sign,
+                                                            SW *__restrict__ w, long long n, double fac,
+                                                            double *__restrict__ partial,
+                                                            unsigned *__restrict__ counters, double *__restrict__ out) {
+  using C = Ar<SW>;
+  constexpr int KV = 16 / sizeof(SV);
+  __shared__ double red[BT / 32];
+  __shared__ bool last;
+  const int r = blockIdx.y, nb = gridDim.x;
+  C coef[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) coef[i] = from_d2<C>(cscale(h[(long long)i * gridDim.y + r], sign));
+  const long long chunk = ((n + nb - 1) / nb + KV - 1) / KV * KV;
+  const long long e0 = min(n, blockIdx.x * chunk), e1 = min(n, e0 + chunk);
+  float a = 0.f;
+#pragma unroll 2
+  for (long long e = e0 + (long long)threadIdx.x * KV; e < e1; e += (long long)BT * KV) {
+    const SV *vp = V + r * vrs + e;
+    SW *wp = w + r * n + e;
+    SW wv[KV];
+    uint4 raw = *reinterpret_cast<const uint4 *>(wp), vraw[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) vraw[i] = __ldg(reinterpret_cast<const uint4 *>(vp + i * vstride));
+    memcpy(wv, &raw, 16);
+    C acc[KV];
+#pragma unroll
+    for (int q = 0; q < KV; ++q) acc[q] = ldc(wv[q]);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      SV vv[KV];
+      memcpy(vv, &vraw[i], 16);
+#pragma unroll
+      for (int q = 0; q < KV; ++q) gfma(acc[q], ldc(vv[q]), coef[i]);
+    }
+#pragma unroll
+    for (int q = 0; q < KV; ++q) {
+      wv[q] = stc<SW>(acc[q]);
+      const C o = ldc(wv[q]);   // the norm of what is stored
+      a = fma(o.x, o.x, a);
+      a = fma(o.y, o.y, a);
+    }
+    memcpy(&raw, wv, 16);
+    *reinterpret_cast<uint4 *>(wp) = raw;
+  }
+  double acc = (double)a;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int q = 0; q < BT / 32; ++q) sum += red[q];
+    partial[(long long)r * nb + blockIdx.x] = sum;
+    __threadfence();
+    last = (atomicAdd(&counters[r], 1u) == (unsigned)(nb - 1));
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  double sum = 0.0;
+  for (int q = threadIdx.x; q < nb; q += 32) sum += __ldcg(partial + (long long)r * nb + q);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (threadIdx.x == 0) {
+    out[r] = sqrt(sum) * fac;
+    counters[r] = 0u;
+  }
 }
 
 constexpr int COMB_CT = 8;      // most output columns per pass in combine
@@ -719,18 +841,21 @@ lqcd_status blas_norms(lqcd_ctx *ctx, const S *x, long long n, int nrhs, double 
   LQCD_TRY(ws_get(ctx, WS_SCAL, sizeof(double) * (size_t)nb * nrhs, &p));
   LQCD_TRY(reduction_counters(ctx, nrhs, &cnt));
   kbegin(ctx);
-  norm_kernel<S><<<dim3(nb, nrhs), BT, 0, ctx->stream>>>(x, n, 1.0 / store_sigma<S>(ctx->N), (double *)p, cnt, norms);
+  constexpr int KV = 16 / (int)sizeof(S);
+  const bool vec = (uintptr_t)x % 16 == 0 && (n * (long long)sizeof(S)) % 16 == 0;
+  (vec ? norm_kernel<S, KV> : norm_kernel<S, 1>)<<<dim3(nb, nrhs), BT, 0, ctx->stream>>>(
+      x, n, 1.0 / store_sigma<S>(ctx->N), (double *)p, cnt, norms);
   return launch_check_bytes(ctx, "norm_kernel", K_NORM, (double)n * nrhs, (double)sizeof(S) * n * nrhs);
 }
 
-static int multidot_chunks(lqcd_ctx *ctx, long long n, int nrhs, int nvec, bool shared) {
-  // element chunks of at least 8 elements per thread; enough blocks (chunks x vector groups x
+static int multidot_chunks(lqcd_ctx *ctx, long long n, int nrhs, int nvec, bool shared, int kv = 1) {
+  // element chunks of at least 8 loads (of kv elements) per thread; enough blocks (chunks x vector groups x
   // right-hand sides) for about 16 per SM, several waves of the 4-6 resident ones, so that no SM
   // idles at the end.  With a basis shared by several right-hand
   // sides, also chunks short enough that the blocks in flight (about 8 per SM) touch at most ~32 MB
   // of L2, so that the basis chunk is read from DRAM once for all of them.
   const int ngroup = (nvec + GROUP - 1) / GROUP;
-  const long long max_chunks = std::max<long long>(1, n / (8LL * BT));
+  const long long max_chunks = std::max<long long>(1, n / (8LL * kv * BT));
   long long want = std::max<long long>(1, (16LL * ctx->sms) / std::max<long long>(1, (long long)nrhs * ngroup));
   if (shared && nrhs > 1) {
     const long long per_chunk_blocks = (long long)nrhs * ngroup;
@@ -776,17 +901,17 @@ lqcd_status blas_multidot(lqcd_ctx *ctx, const SV *V, long long vstride, long lo
     const double bytes = (double)sizeof(SV) * n * nvec + (double)sizeof(SW) * n * nrhs;
     return launch_check_bytes(ctx, "multidot_shared_kernel", K_DOT, (double)n * nrhs * nvec, bytes);
   }
-  const int nchunk = multidot_chunks(ctx, n, nrhs, nvec, vrs == 0);
+  // 16-byte loads for the 4- and 8-byte storage types when every vector starts on a 16-byte boundary
+  const bool vec = sizeof(SV) < 16 && sizeof(SV) == sizeof(SW) && ((uintptr_t)V % 16 == 0) &&
+                   ((uintptr_t)w % 16 == 0) && ((vstride * (long long)sizeof(SV)) % 16 == 0) &&
+                   ((vrs * (long long)sizeof(SV)) % 16 == 0) && ((n * (long long)sizeof(SW)) % 16 == 0);
+  const int nchunk = multidot_chunks(ctx, n, nrhs, nvec, vrs == 0, vec ? 16 / (int)sizeof(SV) : 1);
   if ((long long)nchunk * ngroup * nrhs > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "multidot: grid too large");
   void *p = nullptr;
   unsigned *cnt = nullptr;
   LQCD_TRY(ws_get(ctx, WS_PARTIAL, sizeof(double2) * (size_t)nchunk * nrhs * nvec, &p));
   LQCD_TRY(reduction_counters(ctx, nrhs * ngroup, &cnt));
   const double fac = 1.0 / (store_sigma<SV>(ctx->N) * store_sigma<SW>(ctx->N));
-  // 16-byte loads for the 4- and 8-byte storage types when every vector starts on a 16-byte boundary
-  const bool vec = sizeof(SV) < 16 && sizeof(SV) == sizeof(SW) && ((uintptr_t)V % 16 == 0) &&
-                   ((uintptr_t)w % 16 == 0) && ((vstride * (long long)sizeof(SV)) % 16 == 0) &&
-                   ((vrs * (long long)sizeof(SV)) % 16 == 0) && ((n * (long long)sizeof(SW)) % 16 == 0);
   const unsigned grid = (unsigned)((long long)nchunk * ngroup * nrhs);
   kbegin(ctx);
   // at most two vectors (the Lanczos window): the two-vector form, with a quarter of the registers
@@ -829,6 +954,31 @@ lqcd_status blas_multiaxpy(lqcd_ctx *ctx, const SV *V, long long vstride, long l
   // and written once
   const double bytes = (double)sizeof(SV) * n * nvec * (vrs != 0 ? nrhs : 1) + 2.0 * sizeof(SW) * n * nrhs;
   return launch_check_bytes(ctx, "multiaxpy_kernel", K_AXPY, (double)n * nrhs * nvec, bytes);
+}
+
+template <typename S>
+lqcd_status blas_multiaxpy_norms(lqcd_ctx *ctx, const S *V, long long vstride, long long vrs, int nvec, const double2 *h,
+                                 double sign, S *w, long long n, int nrhs, double *norms) {
+  const bool vec = sizeof(S) < 16 && nvec > 0 && nvec <= AXPY_MAXV && nrhs <= 65535 && ((uintptr_t)V % 16 == 0) &&
+                   ((uintptr_t)w % 16 == 0) && ((vstride * (long long)sizeof(S)) % 16 == 0) &&
+                   ((vrs * (long long)sizeof(S)) % 16 == 0) && ((n * (long long)sizeof(S)) % 16 == 0);
+  if constexpr (sizeof(S) < 16) {
+    // one pass for the one or two vectors of a Lanczos window; more vectors hide the norm's extra pass
+    if (vec && nvec <= 2) {
+      const int nb = partial_blocks(ctx, n, nrhs);
+      void *p;
+      unsigned *cnt;
+      LQCD_TRY(ws_get(ctx, WS_SCAL, sizeof(double) * (size_t)nb * nrhs, &p));
+      LQCD_TRY(reduction_counters(ctx, nrhs, &cnt));
+      kbegin(ctx);
+      (nvec == 1 ? multiaxpy_norm_kernel<S, S, 1> : multiaxpy_norm_kernel<S, S, 2>)<<<dim3(nb, nrhs), BT, 0, ctx->stream>>>(
+          V, vstride, vrs, h, sign, w, n, 1.0 / store_sigma<S>(ctx->N), (double *)p, cnt, norms);
+      const double bytes = (double)sizeof(S) * n * nvec * (vrs != 0 ? nrhs : 1) + 2.0 * sizeof(S) * n * nrhs;
+      return launch_check_bytes(ctx, "multiaxpy_norm_kernel", K_AXPY, (double)n * nrhs * nvec, bytes);
+    }
+  }
+  LQCD_TRY(blas_multiaxpy(ctx, V, vstride, vrs, nvec, h, sign, w, n, nrhs));
+  return blas_norms(ctx, (const S *)w, n, nrhs, norms);
 }
 
 template <typename SV, typename SO>
@@ -891,6 +1041,8 @@ lqcd_status blas_to_f32(lqcd_ctx *ctx, const double2 *x, float2 *y, long long n)
   template lqcd_status blas_axpby<S>(lqcd_ctx *, double2, const S *, double2, S *, long long);                  \
   template lqcd_status blas_zero<S>(lqcd_ctx *, S *, long long);                                                \
   template lqcd_status blas_norms<S>(lqcd_ctx *, const S *, long long, int, double *);                          \
+  template lqcd_status blas_multiaxpy_norms<S>(lqcd_ctx *, const S *, long long, long long, int, const double2 *,  \
+                                               double, S *, long long, int, double *);                          \
   template lqcd_status blas_invscale<S>(lqcd_ctx *, S *, const double *, long long, int);
 #define LQCD_BLAS_INSTANTIATE2(SV, SW)                                                                         \
   template lqcd_status blas_multidot<SV, SW>(lqcd_ctx *, const SV *, long long, long long, int, const SW *,     \

@@ -316,6 +316,10 @@ lqcd_status blas_multidot(lqcd_ctx *ctx, const SV *V, long long vstride, long lo
 template <typename SV, typename SW>
 lqcd_status blas_multiaxpy(lqcd_ctx *ctx, const SV *V, long long vstride, long long vrs, int nvec, const double2 *h,
                            double sign, SW *w, long long n, int nrhs);
+// the same, then norms[r] = ||w^r|| (device), in one pass for reduced-precision vectors and few of them
+template <typename S>
+lqcd_status blas_multiaxpy_norms(lqcd_ctx *ctx, const S *V, long long vstride, long long vrs, int nvec, const double2 *h,
+                                 double sign, S *w, long long n, int nrhs, double *norms);
 // out_c^r = out + c*ostride + r*n = sum_i V_i^r C[(i*ncol + c)*nrhs + r] for c < ncol (no aliasing)
 template <typename SV, typename SO>
 lqcd_status blas_combine(lqcd_ctx *ctx, const SV *V, long long vstride, long long vrs, int nvec, const double2 *C,

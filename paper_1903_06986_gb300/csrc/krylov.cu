@@ -314,12 +314,14 @@ lqcd_status arnoldi_enqueue(void *arg) {
     const int lo = gs_first(a, j);
     const S *vlo = a.Vb + lo * vs;
     LQCD_TRY(blas_multidot(ctx, vlo, vs, N, j + 1 - lo, w, N, a.nrhs, h1 + (long long)lo * a.nrhs));
-    LQCD_TRY(blas_multiaxpy(ctx, vlo, vs, N, j + 1 - lo, h1 + (long long)lo * a.nrhs, -1.0, w, N, a.nrhs));
+    const double2 *hl = h1;
     if (a.passes > 1) {
+      LQCD_TRY(blas_multiaxpy(ctx, vlo, vs, N, j + 1 - lo, h1 + (long long)lo * a.nrhs, -1.0, w, N, a.nrhs));
       LQCD_TRY(blas_multidot(ctx, vlo, vs, N, j + 1 - lo, w, N, a.nrhs, h2 + (long long)lo * a.nrhs));
-      LQCD_TRY(blas_multiaxpy(ctx, vlo, vs, N, j + 1 - lo, h2 + (long long)lo * a.nrhs, -1.0, w, N, a.nrhs));
+      hl = h2;
     }
-    LQCD_TRY(blas_norms(ctx, w, N, a.nrhs, a.nrm + (long long)j * a.nrhs));
+    LQCD_TRY(blas_multiaxpy_norms(ctx, vlo, vs, N, j + 1 - lo, hl + (long long)lo * a.nrhs, -1.0, w, N, a.nrhs,
+                                  a.nrm + (long long)j * a.nrhs));
     LQCD_TRY(blas_invscale(ctx, w, a.nrm + (long long)j * a.nrhs, N, a.nrhs));
   }
   return LQCD_OK;
