@@ -343,11 +343,11 @@ lqcd_status noise_launch(lqcd_ctx *ctx, uint64_t seed, uint32_t first, int nrhs,
 lqcd_status check_finite(lqcd_ctx *ctx, const double *x, long long n, const char *what);
 // Tensor-core split-precision contractions with k vectors E (tcdefl.cu): slices of E made once
 // (tc_slices_make, released by tc_slices_free), then G[q * nrhs + r] = <E_q, X_r> (tc_vhx) and
-// Y_r = sum_q E_q d_q C[q * nrhs + r] (tc_vc; d device k complex or NULL); all device pointers.
+// Y_r = [gamma_5] sum_q E_q d_q C[q * nrhs + r] (tc_vc; d device k complex or NULL); all device pointers.
 lqcd_status tc_slices_make(lqcd_ctx *ctx, const double2 *E, int k, void **out);
 void tc_slices_free(void *slices);
 lqcd_status tc_vhx(lqcd_ctx *ctx, const void *slices, const double2 *X, int nrhs, double2 *G);
-lqcd_status tc_vc(lqcd_ctx *ctx, const void *slices, const double2 *C, const double2 *d, int nrhs, double2 *Y);
+lqcd_status tc_vc(lqcd_ctx *ctx, const void *slices, const double2 *C, const double2 *d, int nrhs, double2 *Y, bool g5);
 // Y = E C for a basis used once (E: k fields, C: k x ncol device): only this product's slices, in
 // context workspace
 lqcd_status tc_vc_oneshot(lqcd_ctx *ctx, const double2 *E, int k, const double2 *C, int ncol, double2 *Y);

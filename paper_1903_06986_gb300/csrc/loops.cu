@@ -793,7 +793,6 @@ static lqcd_status deflate_dev(lqcd_ctx *ctx, const lqcd_defl *defl, const doubl
   const long long N = ctx->N;
   double2 *coef, *tmp;
   LQCD_TRY(ws_get(ctx, WS_EST1, sizeof(double2) * (size_t)k * nrhs, (void **)&coef));
-  LQCD_TRY(ws_get(ctx, WS_TMP4, sizeof(double2) * (size_t)nrhs * N, (void **)&tmp));
   if (ctx->defl_engine == LQCD_DEFL_TENSOR) {
     // split-precision tensor-core products; the slices of E are cached in the deflation object
     lqcd_defl *dm = const_cast<lqcd_defl *>(defl);
@@ -804,9 +803,9 @@ static lqcd_status deflate_dev(lqcd_ctx *ctx, const lqcd_defl *defl, const doubl
     for (int q = 0; q < k; ++q) dh[q] = make_double2(d[q].real(), d[q].imag());
     LQCD_TRY(upload_v(ctx, dh.data(), dd, sizeof(double2) * (size_t)k));
     LQCD_TRY(tc_vhx(ctx, dm->tc, eta, nrhs, coef));
-    LQCD_TRY(tc_vc(ctx, dm->tc, coef, dd, nrhs, tmp));
-    return blas_g5(ctx, tmp, out, nrhs);
+    return tc_vc(ctx, dm->tc, coef, dd, nrhs, out, true);
   }
+  LQCD_TRY(ws_get(ctx, WS_TMP4, sizeof(double2) * (size_t)nrhs * N, (void **)&tmp));
   LQCD_TRY(blas_multidot(ctx, defl->E, N, 0, k, eta, N, nrhs, coef));
   std::vector<double2> c;
   LQCD_TRY(download_v(ctx, coef, c, (size_t)k * nrhs));
