@@ -157,13 +157,12 @@ struct Acc {
 
 __device__ __forceinline__ void add2(long long a[2], long long re, long long im) { a[0] += re; a[1] += im; }
 
-// Adds direction d (2 mu: x + mu, 2 mu + 1: x - mu) to A: q: the field's integers at the neighbour, of
-// which the half spinor is shifted by sh; u: the link of direction mu; pu, pl: component offsets of
-// the upper and lower spin pair (exchanged: -gamma_5 times the field).  d is a run-time value, the
-// same in all threads: the loop over the directions stays rolled, since eight unrolled copies (100 kB
-// of instructions) missed the instruction cache on one issue in six.
-__device__ __forceinline__ void direction(int d, const longlong2 *__restrict__ q, int pu, int pl, int sh,
-                                          const int4 *__restrict__ u, Acc &A) {
+// Colour product of one direction d (2 mu: U h of (1 - g) p, 2 mu + 1: U^dag h of (1 + g) p) for the two
+// components of a half spinor: q: the field's integers at p, of which the half spinor is shifted by sh; u: the
+// links of the site that holds the link; pu, pl: component offsets of the upper and lower spin pair
+// (exchanged: -gamma_5 times the field).  With sh = E - X_u - X - 1 the unit of o is 2^(E - 2101).
+__device__ __forceinline__ void half_product(int d, const longlong2 *__restrict__ q, int pu, int pl, int sh,
+                                             const int4 *__restrict__ u, long long o[2][3][2]) {
   const int mu = d >> 1, bwd = d & 1;
   // half spinor (table at the head of spin.cuh), shifted and split; the t projection is 2 p of one pair
   longlong2 h[2][3];
@@ -212,7 +211,6 @@ __device__ __forceinline__ void direction(int d, const longlong2 *__restrict__ q
       split(sar64(h[k][c].y, sh), hi[k][c][1], lo[k][c][1]);
     }
   // o_a = sum_b U_ab h_b (forward) or conj(U_ba) h_b (backward)
-  long long o[2][3][2];
   const int4 *um = u + mu * 288;
   const int ea = bwd ? 32 : 96, eb = bwd ? 96 : 32, cs = bwd ? -1 : 1;
 #pragma unroll
@@ -253,6 +251,15 @@ __device__ __forceinline__ void direction(int d, const longlong2 *__restrict__ q
 #pragma unroll
       for (int z = 0; z < 2; ++z) o[k][a][z] = madw(hh[k][z], (int)(md[k][z] >> 32), 1);
   }
+}
+
+// Adds direction d (x + mu, x - mu) to A; arguments as half_product.  d is a run-time value, the same in all
+// threads: the loop over the directions stays rolled, since eight unrolled copies (100 kB of
+// instructions) missed the instruction cache on one issue in six.
+__device__ __forceinline__ void direction(int d, const longlong2 *__restrict__ q, int pu, int pl, int sh,
+                                          const int4 *__restrict__ u, Acc &A) {
+  long long o[2][3][2];
+  half_product(d, q, pu, pl, sh, u, o);
   if (d != 6) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {

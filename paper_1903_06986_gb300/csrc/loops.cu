@@ -14,6 +14,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda.h>  // driver types of the context-id query (entry points come from the runtime)
 
@@ -108,16 +109,59 @@ __device__ __forceinline__ Cx<double> psplit(const double2 *U, const double2 *et
   return MU == 3 ? d + d : d;
 }
 
+// The same with the colour products U (1 - g) w and U^dag (1 + g) w on the integer pipes (fxhop.cuh; q, ex:
+// the integers of w at this right-hand side), which leaves the projections of eta and the products with
+// it in FP64: 96 operations of the 240 of both terms.
+template <int MU>
+__device__ __forceinline__ Cx<double> psplit_fx(const longlong2 *q, const int *ex, const fx::Links &L, const double2 *U,
+                                                const double2 *eta, const double2 *w, int s, int sp, long long V,
+                                                const Cx<double> eta_s[4][3]) {
+  const int Xu = __ldg(L.ex + MU * V + s), X1 = Xu + __ldg(ex + s) + 2, X2 = Xu + __ldg(ex + sp) + 2;
+  if (max(X1, X2) > 2900) {   // an entry outside the integers' range
+    Cx<double> ws[4][3];
+    load_spinor<double, false>(w + 12LL * s, ws);
+    return psplit<MU>(U, eta, w, s, sp, V, eta_s, ws);
+  }
+  // both exponents are above 1100 unless a block is zero
+  const double k1 = X1 > 1080 ? __hiloint2double((X1 - 2101 + 1023) << 20, 0) : 0.0;
+  const double k2 = X2 > 1080 ? __hiloint2double((X2 - 2101 + 1023) << 20, 0) : 0.0;
+  const int4 *u = L.q + fx::slot(s, 36);
+  long long o[2][3][2];
+  Cx<double> nb[4][3], h[3], r[3], d1 = mk<double>(0.0, 0.0), d2 = d1;
+  load_spinor<double, false>(eta + 12LL * sp, nb);
+  fx::half_product(2 * MU + 1, q + fx::slot(s, 12), 0, 192, 1, u, o);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
+    half_spinor<MU, 1>(nb, k, h);
+    dot3(h, r, d1);
+  }
+  fx::half_product(2 * MU, q + fx::slot(sp, 12), 0, 192, 1, u, o);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
+    half_spinor<MU, -1>(eta_s, k, h);
+    dot3(h, r, d2);
+  }
+  // the integers of the t direction carry the projector's factor 2
+  return mk<double>(k1 * d1.x - k2 * d2.x, k1 * d1.y - k2 * d2.y);
+}
+
 // partial[((r * Lt + t) * nchunk + chunk) * 9 + op]; grid (nchunk * Lt, nrhs).
 // Bound by FP64 issue (two operations per clock and SM): 152 operations of the local densities, 924 of
 // the point-split ones and 90 of the compensated sums per site and right-hand side.  The local densities
 // share spin products: P, Q the products of the upper and lower pairs (scalar P + Q, gamma_4 P - Q) and
 // X, Y, Z as below.  Ten fields of 24^3 x 32: 17.8 ms with four-spin products and one chunk per timeslice,
-// 9.66 ms now, 8.8 ms of it FP64 issue.
+// 9.66 ms in this FP64 form, 6.19 ms with FX (conversion of w and links included).
+// FX: the point-split colour products from the integers f of w (600 FP64 operations remain); without, all
+// in FP64 for lqcd_contract_noalloc and where there is no memory for the integers.
+template <bool FX>
 __global__ void __launch_bounds__(CBT) contract_kernel(const double2 *__restrict__ U, double kappa,
                                                        const double2 *__restrict__ eta, const double2 *__restrict__ w,
                                                        int Lx, int Ly, int Lz, int Lt, int nchunk,
-                                                       double2 *__restrict__ partial) {
+                                                       double2 *__restrict__ partial, fx::Links L, fx::Field f) {
   const int r = blockIdx.y;
   const int t = blockIdx.x / nchunk;
   const int chunk = blockIdx.x % nchunk;
@@ -152,10 +196,19 @@ __global__ void __launch_bounds__(CBT) contract_kernel(const double2 *__restrict
     const int yp = (y + 1 == Ly) ? s - (Ly - 1) * Lx : s + Lx;
     const int zp = (z + 1 == Lz) ? s - (Lz - 1) * Lx * Ly : s + Lx * Ly;
     const int tp = (t + 1 == Lt) ? s - (Lt - 1) * Vs : s + Vs;
-    d = psplit<0>(U, er, wr, s, xp, V, es, ws); acc[10].add(kappa * d.x); acc[11].add(kappa * d.y);
-    d = psplit<1>(U, er, wr, s, yp, V, es, ws); acc[12].add(kappa * d.x); acc[13].add(kappa * d.y);
-    d = psplit<2>(U, er, wr, s, zp, V, es, ws); acc[14].add(kappa * d.x); acc[15].add(kappa * d.y);
-    d = psplit<3>(U, er, wr, s, tp, V, es, ws); acc[16].add(kappa * d.x); acc[17].add(kappa * d.y);
+    auto split_term = [&](auto mu, int sp) {
+      constexpr int MU = decltype(mu)::value;
+      if constexpr (FX)
+        d = psplit_fx<MU>(f.q + (long long)r * fx::blocks32(V) * 384, f.ex + (long long)r * V, L, U, er, wr, s, sp, V, es);
+      else
+        d = psplit<MU>(U, er, wr, s, sp, V, es, ws);
+      acc[10 + 2 * MU].add(kappa * d.x);
+      acc[11 + 2 * MU].add(kappa * d.y);
+    };
+    split_term(std::integral_constant<int, 0>{}, xp);
+    split_term(std::integral_constant<int, 1>{}, yp);
+    split_term(std::integral_constant<int, 2>{}, zp);
+    split_term(std::integral_constant<int, 3>{}, tp);
   }
   __shared__ double red[CBT / 32][18];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -727,12 +780,24 @@ lqcd_status contract_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const
   const int nchunk = contract_chunks(Vs, nrhs * Lt, ctx->sms);
   void *p;
   LQCD_TRY(ws_get(ctx, WS_EST2, sizeof(double2) * (size_t)nrhs * Lt * nchunk * 9, &p));
-  kbegin(ctx);
-  contract_kernel<<<dim3(nchunk * Lt, nrhs), CBT, 0, ctx->stream>>>(U, kappa, eta, w, d[0], d[1], d[2], d[3], nchunk,
-                                                                   (double2 *)p);
-  // compulsory bytes: eta and w once, the links once (point-split operators)
-  LQCD_TRY(launch_check_bytes(ctx, "contract_kernel", K_CONTRACT, (double)ctx->V * nrhs,
-                              2.0 * nrhs * ctx->N * sizeof(double2) + 36.0 * ctx->V * sizeof(double2)));
+  fx::Links L{};
+  fx::Field f{};
+  bool use;
+  int chunk = nrhs;
+  LQCD_TRY(fx_links(ctx, U, &L, &use));
+  if (use) LQCD_TRY(fx_field(ctx, ctx->V, nrhs, &f, &chunk, &use));
+  for (int r0 = 0; r0 < nrhs; r0 += chunk) {
+    const int nr = std::min(chunk, nrhs - r0);
+    const double2 *e0 = eta + (long long)r0 * ctx->N, *w0 = w + (long long)r0 * ctx->N;
+    if (use) LQCD_TRY(fx_convert(ctx, w0, f, ctx->V, nr));
+    kbegin(ctx);
+    (use ? contract_kernel<true> : contract_kernel<false>)<<<dim3(nchunk * Lt, nr), CBT, 0, ctx->stream>>>(
+        U, kappa, e0, w0, d[0], d[1], d[2], d[3], nchunk, (double2 *)p + (size_t)r0 * Lt * nchunk * 9, L, f);
+    // compulsory bytes: eta and w once, the links once (point-split operators)
+    LQCD_TRY(launch_check_bytes(ctx, "contract_kernel", K_CONTRACT, (double)ctx->V * nr,
+                                2.0 * nr * ctx->N * sizeof(double2) + 36.0 * ctx->V * sizeof(double2)));
+  }
+  if (use && ctx->fx_depth == 0) fx_done(ctx);
   const int tot = nrhs * 9 * Lt;
   kbegin(ctx);
   contract_final<<<ceil_div(tot, 128), 128, 0, ctx->stream>>>((const double2 *)p, nchunk, Lt, nrhs, out_dev);
@@ -1990,9 +2055,9 @@ extern "C" lqcd_status lqcd_contract_noalloc(const int dims[4], const double *li
   const int nchunk = (int)std::max<long long>(1, std::min<long long>(contract_chunks(Vs, nrhs * Lt, sms), fit));
   cudaStream_t st = (cudaStream_t)stream;
   // the kernel writes every partial entry it later reads, so the array needs no clearing
-  contract_kernel<<<dim3(nchunk * Lt, nrhs), CBT, 0, st>>>((const double2 *)links, kappa, (const double2 *)eta,
-                                                           (const double2 *)w, dims[0], dims[1], dims[2], dims[3],
-                                                           nchunk, scratch);
+  contract_kernel<false><<<dim3(nchunk * Lt, nrhs), CBT, 0, st>>>((const double2 *)links, kappa, (const double2 *)eta,
+                                                                  (const double2 *)w, dims[0], dims[1], dims[2],
+                                                                  dims[3], nchunk, scratch, fx::Links{}, fx::Field{});
   if (cudaGetLastError() != cudaSuccess) return LQCD_ERR_CUDA;
   const int tot = nrhs * 9 * Lt;
   contract_final<<<ceil_div(tot, 128), 128, 0, st>>>(scratch, nchunk, Lt, nrhs, (double2 *)out);
