@@ -236,6 +236,7 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
     delete c;
     return LQCD_ERR_CUDA;
   }
+  fx_reserve_small(c);
   *out = c;
   return LQCD_OK;
 }

@@ -346,6 +346,7 @@ extern "C" lqcd_status lqcd_ctx_create_evenodd(lqcd_ctx **out, const int dims[4]
   c->V = (int)V;
   c->N = 12 * V;
   c->eo = 1;
+  fx_reserve_small(c);
   *out = c;
   return LQCD_OK;
 }

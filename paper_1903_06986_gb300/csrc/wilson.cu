@@ -1,5 +1,8 @@
 // Wilson-Dirac operator M = 1 - kappa P (Eq. xyz556) on blocks of right-hand sides.
 //
+// FP64 fields run in block fixed point on the integer pipes (fxhop.cuh, kernels wilson_fx_kernel and its
+// conversions below); the stencil stated here in floating point serves FP32 arithmetic, and FP64 where
+// no workspace may be taken.
 // One thread owns one (site, right-hand side) pair and produces its 12 output components.  Each
 // of the eight hopping terms is computed in the two-component ("half spinor") form: the spin
 // projector (1 -+ gamma_mu) has rank two in the Dirac basis, so the neighbour spinor is projected
@@ -315,6 +318,19 @@ lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *ch
   f->q = (longlong2 *)p;
   f->ex = (int *)(p + *chunk * qper);
   return st;
+}
+
+void fx_reserve_small(lqcd_ctx *ctx) {
+  // the first FP64 application on a small lattice would otherwise spend more on its two allocations
+  // (about 70 us each) than on the operator; large ones allocate on first use
+  const long long VL = ctx->eo ? 2LL * ctx->V : ctx->V;
+  const long long links = fx::blocks32(VL) * 32 * 36 * (long long)sizeof(int4) + 4 * VL * (long long)sizeof(int);
+  const long long field = fx::blocks32(ctx->V) * 32 * 12 * (long long)sizeof(longlong2) + ctx->V * (long long)sizeof(int);
+  const long long n = std::min<long long>(16, ((64ll << 20) - links) / field);
+  if (n < 1) return;
+  void *p;
+  if (ws_get(ctx, WS_FX_LINKS, (size_t)links, &p) != LQCD_OK || ws_get(ctx, WS_FX_FIELD, (size_t)(n * field), &p) != LQCD_OK)
+    ctx->err.clear();   // without: the first use tries again
 }
 
 lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs) {
