@@ -70,8 +70,8 @@ __device__ __forceinline__ double2 warp_sum2(double2 v) {
 // Sums of N doubles per lane over the warp (N = 4 or 16): the halves of the values go to the halves of the
 // lanes, so that N - 1 + log2(32 / N) additions do instead of 5 N; returns sum number
 // (lane >> (5 - log2 N)), valid in every lane.  FP64 additions cost 16 clocks per warp and SM, and the
-// 5 N form was most of a two-vector product on short vectors (45 us for eight right-hand sides of
-// 12^3 x 24 in FP16, with the launch shape of multidot_chunks 12).
+// 5 N form in 16 blocks per SM was most of a two-vector product on short vectors: 45 us for eight
+// right-hand sides of 12^3 x 24 in FP16, 17 us with this and the chunks of multidot_chunks.
 template <int N>
 __device__ __forceinline__ double warp_sums(double *v) {
   const int lane = threadIdx.x & 31;
@@ -997,7 +997,7 @@ lqcd_status blas_combine(lqcd_ctx *ctx, const SV *V, long long vstride, long lon
         V, vstride, vrs, nvec, C, ncol, fac, out, ostride, n, nrhs);
   } else {
     // one column (the residual of a GMRES-Proj cycle, the HFES product) does not pay for eight: 7.8 ms with
-    // the wide form, 1.9 ms with one column, for 31 vectors of 50 right-hand sides of 8^3 x 16
+    // the wide form, 1.0 ms with one column, for 31 vectors of 50 right-hand sides of 8^3 x 16
     (ncol == 1 ? combine_kernel<SV, SO, 1> : combine_kernel<SV, SO, COMB_CT>)
         <<<(unsigned)((long long)ceil_div(n, BT) * nrhs), BT, 0, ctx->stream>>>(V, vstride, vrs, nvec, C, ncol, fac,
                                                                                out, ostride, n, nrhs);

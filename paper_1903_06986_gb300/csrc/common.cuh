@@ -157,7 +157,8 @@ lqcd_status host_stage(lqcd_ctx *ctx, size_t bytes, double **ptr);
 // not change; nothing is kept beyond it).  use = false: the caller runs the plain FP64 stencil, which
 // needs no workspace (a stream under the caller's capture, or no memory for the workspace).
 namespace fx { struct Links; struct Field; }
-lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use);
+// pending (optional): set instead of launching the conversion, which the caller then launches with its own.
+lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use, bool *pending = nullptr);
 // workspace for up to chunk fields of S sites in that form (use as above), and the conversion into it
 lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *chunk, bool *use);
 lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs);

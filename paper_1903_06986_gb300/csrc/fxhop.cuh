@@ -469,8 +469,9 @@ __device__ __forceinline__ void run(char *smem, const double2 *U, const Links &L
   }
 }
 
-// Blocks of 128 threads for n sites per right-hand side; the split form up to 8 warps per SM of the plain
-// one, measured on 8^3 x 16 with 1 and 4 right-hand sides (256 and 1024 warps of 152 SMs)
+// Whether n sites of nrhs right-hand sides take the split form: up to 8 warps per SM of the plain one.  Measured
+// on 8^3 x 16 (256 warps a right-hand side, 152 SMs): 12.5 against 21.2 us for one, 24.6 against 27.6 for
+// four; eight (37.9 us) are past the line and gain nothing.
 inline bool use_split(long long n, int nrhs, int sms) { return blocks32(n) * nrhs <= 8LL * sms; }
 
 }  // namespace fx
