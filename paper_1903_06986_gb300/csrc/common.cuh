@@ -180,6 +180,10 @@ lqcd_status fx_multiaxpy(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, co
 // arrival counters of the single-launch reductions (zeroed once, left at zero)
 lqcd_status reduction_counters(lqcd_ctx *ctx, int n, unsigned **c);
 void fx_done(lqcd_ctx *ctx);   // records the end of a use (outside scopes; a scope does it at its end)
+// gives the integers of a Krylov basis (WS_FX_BASIS) back; not while a cycle uses them
+void fx_release_basis(lqcd_ctx *ctx);
+// kept from one call to the next up to this size (a larger one is given back at the end of the call)
+constexpr size_t FX_BASIS_KEEP = (size_t)4 << 30;
 struct FxScope {
   lqcd_ctx *ctx;
   explicit FxScope(lqcd_ctx *c) : ctx(c) {
@@ -189,6 +193,7 @@ struct FxScope {
     if (--ctx->fx_depth == 0) {
       if (ctx->fx_src) fx_done(ctx);
       ctx->fx_src = nullptr;
+      if (ctx->ws_size[WS_FX_BASIS] > FX_BASIS_KEEP) fx_release_basis(ctx);
     }
   }
   FxScope(const FxScope &) = delete;

@@ -90,6 +90,12 @@ lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
     }
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && slot != WS_FX_BASIS && ctx->ws_ptr[WS_FX_BASIS]) {
+      // the integers of a Krylov basis are only the faster form: they make room for what a call needs
+      cudaGetLastError();
+      fx_release_basis(ctx);
+      e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       return set_err(ctx, LQCD_ERR_OOM, "workspace slot %d: cudaMalloc(%zu) failed: %s", slot, bytes, cudaGetErrorString(e));
@@ -99,6 +105,15 @@ lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
   }
   *ptr = ctx->ws_ptr[slot];
   return LQCD_OK;
+}
+
+void fx_release_basis(lqcd_ctx *ctx) {
+  if (!ctx->ws_ptr[WS_FX_BASIS]) return;
+  graph_cache_clear(ctx);   // captured cycles hold its address
+  cudaStreamSynchronize(ctx->stream);
+  cudaFree(ctx->ws_ptr[WS_FX_BASIS]);
+  ctx->ws_ptr[WS_FX_BASIS] = nullptr;
+  ctx->ws_size[WS_FX_BASIS] = 0;
 }
 
 void graph_cache_clear(lqcd_ctx *ctx) {

@@ -285,6 +285,8 @@ inline lqcd_status arnoldi_fx(Arnoldi &a) {
     LQCD_CUDA(ctx, cudaMemGetInfo(&fr, &total));
     if (bytes > (fr + ctx->ws_size[WS_FX_BASIS]) / 3) return LQCD_OK;
   }
+  // last of the cycle's workspaces, so that none of the others takes its memory back (ws_get)
+  LQCD_TRY(fx_blas_reserve(ctx, V, a.nrhs, a.m));
   char *p;
   const lqcd_status st = ws_get(ctx, WS_FX_BASIS, bytes, (void **)&p);
   if (st == LQCD_ERR_OOM) {
@@ -294,7 +296,7 @@ inline lqcd_status arnoldi_fx(Arnoldi &a) {
   LQCD_TRY(st);
   a.fx.q = (longlong2 *)p;
   a.fx.ex = (int *)(p + qb);
-  return fx_blas_reserve(ctx, V, a.nrhs, a.m);
+  return LQCD_OK;
 }
 
 template <typename S>
@@ -745,6 +747,8 @@ lqcd_status gmresdr_core(lqcd_ctx *ctx, const Op &op, const double2 *b, double2 
       d->N = N;
       d->V = d->E = nullptr;
       d->Hbar_dev = nullptr;
+      // the cycles are over: a large integer basis makes room for the space
+      if (ctx->ws_size[WS_FX_BASIS] > FX_BASIS_KEEP) fx_release_basis(ctx);
       cudaError_t e1 = cudaMalloc(&d->V, sizeof(double2) * (size_t)(k + 1) * N);
       cudaError_t e2 = cudaMalloc(&d->E, sizeof(double2) * (size_t)k * N);
       cudaError_t e3 = cudaMalloc(&d->Hbar_dev, sizeof(double2) * (size_t)(k + 1) * k);
