@@ -117,36 +117,39 @@ __device__ __forceinline__ Cx<double> psplit_fx(const longlong2 *q, const int *e
                                                 const double2 *eta, const double2 *w, int s, int sp, long long V,
                                                 const Cx<double> eta_s[4][3]) {
   const int Xu = __ldg(L.ex + MU * V + s), X1 = Xu + __ldg(ex + s) + 2, X2 = Xu + __ldg(ex + sp) + 2;
-  if (max(X1, X2) > 2900) {   // an entry outside the integers' range
-    Cx<double> ws[4][3];
-    load_spinor<double, false>(w + 12LL * s, ws);
-    return psplit<MU>(U, eta, w, s, sp, V, eta_s, ws);
+  if (max(X1, X2) <= 2900) {   // every entry in the integers' range
+    // both exponents are above 1100 unless a block is zero
+    const double k1 = X1 > 1080 ? __hiloint2double((X1 - 2101 + 1023) << 20, 0) : 0.0;
+    const double k2 = X2 > 1080 ? __hiloint2double((X2 - 2101 + 1023) << 20, 0) : 0.0;
+    const int4 *u = L.q + fx::slot(s, 36);
+    long long o[2][3][2];
+    Cx<double> nb[4][3], h[3], r[3], d1 = mk<double>(0.0, 0.0), d2 = d1;
+    load_spinor<double, false>(eta + 12LL * sp, nb);
+    fx::half_product(2 * MU + 1, q + fx::slot(s, 12), 0, 192, 1, u, o);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
+      half_spinor<MU, 1>(nb, k, h);
+      dot3(h, r, d1);
+    }
+    fx::half_product(2 * MU, q + fx::slot(sp, 12), 0, 192, 1, u, o);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
+      half_spinor<MU, -1>(eta_s, k, h);
+      dot3(h, r, d2);
+    }
+    // the integers of the t direction carry the projector's factor 2
+    const Cx<double> d = mk<double>(k1 * d1.x - k2 * d2.x, k1 * d1.y - k2 * d2.y);
+    // eta above 2^960 leaves the range of FP64 times the integers (up to 2^62), which k1 and k2 take out
+    // only here: an Inf or NaN in d1 or d2 stays one
+    if (isfinite(d.x) && isfinite(d.y)) return d;
   }
-  // both exponents are above 1100 unless a block is zero
-  const double k1 = X1 > 1080 ? __hiloint2double((X1 - 2101 + 1023) << 20, 0) : 0.0;
-  const double k2 = X2 > 1080 ? __hiloint2double((X2 - 2101 + 1023) << 20, 0) : 0.0;
-  const int4 *u = L.q + fx::slot(s, 36);
-  long long o[2][3][2];
-  Cx<double> nb[4][3], h[3], r[3], d1 = mk<double>(0.0, 0.0), d2 = d1;
-  load_spinor<double, false>(eta + 12LL * sp, nb);
-  fx::half_product(2 * MU + 1, q + fx::slot(s, 12), 0, 192, 1, u, o);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
-    half_spinor<MU, 1>(nb, k, h);
-    dot3(h, r, d1);
-  }
-  fx::half_product(2 * MU, q + fx::slot(sp, 12), 0, 192, 1, u, o);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) r[c] = mk<double>((double)o[k][c][0], (double)o[k][c][1]);
-    half_spinor<MU, -1>(eta_s, k, h);
-    dot3(h, r, d2);
-  }
-  // the integers of the t direction carry the projector's factor 2
-  return mk<double>(k1 * d1.x - k2 * d2.x, k1 * d1.y - k2 * d2.y);
+  Cx<double> ws[4][3];
+  load_spinor<double, false>(w + 12LL * s, ws);
+  return psplit<MU>(U, eta, w, s, sp, V, eta_s, ws);
 }
 
 // partial[((r * Lt + t) * nchunk + chunk) * 9 + op]; grid (nchunk * Lt, nrhs).
@@ -154,7 +157,7 @@ __device__ __forceinline__ Cx<double> psplit_fx(const longlong2 *q, const int *e
 // the point-split ones and 90 of the compensated sums per site and right-hand side.  The local densities
 // share spin products: P, Q the products of the upper and lower pairs (scalar P + Q, gamma_4 P - Q) and
 // X, Y, Z as below.  Ten fields of 24^3 x 32: 17.8 ms with four-spin products and one chunk per timeslice,
-// 9.66 ms in this FP64 form, 6.19 ms with FX (conversion of w and links included).
+// 9.66 ms in this FP64 form, 6.25 ms with FX (conversion of w and links included).
 // FX: the point-split colour products from the integers f of w (600 FP64 operations remain); without, all
 // in FP64 for lqcd_contract_noalloc and where there is no memory for the integers.
 template <bool FX>
