@@ -21,6 +21,7 @@
 //            1 + g = diag(2,2,0,0): only the upper pair, (2 p0, 2 p1)
 // gamma_5 = -[[0, 1], [1, 0]] in this basis: (g5 p) = (-p2, -p3, -p0, -p1).
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fxhop.cuh"
@@ -726,12 +727,12 @@ __device__ __forceinline__ __nv_bfloat162 b_fromf(float2 a) { return __float22bf
 template <> struct PairIO<__half2> : PairIOHalf<__half2, h2x2, h_lo, h_hi, h_tof, h_fromf> {};
 template <> struct PairIO<__nv_bfloat162> : PairIOHalf<__nv_bfloat162, b2x2, b_lo, b_hi, b_tof, b_fromf> {};
 
-// Blocks of 64 threads fill the last wave better than 128 (12^3 x 24, 8 right-hand sides: 22.5 us with 128);
-// FP16 / BF16 fields with rebuilt links take 168 registers (20.5 us, and 227 against 234 us for 10
-// right-hand sides of 24^3 x 32), the others 128 (FP32: 250 against 256 us).
+// Blocks of 64 threads fill the last wave better than 128 (12^3 x 24, 8 right-hand sides: 22.5 us with 128).
+// RES: resident blocks per SM the registers are limited for: 8 (128 registers), or 6 (168) for FP16 / BF16
+// fields with rebuilt links where pair_launch takes it.
 constexpr int PAIR_BT = 64;
-template <typename S, int RECON, int MODE>
-__global__ void __launch_bounds__(PAIR_BT, sizeof(typename Chunk<S>::T) == 8 && RECON == 12 ? 6 : 8) wilson_pair_kernel(const float4 *__restrict__ U,
+template <typename S, int RECON, int MODE, int RES>
+__global__ void __launch_bounds__(PAIR_BT, RES) wilson_pair_kernel(const float4 *__restrict__ U,
                                                           const typename Chunk<S>::T *__restrict__ in,
                                                           typename Chunk<S>::T *__restrict__ out, float kappa,
                                                           int Lx, int Ly, int Lz, int Lt, int V, int nrhs,
@@ -1089,6 +1090,28 @@ __global__ void pack_links_kernel(const double2 *__restrict__ U, float4 *__restr
   }
 }
 
+template <typename S, int RECON, int MODE>
+void pair_launch_mode(lqcd_ctx *ctx, const float4 *U, float k, const typename Chunk<S>::T *in, typename Chunk<S>::T *out,
+                      int nrhs, int groups, int bs, unsigned grid) {
+  const int *d = ctx->dims;
+  if constexpr (sizeof(typename Chunk<S>::T) == 8 && RECON == 12) {
+    // FP16 / BF16 with rebuilt links: 168 registers up to two waves of the blocks that then fit (3 to 18 % less
+    // time: 8^3 x 16, 2 fields 4.13 against 4.64 us; 12^3 x 24, 3 fields 11.96 against 12.31).  On more sites the
+    // 128-register form with its 8 blocks gains 2 to 4 % (16^3 x 32, 10 FP16 fields, M: 68.6 against 71.5 us; 24^3 x
+    // 32: 224 against 229), except for M gamma_5 and P on FP16 (24^3 x 32: 224 against 230, 210 against 214 us) and
+    // M on BF16 (225 against 232).
+    constexpr bool f16 = std::is_same<S, __half2>::value;
+    constexpr bool always = f16 ? MODE == 1 || MODE == 3 : MODE == 0;
+    if (always || (long long)grid * bs <= 2LL * 6 * PAIR_BT * ctx->sms) {
+      wilson_pair_kernel<S, RECON, MODE, 6><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V,
+                                                                       nrhs, groups);
+      return;
+    }
+  }
+  wilson_pair_kernel<S, RECON, MODE, 8><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V, nrhs,
+                                                                   groups);
+}
+
 template <typename S, int RECON>
 lqcd_status pair_launch(lqcd_ctx *ctx, const float4 *U, double kappa, const void *in_, void *out_, int nrhs, int flags) {
   using T = typename Chunk<S>::T;
@@ -1099,15 +1122,14 @@ lqcd_status pair_launch(lqcd_ctx *ctx, const float4 *U, double kappa, const void
   while (bs > 32 && (long long)ceil_div(ctx->V, bs) * groups < 2LL * ctx->sms) bs /= 2;
   const long long nblk = (long long)ceil_div(ctx->V, bs) * groups;
   if (nblk > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "packed wilson: grid too large");
-  dim3 grid((unsigned)nblk);
-  const int *d = ctx->dims;
+  const unsigned grid = (unsigned)nblk;
   const float k = (float)kappa;
   kbegin(ctx);
   switch (flags) {
-    case LQCD_APPLY_M: wilson_pair_kernel<S, RECON, 0><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V, nrhs, groups); break;
-    case LQCD_APPLY_G5R: wilson_pair_kernel<S, RECON, 1><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V, nrhs, groups); break;
-    case LQCD_APPLY_DAG: wilson_pair_kernel<S, RECON, 2><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V, nrhs, groups); break;
-    case LQCD_APPLY_HOP: wilson_pair_kernel<S, RECON, 3><<<grid, bs, 0, ctx->stream>>>(U, in, out, k, d[0], d[1], d[2], d[3], ctx->V, nrhs, groups); break;
+    case LQCD_APPLY_M: pair_launch_mode<S, RECON, 0>(ctx, U, k, in, out, nrhs, groups, bs, grid); break;
+    case LQCD_APPLY_G5R: pair_launch_mode<S, RECON, 1>(ctx, U, k, in, out, nrhs, groups, bs, grid); break;
+    case LQCD_APPLY_DAG: pair_launch_mode<S, RECON, 2>(ctx, U, k, in, out, nrhs, groups, bs, grid); break;
+    case LQCD_APPLY_HOP: pair_launch_mode<S, RECON, 3>(ctx, U, k, in, out, nrhs, groups, bs, grid); break;
     default: return set_err(ctx, LQCD_ERR_INVALID_ARG, "packed wilson: unknown flags %d", flags);
   }
   const double bytes = 2.0 * nrhs * ctx->V * 6 * sizeof(T) + 4.0 * ctx->V * (RECON == 12 ? 3 : 5) * 16;

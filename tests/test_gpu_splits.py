@@ -73,3 +73,20 @@ def test_hop_traces_by_site_against_the_oracle():
     ctx = context(dims)
     U = synth.su3_links(dims, 0.5, 12)
     assert rel_err(ctx.hop_traces(dev(U), 0.13, K), O.per_t(S.hop_traces(U, 0.13, K, dims))) < 1e-13
+
+
+@pytest.mark.parametrize("prec,eps", [(lqcd.PREC_F16, 2.0 ** -11), (lqcd.PREC_BF16, 2.0 ** -8)])
+def test_packed_register_forms(prec, eps):
+    """Six fields of 12^3 x 24 are more than two waves of the wide form's blocks, a pair of them less: each pair
+    against the same fields in the block, to one rounding of the storage."""
+    dims, n = (12, 12, 12, 24), 6
+    ctx = context(dims)
+    Up = ctx.pack_links_f32(dev(synth.su3_links(dims, 0.4323, 13)), 12)
+    p = ctx.pack_half(dev(fields(dims, n, 14)), prec)
+    for flag in (0, 1, 2, 3):
+        whole = host(ctx.unpack_half(ctx.wilson_apply_half(Up, 12, 0.137, p, flags=flag, prec=prec), prec))
+        for r in (0, 4):
+            pair = host(ctx.unpack_half(ctx.wilson_apply_half(Up, 12, 0.137, p[r:r + 2].contiguous(), flags=flag,
+                                                              prec=prec), prec))
+            for a, b in ((pair.real, whole[r:r + 2].real), (pair.imag, whole[r:r + 2].imag)):
+                assert (np.abs(a - b) <= 2 * eps * np.abs(b) + 1e-7 * np.abs(whole).max()).all()
