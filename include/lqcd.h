@@ -317,6 +317,15 @@ lqcd_status lqcd_tc_v_c(lqcd_ctx *ctx, const double *E, int k, const double *C, 
  * or more than 2^28 sites, the limits of lqcd_ctx_create), k outside 1..4096 or a NULL bytes. */
 lqcd_status lqcd_tc_slice_bytes(const int dims[4], int k, size_t *bytes);
 
+/* Inner products and update of a Gram-Schmidt step, as the FP64 Krylov cycles take them: the nvec x nrhs
+ * fields V (device; vector i of right-hand side r is field i * nrhs + r) in block fixed point, 60 bits
+ * relative to the largest entry of each site.  Sites that this form does not hold (NaN, Inf, largest entry
+ * outside 2^-623 .. 2^1023) take FP64 sums.  1 <= nvec <= 512; h: device, nvec x nrhs complex128.
+ * lqcd_basis_dot: h[i * nrhs + r] = V_i^r^dagger w^r;  lqcd_basis_update: w^r -= sum_i V_i^r h[i * nrhs + r].
+ * LQCD_ERR_OOM if the second copy of V does not fit. */
+lqcd_status lqcd_basis_dot(lqcd_ctx *ctx, const double *V, int nvec, const double *w, int nrhs, double *h);
+lqcd_status lqcd_basis_update(lqcd_ctx *ctx, const double *V, int nvec, const double *h, double *w, int nrhs);
+
 /* ---- perturbative and polynomial series (Sec. 5.1, 5.2) ---------------------- */
 
 /* out = sum_{k=0}^{K-1} c_k (kappa P)^k eta; c: host K complex, or NULL for all ones (PS). */

@@ -79,9 +79,9 @@ __global__ void __launch_bounds__(FB, 2) fx_multidot_kernel(Field f, const doubl
     const double2 *m = st.mine();
     int mx = 0;
 #pragma unroll
-    for (int e = 0; e < 12; ++e) mx = max(mx, max(abs_hi(m[e].x), abs_hi(m[e].y)));
+    for (int e = 0; e < 12; ++e) mx = max(mx, max(mag(m[e].x), mag(m[e].y)));
     const int Xw = mx >> 20;
-    const bool live = s0 < S && mx != 0;
+    const bool held = Xw >= FX_MINX && Xw < 0x7ff;   // the integers of w are its values
     int wh[12][2], wl[12][2];
 #pragma unroll
     for (int e = 0; e < 12; ++e) {
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(FB, 2) fx_multidot_kernel(Field f, const doubl
       if (j >= ng) break;
       issue(j + 2);
       const long long fld = (long long)(i0 + j) * nrhs + r;
-      const int X = __ldg(f.ex + fld * S + s) + Xw;
+      const int xv = __ldg(f.ex + fld * S + s), X = xv + Xw;
       wait_but<2>();
       __syncwarp();
       const longlong2 *q = (const longlong2 *)(ring + (j % DRING) * DSTAGE) + lane;
@@ -125,12 +125,12 @@ __global__ void __launch_bounds__(FB, 2) fx_multidot_kernel(Field f, const doubl
         re = madw(re, (int)(mr >> 32), 1);
         im = madw(im, (int)(mi >> 32), 1);
       }
-      if (live) {
-        if (X >= X_LOW && X <= X_HIGH) {
+      if (s0 < S) {
+        if (held && X >= X_LOW && X <= X_HIGH) {
           const double k = pow2(X - 2100);
           acc[2 * j] = fma((double)re, k, acc[2 * j]);
           acc[2 * j + 1] = fma((double)im, k, acc[2 * j + 1]);
-        } else if (X - Xw != FX_MINX) {   // not a block of zeros: in FP64
+        } else if (mx == 0 ? xv == FX_BAD : xv != FX_MINX || Xw == 0x7ff) {   // no block of zeros, or one against NaN, Inf
           const double2 *v = V + (fld * S + s) * 12;
           double dr = 0.0, di = 0.0;
 #pragma unroll 1
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(FB * VS, 8 / VS) fx_multiaxpy_kernel(Field f, 
   bool odd = false;   // a coefficient outside the range of the integers
   for (int i = threadIdx.x; i < nvec; i += FB * VS) {
     const double2 a = h[(long long)i * nrhs + r];
-    const int X = max(abs_hi(a.x), abs_hi(a.y)) >> 20;
+    const int X = max(mag(a.x), mag(a.y)) >> 20;
     const bool zero = a.x == 0.0 && a.y == 0.0;
     odd = odd || X >= 0x7fe || (X < FX_MIN_FIELD && !zero);
     int4 c;
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(FB * VS, 8 / VS) fx_multiaxpy_kernel(Field f, 
 #pragma unroll 4
   for (int i = gw; i < nvec; i += 4 * VS) {
     const int xv = __ldg(f.ex + ((long long)i * nrhs + r) * S + s), xh = cx[i];
-    if (xv == FX_MINX || xh == 0) continue;
+    if (xv == FX_MINX || (xh == 0 && xv != FX_BAD)) continue;
     const int X = xv + xh;
     odd = odd || X > X_HIGH || X < X_LOW;
     share(E, tot, X, 1.f);
@@ -392,4 +392,37 @@ lqcd_status fx_multiaxpy(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, co
   (vs == 4 ? fx_multiaxpy_kernel<4> : fx_multiaxpy_kernel<1>)
       <<<(unsigned)grid, FB * vs, nvec * (sizeof(int4) + sizeof(int)), ctx->stream>>>(f, V, h, sign, w, (int)S, nvec, nrhs);
   return launch_check_bytes(ctx, "fx_multiaxpy_kernel", K_AXPY, 12.0 * S * nrhs * nvec, 196.0 * S * nrhs * nvec + 384.0 * S * nrhs);
+}
+
+// Integers of nvec x nrhs canonical fields V in WS_FX_BASIS
+static lqcd_status basis_field(lqcd_ctx *ctx, const double2 *V, int nvec, int nrhs, fx::Field *f) {
+  const long long S = ctx->V, cnt = (long long)nvec * nrhs;
+  if ((S / 32 + 1) * cnt > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "basis product: too many vectors");
+  const size_t qb = (size_t)cnt * fx::blocks32(S) * 384 * sizeof(longlong2);
+  char *p;
+  LQCD_TRY(ws_get(ctx, WS_FX_BASIS, qb + (size_t)cnt * S * sizeof(int), (void **)&p));
+  f->q = (longlong2 *)p;
+  f->ex = (int *)(p + qb);
+  return fx_convert(ctx, V, *f, S, (int)cnt);
+}
+
+extern "C" lqcd_status lqcd_basis_dot(lqcd_ctx *ctx, const double *V, int nvec, const double *w, int nrhs, double *h) {
+  if (!ctx) return LQCD_ERR_INVALID_ARG;
+  if (!V || !w || !h || nvec < 1 || nvec > FAXPY_MAXV || nrhs < 1 || nrhs > 65535)
+    return set_err(ctx, LQCD_ERR_INVALID_ARG, "basis_dot: bad arguments");
+  FxScope scope(ctx);
+  fx::Field f;
+  LQCD_TRY(fx_blas_reserve(ctx, ctx->V, nrhs, nvec));
+  LQCD_TRY(basis_field(ctx, (const double2 *)V, nvec, nrhs, &f));
+  return fx_multidot(ctx, f, (const double2 *)V, (const double2 *)w, ctx->V, nvec, nrhs, (double2 *)h);
+}
+
+extern "C" lqcd_status lqcd_basis_update(lqcd_ctx *ctx, const double *V, int nvec, const double *h, double *w, int nrhs) {
+  if (!ctx) return LQCD_ERR_INVALID_ARG;
+  if (!V || !w || !h || nvec < 1 || nvec > FAXPY_MAXV || nrhs < 1 || nrhs > 65535)
+    return set_err(ctx, LQCD_ERR_INVALID_ARG, "basis_update: bad arguments");
+  FxScope scope(ctx);
+  fx::Field f;
+  LQCD_TRY(basis_field(ctx, (const double2 *)V, nvec, nrhs, &f));
+  return fx_multiaxpy(ctx, f, (const double2 *)V, (const double2 *)h, -1.0, (double2 *)w, ctx->V, nvec, nrhs);
 }

@@ -78,7 +78,8 @@ __device__ __forceinline__ unsigned long long mantissa(double x) {
   return (((unsigned long long)((__double2hiint(x) & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x)) << 11;
 }
 __device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-__device__ __forceinline__ int abs_hi(double x) { return __double2hiint(x) & 0x7fffffff; }
+// for maxima over a block: its exponent field is that of the largest real, and 0 means that all are zero
+__device__ __forceinline__ int mag(double x) { return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0); }
 // x -> trunc(x 2^(1086 - base)), base = X + 4 for 60 bits
 __device__ __forceinline__ long long fixed(double x, int base) {
   const long long s = __double2hiint(x) >> 31;

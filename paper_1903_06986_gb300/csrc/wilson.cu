@@ -155,7 +155,7 @@ __device__ __forceinline__ void links_block(const double2 *__restrict__ U, int4 
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     v[e] = __ldg(u + e);
-    mx = max(mx, max(fx::abs_hi(v[e].x), fx::abs_hi(v[e].y)));
+    mx = max(mx, max(fx::mag(v[e].x), fx::mag(v[e].y)));
   }
   const int X = max(mx >> 20, fx::FX_MINX);
   ex[(long long)mu * VL + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_LINK) ? fx::FX_BAD : X;
@@ -188,7 +188,7 @@ __device__ __forceinline__ void convert_block(const double2 *__restrict__ in, co
 #pragma unroll
   for (int c = 0; c < 12; ++c) {
     v[c] = st.mine()[c];
-    mx = max(mx, max(fx::abs_hi(v[c].x), fx::abs_hi(v[c].y)));
+    mx = max(mx, max(fx::mag(v[c].x), fx::mag(v[c].y)));
   }
   const int X = max(mx >> 20, fx::FX_MINX);
   f.ex[(long long)r * S + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_FIELD) ? fx::FX_BAD : X;

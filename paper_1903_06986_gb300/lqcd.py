@@ -136,6 +136,8 @@ def load(path=None):
         "lqcd_deflate_project": [vp, vp, vp, vp, i, vp],
         "lqcd_set_defl_engine": [vp, i],
         "lqcd_set_wait_limit": [vp, d],
+        "lqcd_basis_dot": [vp, vp, i, vp, i, vp],
+        "lqcd_basis_update": [vp, vp, i, vp, vp, i],
         "lqcd_inject_tc_stall": [vp, i],
         "lqcd_tc_vdag_x": [vp, vp, i, vp, i, vp],
         "lqcd_tc_v_c": [vp, vp, i, vp, i, vp],
@@ -607,6 +609,17 @@ class Context:
         Y = _torch().empty((nrhs,) + tuple(E.shape[1:]), dtype=_torch().complex128, device=E.device)
         self._check(self.lib.lqcd_tc_v_c(self.h, _ptr(E), k, _ptr(Cm.contiguous()), nrhs, _ptr(Y)))
         return Y
+
+    def basis_dot(self, V, w):
+        """h[i, r] = <V_i^r, w^r> as in the FP64 Krylov cycles; V (nvec, nrhs, ...) and w (nrhs, ...) fields."""
+        h = _torch().empty(tuple(V.shape[:2]), dtype=_torch().complex128, device=V.device)
+        self._check(self.lib.lqcd_basis_dot(self.h, _ptr(V), V.shape[0], _ptr(w), w.shape[0], _ptr(h)))
+        return h
+
+    def basis_update(self, V, h, w):
+        """w^r -= sum_i V_i^r h[i, r] (in place) as in the FP64 Krylov cycles."""
+        self._check(self.lib.lqcd_basis_update(self.h, _ptr(V), V.shape[0], _ptr(h.contiguous()), _ptr(w), w.shape[0]))
+        return w
 
     # perturbative and polynomial series
     def hop_series(self, links, kappa, eta, K, c=None):
