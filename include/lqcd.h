@@ -162,7 +162,15 @@ lqcd_status lqcd_noise_z4(lqcd_ctx *ctx, uint64_t seed, uint32_t first_noise, in
 
 /* out = A in for nrhs fields, A selected by flags (LQCD_APPLY_*).  links: device gauge field;
  * in/out: device, nrhs * 12 V complex128, must not overlap.  prec must be LQCD_PREC_F64 or
- * LQCD_PREC_F32 (FP32 arithmetic on FP64 data, for testing the inner operator). */
+ * LQCD_PREC_F32 (FP32 arithmetic on FP64 data, for testing the inner operator).
+ * LQCD_PREC_F64 forms the hopping term of a site in block fixed point (60 bits relative to the largest
+ * entry of each neighbour and link) and its share in the result to about 2^-53 of the largest
+ * product around the site.  Sites where that would lose an entry of FP64 are computed in FP64 entry by
+ * entry: NaN, Inf or magnitudes near the ends of the exponent range; a non-zero complex entry of a
+ * neighbour or link below 2^-12 of that block's largest real, or a non-zero real below 2^-24 of it;
+ * neighbours whose products are more than 2^8 apart.  The same holds for the even/odd operators and
+ * the point-split terms of lqcd_contract.  The Gram-Schmidt sums of FP64 Krylov cycles are exact to about
+ * 2^-53 of the largest product of each site (lqcd_basis_dot), with no such rule for small entries. */
 lqcd_status lqcd_wilson_apply(lqcd_ctx *ctx, const double *links, double kappa, const double *in,
                               double *out, int nrhs, int prec, int flags);
 

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(FB, 2) fx_multidot_kernel(Field f, const doubl
       if (j >= ng) break;
       issue(j + 2);
       const long long fld = (long long)(i0 + j) * nrhs + r;
-      const int xv = __ldg(f.ex + fld * S + s), X = xv + Xw;
+      const int xv = __ldg(f.ex + fld * S + s) & ~FX_WIDE, X = xv + Xw;
       wait_but<2>();
       __syncwarp();
       const longlong2 *q = (const longlong2 *)(ring + (j % DRING) * DSTAGE) + lane;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(FB * VS, 8 / VS) fx_multiaxpy_kernel(Field f, 
   };
 #pragma unroll 4
   for (int i = gw; i < nvec; i += 4 * VS) {
-    const int xv = __ldg(f.ex + ((long long)i * nrhs + r) * S + s), xh = cx[i];
+    const int xv = __ldg(f.ex + ((long long)i * nrhs + r) * S + s) & ~FX_WIDE, xh = cx[i];
     if (xv == FX_MINX || (xh == 0 && xv != FX_BAD)) continue;
     const int X = xv + xh;
     odd = odd || X > X_HIGH || X < X_LOW;
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(FB * VS, 8 / VS) fx_multiaxpy_kernel(Field f, 
 #pragma unroll 4
     for (int i = vg; i < nvec; i += VS, q += (long long)VS * nrhs * fq, ex += (long long)VS * nrhs * S) {
       const int4 k = cf[i];
-      const int sh = max(0, min(E - __ldg(ex) - cx[i], 63));   // out of 0..63 only where the product is 0
+      const int sh = max(0, min(E - (__ldg(ex) & ~FX_WIDE) - cx[i], 63));   // out of 0..63 only where the product is 0
       const int nzh = -k.z, nzl = -k.w;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {

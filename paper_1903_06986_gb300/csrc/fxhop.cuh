@@ -21,7 +21,7 @@
 // below the roundings of the FP64 chain it replaces (tests/test_gpu_fxhop.py compares both with
 // extended precision).
 // Sites or links with a NaN, an Inf, or a scale near the ends of the exponent range carry the exponent
-// FX_BAD; the threads that meet one run the plain FP64 stencil.
+// FX_BAD, those with entries far apart FX_WIDE; the threads that meet one run the plain FP64 stencil.
 //
 // Layout: blocks of 32 sites, [block][component][site of the block] with 16 bytes each (components: the
 // 12 of a field; 9 entries of each of the four links), so that a warp reads 512 contiguous bytes and
@@ -51,6 +51,14 @@ __device__ __forceinline__ long long slot(int s, int per) { return (long long)(s
 constexpr int FX_BAD = 1 << 20;       // exponent that sends the thread to the FP64 stencil
 constexpr int FX_MINX = 64;           // X of a block of zeros (and the least a shift may start from)
 constexpr int FX_MIN_FIELD = 400, FX_MIN_LINK = 700;   // smaller non-zero blocks are FX_BAD
+// Entries far apart: the integers hold an entry to 2^-60 of its block's largest, where FP64 holds each to its own
+// 53 bits.  A block with a non-zero complex entry below 2^-12 of the largest real, or a real below 2^-24, has
+// FX_WIDE added to its exponent, and the stencil and the contraction read it in FP64; so do sites whose
+// neighbours' products are more than FX_SPREAD binary orders apart.  The lines lie where fields of Gaussian
+// entries hardly ever cross them: 3e-6 of the sites, so that one warp in a thousand of the stencil (32 sites and
+// their neighbours) takes its FP64 form; at 2^-8 and 2^-16 one in four would.  Sums over a site (fxblas.cu)
+// use the integers.
+constexpr int FX_WIDE = 1 << 16, FX_ENTRY = 12, FX_REAL = 24, FX_SPREAD = 8;
 constexpr int SITE_BYTES = 208;       // 192 + 16: lanes of a quarter warp fall on distinct banks
 constexpr int WARP_BYTES = 32 * SITE_BYTES;
 
@@ -80,6 +88,24 @@ __device__ __forceinline__ unsigned long long mantissa(double x) {
 __device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 // for maxima over a block: its exponent field is that of the largest real, and 0 means that all are zero
 __device__ __forceinline__ int mag(double x) { return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0); }
+// Exponent of a block of complex entries, as it is stored: X [+ FX_WIDE], or FX_BAD
+struct Range {
+  int mx = 0;                              // largest magnitude word
+  unsigned entry = ~0u, real = ~0u;        // smallest of the non-zero entries and reals, minus 1
+  __device__ __forceinline__ void add(double2 v) {
+    const int a = mag(v.x), b = mag(v.y), m = max(a, b);
+    mx = max(mx, m);
+    entry = min(entry, (unsigned)m - 1u);
+    real = min(real, min((unsigned)a - 1u, (unsigned)b - 1u));
+  }
+  __device__ __forceinline__ int X() const { return max(mx >> 20, FX_MINX); }
+  __device__ __forceinline__ int stored(int least) const {
+    const int x = X();
+    if (x == 0x7ff || (mx != 0 && x < least)) return FX_BAD;
+    const bool wide = mx != 0 && ((int)((entry + 1) >> 20) < x - FX_ENTRY || (int)((real + 1) >> 20) < x - FX_REAL);
+    return wide ? x + FX_WIDE : x;
+  }
+};
 // x -> trunc(x 2^(1086 - base)), base = X + 4 for 60 bits
 __device__ __forceinline__ long long fixed(double x, int base) {
   const long long s = __double2hiint(x) >> 31;
@@ -300,16 +326,21 @@ __device__ __forceinline__ void hop(const Field &f, int r, long long S, bool g5,
   const longlong2 *q = f.q + (long long)r * blocks32(S) * 384;
   const int *ex = f.ex + (long long)r * S;
   A.E = 0;
+  int low = 1 << 30;   // the least of the products that are not zero
 #pragma unroll
   for (int d = 0; d < 8; ++d) {
     const int n = nbr(d);
-    A.E = max(A.E, __ldg(ex + (COMPACT ? n >> 1 : n)) + __ldg(L.ex + (d >> 1) * VL + ((d & 1) ? n : s)) + 2);
+    const int xf = __ldg(ex + (COMPACT ? n >> 1 : n)), xl = __ldg(L.ex + (d >> 1) * VL + ((d & 1) ? n : s));
+    A.E = max(A.E, xf + xl + 2);
+    if (xf != FX_MINX && xl != FX_MINX) low = min(low, xf + xl + 2);
   }
-  A.bad = A.E > 2900;   // FX_BAD among them, or kappa 2^(E - 2101) without room to the end of the range
+  // FX_BAD or FX_WIDE among them, products far apart, or kappa 2^(E - 2101) without room to the end of the range
+  A.bad = A.E > 2900 || A.E - low > FX_SPREAD;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) A.v[a][c][0] = A.v[a][c][1] = 0;
+  if (__all_sync(0xffffffffu, A.bad)) return;
 #pragma unroll 1
   for (int d = d0; d < d1; ++d) {
     const int n = nbr(d), m = COMPACT ? n >> 1 : n, l = (d & 1) ? n : s;

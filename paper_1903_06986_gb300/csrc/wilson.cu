@@ -151,14 +151,14 @@ __device__ __forceinline__ void links_block(const double2 *__restrict__ U, int4 
   if (s >= VL) return;
   const double2 *u = U + ((long long)mu * VL + s) * 9;
   double2 v[9];
-  int mx = 0;
+  fx::Range rg;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     v[e] = __ldg(u + e);
-    mx = max(mx, max(fx::mag(v[e].x), fx::mag(v[e].y)));
+    rg.add(v[e]);
   }
-  const int X = max(mx >> 20, fx::FX_MINX);
-  ex[(long long)mu * VL + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_LINK) ? fx::FX_BAD : X;
+  const int X = rg.X();
+  ex[(long long)mu * VL + s] = rg.stored(fx::FX_MIN_LINK);
   int4 *o = q + fx::slot(s, 36) + mu * 9 * 32;
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
@@ -184,14 +184,14 @@ __device__ __forceinline__ void convert_block(const double2 *__restrict__ in, co
   __syncwarp();
   if (s0 >= S) return;
   double2 v[12];
-  int mx = 0;
+  fx::Range rg;
 #pragma unroll
   for (int c = 0; c < 12; ++c) {
     v[c] = st.mine()[c];
-    mx = max(mx, max(fx::mag(v[c].x), fx::mag(v[c].y)));
+    rg.add(v[c]);
   }
-  const int X = max(mx >> 20, fx::FX_MINX);
-  f.ex[(long long)r * S + s] = X == 0x7ff || (mx != 0 && X < fx::FX_MIN_FIELD) ? fx::FX_BAD : X;
+  const int X = rg.X();
+  f.ex[(long long)r * S + s] = rg.stored(fx::FX_MIN_FIELD);
   longlong2 *o = f.q + (long long)r * fx::blocks32(S) * 384 + fx::slot(s, 12);
 #pragma unroll
   for (int c = 0; c < 12; ++c) o[c * 32] = make_longlong2(fx::fixed(v[c].x, 4 + X), fx::fixed(v[c].y, 4 + X));

@@ -4,7 +4,7 @@ import pytest
 
 from oracle import lattice as L, operators as O
 from paper_1903_06986_gb300 import synth
-from tests.gpu_util import context, dev, rel_err
+from tests.gpu_util import context, dev, host, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -27,3 +27,95 @@ def test_contract_where_eta_times_the_integers_leaves_fp64(scale):
     assert np.isfinite(got).all()
     assert rel_err(got[0], ref[0]) < 1e-13
     assert rel_err(got[1] / scale, ref[1]) < 1e-13
+
+
+KAPPA, EPS = 0.157, 2.0 ** -53
+
+
+def abs_hop(U, psi):
+    """sum over the directions of |1 -+ gamma| |U| |psi|: what roundings of the FP64 stencil are relative to."""
+    a, out = np.abs(psi), 0.0
+    for mu in range(4):
+        m, p = np.abs(L.ONE4 - L.G[mu]), np.abs(L.ONE4 + L.G[mu])
+        out = out + L.spin_apply(m, L.color_apply(np.abs(U[mu]), L.shift(a, mu, +1)))
+        out = out + L.shift(L.spin_apply(p, L.color_apply_dag(np.abs(U[mu]).astype(complex), a)), mu, -1)
+    return np.abs(out)
+
+
+def around(dims, psi):
+    """Largest real of the neighbours of each site, and the smallest such largest real that is not zero."""
+    big = np.maximum(np.abs(psi.real), np.abs(psi.imag)).max(axis=(-1, -2))[..., None, None]
+    nb = np.stack([L.shift(big, mu, s) for mu in range(4) for s in (+1, -1)])
+    return nb.max(0), np.where(nb > 0, nb, np.inf).min(0)
+
+
+def links(dims, kind):
+    U = synth.su3_links(dims, 0.4323, 5)
+    if kind != "su3":
+        U = np.broadcast_to(np.eye(3, dtype=complex), U.shape).copy()
+    if kind == "weak":
+        r = np.random.default_rng(6)
+        U += 1e-7 * (r.standard_normal(U.shape) + 1j * r.standard_normal(U.shape))
+    return U
+
+
+def spread(dims, n, kind):
+    r = np.random.default_rng(7)
+    psi = field(dims, n, 8)
+    if kind == "within a site":        # 14 decades between the entries of a site
+        psi *= 10.0 ** -r.uniform(0, 14, psi.shape)
+    if kind == "reals":                # real and imaginary parts nine decades apart
+        psi = psi.real + 1e-9j * psi.imag
+    if kind == "spins":
+        psi[..., 1, :] *= 1e-8
+    if kind == "sites":                # neighbours 2^-20 of each other
+        psi *= np.where(r.random(psi.shape[:5]) < 0.5, 1.0, 2.0 ** -20)[..., None, None]
+    if kind == "point":
+        psi[:] = 0.0
+        psi[:, 1, 0, 1, 2, 2, 1] = 1.0 - 0.5j
+    return psi
+
+
+@pytest.mark.parametrize("kind", ["within a site", "reals", "spins", "sites", "point"])
+@pytest.mark.parametrize("glue", ["unit", "weak", "su3"])
+@pytest.mark.parametrize("dims,n", [((4, 3, 4, 5), 2), ((8, 8, 8, 16), 5)])
+def test_operator_keeps_entries_far_below_the_largest(dims, n, glue, kind):
+    """Entry by entry to FP64 roundings, in both launch forms (one thread per site, four warps per 32 sites), where
+    entries, links or neighbours lie further apart than the integers hold them; closer ones to the
+    integers' unit relative to 2^9 of the smallest neighbour (products at most 2^8 apart, one bit of the mantissas)."""
+    ctx = context(dims)
+    U, psi = links(dims, glue), spread(dims, n, kind)
+    got = host(ctx.wilson_apply(dev(U), KAPPA, dev(psi)))
+    ref = L.wilson(U.astype(np.clongdouble), np.longdouble(KAPPA), psi.astype(np.clongdouble))
+    top, low = around(dims, psi)
+    m = 0.0 if glue == "weak" or kind in ("within a site", "reals", "spins") else np.minimum(top, 2.0 ** 9 * low)
+    m = np.where(np.isfinite(m), m, 0.0)
+    # FP64: at most 24 + 8 + 2 roundings in a chain; integers: as in test_gpu_fxhop
+    tol = 40 * EPS * (np.abs(psi) + KAPPA * abs_hop(U, psi)) + KAPPA * 8 * 6 * 2.0 ** -54 * m
+    assert (np.abs(got - ref) <= tol).all()
+
+
+@pytest.mark.parametrize("kind", ["within a site", "spins"])
+def test_evenodd_hop_keeps_small_entries(kind):
+    from paper_1903_06986_gb300 import lqcd
+    dims = (4, 6, 4, 2)
+    context(dims)
+    ctx = lqcd.EvenOddContext(dims)
+    U, psi = links(dims, "unit"), spread(dims, 3, kind)
+    e, o = ctx.split(dev(psi))
+    ref = host(ctx.split(dev(L.hop(U.astype(np.clongdouble), psi.astype(np.clongdouble)).astype(complex)))[0])
+    tol = host(ctx.split(dev(abs_hop(U, psi).astype(complex)))[0]).real
+    assert (np.abs(host(ctx.hop(dev(U), o, 0)) - ref) <= 41 * EPS * tol).all()
+
+
+def test_contract_keeps_small_entries_of_w():
+    """eta picks the small entries of w alone: point-split densities relative to them."""
+    dims = (4, 3, 4, 6)
+    ctx = context(dims)
+    U, w = links(dims, "unit"), field(dims, 2, 9)
+    w[..., :, 1] *= 1e-8                                   # one colour; unit links do not mix them
+    eta = np.zeros_like(w)
+    eta[..., :, 1] = field(dims, 2, 10)[..., :, 1]
+    got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
+    ref = O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
+    assert rel_err(got, ref) < 1e-13
