@@ -360,6 +360,21 @@ lqcd_status lqcd_poly_coeffs(lqcd_ctx *ctx, const double *links, double kappa, u
  * all: every column of P^k is followed from its source within min(k, K - k) hops. */
 lqcd_status lqcd_hop_traces(lqcd_ctx *ctx, const double *links, double kappa, int K, double *t);
 
+/* Most device memory that the context takes for the integers of its FP64 kernels: converted fields (in
+ * pieces of at most field_bytes, at least one field; the converted links, 592 bytes per site, come
+ * beside them) and the converted basis of an FP64 Krylov cycle.  0 leaves them out: the operator and the
+ * contraction (field_bytes) or the Gram-Schmidt steps (either) run on FP64 sums, 2 to 3 times slower.
+ * Default: 1 GiB and 32 GiB; a basis of up to 4 GiB is kept from call to call.  What exceeds the new
+ * limits is given back, all of it with (0, 0).  Memory that is not there never fails a call: it takes
+ * smaller pieces or the FP64 kernels, for the whole call. */
+lqcd_status lqcd_set_integer_workspace(lqcd_ctx *ctx, size_t field_bytes, size_t basis_bytes);
+
+/* Device bytes of the context's workspace (0 for NULL), and failure injection for tests of the paths that
+ * run out of memory: while bytes > 0, an allocation that would take the workspace beyond bytes fails as if
+ * the device had no more. */
+size_t lqcd_workspace_bytes(const lqcd_ctx *ctx);
+lqcd_status lqcd_inject_memory_limit(lqcd_ctx *ctx, size_t bytes);
+
 /* Full-lattice applications of P per probe in lqcd_hop_traces and in the setup of loop estimates:
  * depth in 1..64 fixes it, capped at K - 1 (every order a full application) and raised where an
  * order would otherwise be completed more than 8 hops around the members; 0 = chosen per call to

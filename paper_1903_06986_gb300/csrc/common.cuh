@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -80,6 +81,11 @@ struct lqcd_ctx {
   // the end of their last use with its stream (a later call on another stream waits for it)
   const void *fx_src;
   int fx_depth;
+  // most bytes of converted fields and of a converted basis (lqcd_set_integer_workspace; 0: FP64 kernels), and
+  // what is left of them in the running call after an allocation failed (one decision for the whole call:
+  // its captured launches must find what the check before them found)
+  size_t fx_field_max, fx_basis_max, fx_field_now, fx_basis_now;
+  size_t memory_limit;       // injected: allocations beyond it fail (lqcd_inject_memory_limit; 0: none)
   cudaEvent_t fx_event;
   cudaStream_t fx_event_stream;
   int inner_window;          // Lanczos window of Hermitian mixed-precision inner cycles (0 = full Gram-Schmidt)
@@ -140,6 +146,7 @@ enum WsSlot {
   WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_FX_LINKS, WS_FX_FIELD, WS_FX_BASIS, WS_NSLOTS
 };
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr);
+void ws_free(lqcd_ctx *ctx, int slot);   // gives the slot's buffer back after the work that uses it
 void graph_cache_clear(lqcd_ctx *ctx);
 // Append the raw bytes of v to a graph key
 template <typename T> inline void key_add(std::string &k, const T &v) { k.append((const char *)&v, sizeof(T)); }
@@ -182,18 +189,25 @@ lqcd_status reduction_counters(lqcd_ctx *ctx, int n, unsigned **c);
 void fx_done(lqcd_ctx *ctx);   // records the end of a use (outside scopes; a scope does it at its end)
 // gives the integers of a Krylov basis (WS_FX_BASIS) back; not while a cycle uses them
 void fx_release_basis(lqcd_ctx *ctx);
-// kept from one call to the next up to this size (a larger one is given back at the end of the call)
+// most bytes of converted fields and of a converted basis, and what is kept of a basis from one call to the next (a larger one is given back at the end of the call)
+// to the next: 1 GiB is 12 fields of 24^3 x 32, enough that the links (0.25 GB there) count little; 32 GiB
+// hold MINRES-DR(240, 200) on that lattice (20.9 GB) and are a ninth of the device
+constexpr size_t FX_FIELD_MAX = (size_t)1 << 30, FX_BASIS_MAX = (size_t)32 << 30;
 constexpr size_t FX_BASIS_KEEP = (size_t)4 << 30;
 struct FxScope {
   lqcd_ctx *ctx;
   explicit FxScope(lqcd_ctx *c) : ctx(c) {
-    if (ctx->fx_depth++ == 0) ctx->fx_src = nullptr;
+    if (ctx->fx_depth++ == 0) {
+      ctx->fx_src = nullptr;
+      ctx->fx_field_now = ctx->fx_field_max;
+      ctx->fx_basis_now = ctx->fx_basis_max;
+    }
   }
   ~FxScope() {
     if (--ctx->fx_depth == 0) {
       if (ctx->fx_src) fx_done(ctx);
       ctx->fx_src = nullptr;
-      if (ctx->ws_size[WS_FX_BASIS] > FX_BASIS_KEEP) fx_release_basis(ctx);
+      if (ctx->ws_size[WS_FX_BASIS] > std::min(FX_BASIS_KEEP, ctx->fx_basis_max)) fx_release_basis(ctx);
     }
   }
   FxScope(const FxScope &) = delete;

@@ -75,6 +75,20 @@ static lqcd_status timing_collect(lqcd_ctx *ctx) {
   return LQCD_OK;
 }
 
+static size_t ws_bytes(const lqcd_ctx *ctx) {
+  size_t n = 0;
+  for (size_t b : ctx->ws_size) n += b;
+  return n;
+}
+
+static cudaError_t device_alloc(lqcd_ctx *ctx, void **p, size_t bytes) {
+  *p = nullptr;
+  // an allocation would invalidate the capture; whoever captures has sized its workspace before
+  if (ctx->stream == ctx->cap_stream) return cudaErrorStreamCaptureUnsupported;
+  if (ctx->memory_limit && ws_bytes(ctx) + bytes > ctx->memory_limit) return cudaErrorMemoryAllocation;
+  return cudaMalloc(p, bytes);
+}
+
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
   if (slot < 0 || slot >= WS_NSLOTS) return set_err(ctx, LQCD_ERR_INVALID_ARG, "bad workspace slot %d", slot);
   if (bytes == 0) bytes = 16;
@@ -89,16 +103,16 @@ lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
       ctx->ws_size[slot] = 0;
     }
     void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = device_alloc(ctx, &p, bytes);
     if (e == cudaErrorMemoryAllocation && slot != WS_FX_BASIS && ctx->ws_ptr[WS_FX_BASIS]) {
       // the integers of a Krylov basis are only the faster form: they make room for what a call needs
       cudaGetLastError();
       fx_release_basis(ctx);
-      e = cudaMalloc(&p, bytes);
+      e = device_alloc(ctx, &p, bytes);
     }
     if (e != cudaSuccess) {
       cudaGetLastError();
-      return set_err(ctx, LQCD_ERR_OOM, "workspace slot %d: cudaMalloc(%zu) failed: %s", slot, bytes, cudaGetErrorString(e));
+      return set_err(ctx, e == cudaErrorStreamCaptureUnsupported ? LQCD_ERR_CUDA : LQCD_ERR_OOM, "workspace slot %d: cudaMalloc(%zu) failed: %s", slot, bytes, cudaGetErrorString(e));
     }
     ctx->ws_ptr[slot] = p;
     ctx->ws_size[slot] = bytes;
@@ -107,14 +121,16 @@ lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
   return LQCD_OK;
 }
 
-void fx_release_basis(lqcd_ctx *ctx) {
-  if (!ctx->ws_ptr[WS_FX_BASIS]) return;
+void ws_free(lqcd_ctx *ctx, int slot) {
+  if (!ctx->ws_ptr[slot]) return;
   graph_cache_clear(ctx);   // captured cycles hold its address
   cudaStreamSynchronize(ctx->stream);
-  cudaFree(ctx->ws_ptr[WS_FX_BASIS]);
-  ctx->ws_ptr[WS_FX_BASIS] = nullptr;
-  ctx->ws_size[WS_FX_BASIS] = 0;
+  cudaFree(ctx->ws_ptr[slot]);   // waits for what other streams still read
+  ctx->ws_ptr[slot] = nullptr;
+  ctx->ws_size[slot] = 0;
 }
+
+void fx_release_basis(lqcd_ctx *ctx) { ws_free(ctx, WS_FX_BASIS); }
 
 void graph_cache_clear(lqcd_ctx *ctx) {
   if (ctx->graph_cache.empty()) return;
@@ -236,8 +252,11 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
   c->inner_gs_passes = 0;
   c->probe_depth = 0;
   c->inner_window = 0;
+  c->memory_limit = 0;
   c->fx_src = nullptr;
   c->fx_depth = 0;
+  c->fx_field_max = c->fx_field_now = FX_FIELD_MAX;
+  c->fx_basis_max = c->fx_basis_now = FX_BASIS_MAX;
   c->fx_event = nullptr;
   c->fx_event_stream = nullptr;
   c->eo = 0;
@@ -304,6 +323,25 @@ lqcd_status lqcd_set_inner_window(lqcd_ctx *ctx, int window) {
     return set_err(ctx, LQCD_ERR_INVALID_ARG, "set_inner_window: window must be 0 or in 2..1024");
   if (window != ctx->inner_window) graph_cache_clear(ctx);
   ctx->inner_window = window;
+  return LQCD_OK;
+}
+
+lqcd_status lqcd_set_integer_workspace(lqcd_ctx *ctx, size_t field_bytes, size_t basis_bytes) {
+  if (!ctx) return LQCD_ERR_INVALID_ARG;
+  graph_cache_clear(ctx);   // captured cycles hold the form that the old limits gave
+  ctx->fx_field_max = ctx->fx_field_now = field_bytes;
+  ctx->fx_basis_max = ctx->fx_basis_now = basis_bytes;
+  if (ctx->ws_size[WS_FX_BASIS] > basis_bytes) ws_free(ctx, WS_FX_BASIS);
+  if (ctx->ws_size[WS_FX_FIELD] > field_bytes) ws_free(ctx, WS_FX_FIELD);
+  if (field_bytes == 0) ws_free(ctx, WS_FX_LINKS);
+  return LQCD_OK;
+}
+
+size_t lqcd_workspace_bytes(const lqcd_ctx *ctx) { return ctx ? ws_bytes(ctx) : 0; }
+
+lqcd_status lqcd_inject_memory_limit(lqcd_ctx *ctx, size_t bytes) {
+  if (!ctx) return LQCD_ERR_INVALID_ARG;
+  ctx->memory_limit = bytes;
   return LQCD_OK;
 }
 

@@ -268,7 +268,7 @@ inline lqcd_status arnoldi_enqueue_fx(Arnoldi &a, int j0) {
 
 // Workspace of the integers of a cycle's basis; none (the plain kernels) for a polynomial preconditioner,
 // for the FP32 operator, where the operator itself has no integers, or where the second copy of the
-// basis would take more than a third of the free memory.
+// basis is beyond the context's limit or does not fit.
 inline lqcd_status arnoldi_fx(Arnoldi &a) {
   lqcd_ctx *ctx = a.ctx;
   a.fx = fx::Field{nullptr, nullptr};
@@ -280,17 +280,14 @@ inline lqcd_status arnoldi_fx(Arnoldi &a) {
   const long long V = ctx->V, cnt = (long long)(a.m + 1) * a.nrhs;
   if ((V / 32 + 1) * cnt > 0x7fffffffLL) return LQCD_OK;
   const size_t qb = (size_t)cnt * fx::blocks32(V) * 384 * sizeof(longlong2), bytes = qb + (size_t)cnt * V * sizeof(int);
-  if (ctx->ws_size[WS_FX_BASIS] < bytes) {
-    size_t fr = 0, total = 0;
-    LQCD_CUDA(ctx, cudaMemGetInfo(&fr, &total));
-    if (bytes > (fr + ctx->ws_size[WS_FX_BASIS]) / 3) return LQCD_OK;
-  }
+  if (bytes > ctx->fx_basis_now) return LQCD_OK;
   // last of the cycle's workspaces, so that none of the others takes its memory back (ws_get)
   LQCD_TRY(fx_blas_reserve(ctx, V, a.nrhs, a.m));
   char *p;
   const lqcd_status st = ws_get(ctx, WS_FX_BASIS, bytes, (void **)&p);
   if (st == LQCD_ERR_OOM) {
     ctx->err.clear();
+    ctx->fx_basis_now = 0;
     return LQCD_OK;
   }
   LQCD_TRY(st);
@@ -351,6 +348,8 @@ lqcd_status arnoldi_launch(ArnoldiT<S> &a, int j0) {
   key_add(key, a.passes);
   key_add(key, a.window);
   key_add(key, a.fx.q);
+  // the form of the FP64 operator
+  if (std::is_same<S, double2>::value) key_add(key, a.ctx->fx_src != nullptr && a.ctx->fx_field_now > 0);
   key_add(key, a.ctx->packed_nr);
   ArnoldiLaunch<S> arg{&a, j0};
   return graph_cached(a.ctx, key, &arnoldi_enqueue<S>, &arg);

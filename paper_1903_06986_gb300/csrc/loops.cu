@@ -1432,6 +1432,8 @@ lqcd_status eo_noise_solve(lqcd_loop *L, const double2 *U, const double2 *eta, d
                            lqcd_solve_info *info) {
   lqcd_ctx *ctx = L->ctx, *ce = L->ce;
   ce->stream = ctx->stream;
+  ce->fx_field_max = ctx->fx_field_max;
+  ce->fx_basis_max = ctx->fx_basis_max;
   FxScope scope_e(ce);
   const long long Ne = ce->N, N = ctx->N;
   double2 *be, *xe, *ye;
@@ -1722,6 +1724,8 @@ lqcd_status loop_setup(lqcd_ctx *ctx, const double *links, double kappa, const l
       return set_err(ctx, LQCD_ERR_CUDA, "loop setup: reduced context creation failed");
     L->ce->graphs = ctx->graphs;
     L->ce->defl_engine = ctx->defl_engine;
+    L->ce->fx_field_max = ctx->fx_field_max;
+    L->ce->fx_basis_max = ctx->fx_basis_max;
     const long long Ne = L->ce->N;
     double2 *be;
     LQCD_TRY(ws_get(L->ce, WS_SPEC, sizeof(double2) * (size_t)Ne * 2, (void **)&be));

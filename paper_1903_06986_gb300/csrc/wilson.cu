@@ -309,7 +309,8 @@ lqcd_status fx_launch(lqcd_ctx *ctx, const double2 *U, double kappa, const doubl
 lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use, bool *pending) {
   const int VL = ctx->eo ? 2 * ctx->V : ctx->V;
   const size_t n = (size_t)4 * VL, qbytes = (size_t)fx::blocks32(VL) * 32 * 36 * sizeof(int4), bytes = qbytes + n * sizeof(int);
-  *use = true;
+  *use = (ctx->fx_depth > 0 ? ctx->fx_field_now : ctx->fx_field_max) > 0;
+  if (!*use) return LQCD_OK;
   const bool have = ctx->fx_depth > 0 && ctx->fx_src == U;   // converted earlier in this call
   if (!have) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -325,6 +326,7 @@ lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use, b
   const lqcd_status st = ws_get(ctx, WS_FX_LINKS, bytes, (void **)&p);
   if (st == LQCD_ERR_OOM) {
     ctx->err.clear();
+    if (ctx->fx_depth > 0) ctx->fx_field_now = 0;
     *use = false;
     return LQCD_OK;
   }
@@ -344,21 +346,28 @@ lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use, b
 }
 
 lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *chunk, bool *use) {
-  // at most 1 GiB of integers: 12 fields of 24^3 x 32, enough that the links (0.25 GB there) count
-  // little, and a bounded share of the memory beside a Krylov basis or hundreds of eigenvectors.
+  // at least one field where any are allowed.
   // Blocks are numbered 32-bit within a chunk: (S / FX_BS + 1) x chunk < 2^31 for all S <= 2^28.
   const size_t qper = (size_t)fx::blocks32(S) * 32 * 12 * sizeof(longlong2), per = qper + S * sizeof(int);
-  *chunk = (int)std::max<long long>(1, std::min<long long>(nrhs, (1ll << 30) / (long long)per));
-  char *p;
-  const lqcd_status st = ws_get(ctx, WS_FX_FIELD, *chunk * per, (void **)&p);
-  *use = st != LQCD_ERR_OOM;
-  if (!*use) {
-    ctx->err.clear();
-    return LQCD_OK;
+  size_t most = ctx->fx_depth > 0 ? ctx->fx_field_now : ctx->fx_field_max;
+  *use = most > 0;
+  while (*use) {
+    *chunk = (int)std::max<long long>(1, std::min<long long>(nrhs, (long long)(most / per)));
+    char *p;
+    const lqcd_status st = ws_get(ctx, WS_FX_FIELD, *chunk * per, (void **)&p);
+    if (st == LQCD_ERR_OOM) {   // fewer fields at a time, then none, until the end of the call
+      ctx->err.clear();
+      most = *chunk > 1 ? *chunk / 2 * per : 0;
+      if (ctx->fx_depth > 0) ctx->fx_field_now = most;
+      *use = most > 0;
+      continue;
+    }
+    LQCD_TRY(st);
+    f->q = (longlong2 *)p;
+    f->ex = (int *)(p + *chunk * qper);
+    break;
   }
-  f->q = (longlong2 *)p;
-  f->ex = (int *)(p + *chunk * qper);
-  return st;
+  return LQCD_OK;
 }
 
 void fx_reserve_small(lqcd_ctx *ctx) {

@@ -136,6 +136,8 @@ def load(path=None):
         "lqcd_deflate_project": [vp, vp, vp, vp, i, vp],
         "lqcd_set_defl_engine": [vp, i],
         "lqcd_set_wait_limit": [vp, d],
+        "lqcd_set_integer_workspace": [vp, C.c_size_t, C.c_size_t],
+        "lqcd_inject_memory_limit": [vp, C.c_size_t],
         "lqcd_basis_dot": [vp, vp, i, vp, i, vp],
         "lqcd_basis_update": [vp, vp, i, vp, vp, i],
         "lqcd_inject_tc_stall": [vp, i],
@@ -179,6 +181,8 @@ def load(path=None):
     lib.lqcd_version.argtypes = []
     lib.lqcd_version.restype = C.c_char_p
     lib.lqcd_kernel_launches.argtypes = [vp]
+    lib.lqcd_workspace_bytes.restype = C.c_size_t
+    lib.lqcd_workspace_bytes.argtypes = [vp]
     lib.lqcd_kernel_launches.restype = C.c_long
     lib.lqcd_timing_enable.argtypes = [vp, i]
     lib.lqcd_timing_enable.restype = C.c_int
@@ -692,6 +696,19 @@ class Context:
     def set_inner_window(self, window):
         """lqcd_set_inner_window: Lanczos window of Hermitian mixed-precision inner cycles (0 = full)."""
         self._check(self.lib.lqcd_set_inner_window(self.h, window))
+
+    def set_integer_workspace(self, field_bytes, basis_bytes):
+        """Most bytes of the integers of the FP64 kernels: converted fields and Krylov basis (0: FP64 sums)."""
+        self._check(self.lib.lqcd_set_integer_workspace(self.h, field_bytes, basis_bytes))
+
+    @property
+    def workspace_bytes(self):
+        """Device bytes of the context's workspace."""
+        return self.lib.lqcd_workspace_bytes(self.h)
+
+    def inject_memory_limit(self, limit):
+        """Failure injection (tests): allocations beyond `limit` bytes of workspace fail (0: off)."""
+        self._check(self.lib.lqcd_inject_memory_limit(self.h, limit))
 
     def set_probe_depth(self, depth):
         """lqcd_set_probe_depth: full applications of P per probe in the hopping traces (0 = by cost)."""
