@@ -365,13 +365,15 @@ lqcd_status lqcd_hop_traces(lqcd_ctx *ctx, const double *links, double kappa, in
  * beside them) and the converted basis of an FP64 Krylov cycle.  0 leaves them out: the operator and the
  * contraction (field_bytes) or the Gram-Schmidt steps (either) run on FP64 sums, 2 to 3 times slower.
  * Default: 1 GiB and 32 GiB; a basis of up to 4 GiB is kept from call to call.  What exceeds the new
- * limits is given back, all of it with (0, 0).  Memory that is not there never fails a call: it takes
- * smaller pieces or the FP64 kernels, for the whole call. */
+ * limits is given back, all of it with (0, 0).  Memory that is not there for them never fails a call: it
+ * takes smaller pieces or the FP64 kernels, for the whole call; and where another allocation of the
+ * context finds no memory, they are given back first. */
 lqcd_status lqcd_set_integer_workspace(lqcd_ctx *ctx, size_t field_bytes, size_t basis_bytes);
 
-/* Device bytes of the context's workspace (0 for NULL), and failure injection for tests of the paths that
- * run out of memory: while bytes > 0, an allocation that would take the workspace beyond bytes fails as if
- * the device had no more. */
+/* Device bytes of the workspace of the context and of the reduced contexts of its even/odd loop estimates (0
+ * for NULL), and failure injection for tests of the paths that
+ * run out of memory: while bytes > 0, an allocation that would take the workspace beyond bytes (counting
+ * its own size on top) fails as if the device had no more. */
 size_t lqcd_workspace_bytes(const lqcd_ctx *ctx);
 lqcd_status lqcd_inject_memory_limit(lqcd_ctx *ctx, size_t bytes);
 

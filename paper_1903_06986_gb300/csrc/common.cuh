@@ -85,6 +85,8 @@ struct lqcd_ctx {
   // what is left of them in the running call after an allocation failed (one decision for the whole call:
   // its captured launches must find what the check before them found)
   size_t fx_field_max, fx_basis_max, fx_field_now, fx_basis_now;
+  int fx_hold;               // > 0 while launches that read the integer basis are being enqueued
+  std::vector<lqcd_ctx *> kin;   // full and reduced context of one loop estimate: used by the same calls
   size_t memory_limit;       // injected: allocations beyond it fail (lqcd_inject_memory_limit; 0: none)
   cudaEvent_t fx_event;
   cudaStream_t fx_event_stream;
@@ -146,6 +148,9 @@ enum WsSlot {
   WS_POLY1, WS_POLY2, WS_POLY3, WS_EO, WS_TC_AC, WS_TC_REXP, WS_PROBE_OFF, WS_HOST_LINKS, WS_FX_LINKS, WS_FX_FIELD, WS_FX_BASIS, WS_NSLOTS
 };
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr);
+// cudaMalloc for everything the library holds on the device: where there is no memory, the integers of the FP64
+// kernels (ctx's and its kin's; the basis first) make room, since they are only the faster form
+cudaError_t dev_malloc(lqcd_ctx *ctx, void **p, size_t bytes);
 void ws_free(lqcd_ctx *ctx, int slot);   // gives the slot's buffer back after the work that uses it
 void graph_cache_clear(lqcd_ctx *ctx);
 // Append the raw bytes of v to a graph key
@@ -187,11 +192,9 @@ lqcd_status fx_multiaxpy(lqcd_ctx *ctx, const fx::Field &f, const double2 *V, co
 // arrival counters of the single-launch reductions (zeroed once, left at zero)
 lqcd_status reduction_counters(lqcd_ctx *ctx, int n, unsigned **c);
 void fx_done(lqcd_ctx *ctx);   // records the end of a use (outside scopes; a scope does it at its end)
-// gives the integers of a Krylov basis (WS_FX_BASIS) back; not while a cycle uses them
-void fx_release_basis(lqcd_ctx *ctx);
-// most bytes of converted fields and of a converted basis, and what is kept of a basis from one call to the next (a larger one is given back at the end of the call)
-// to the next: 1 GiB is 12 fields of 24^3 x 32, enough that the links (0.25 GB there) count little; 32 GiB
-// hold MINRES-DR(240, 200) on that lattice (20.9 GB) and are a ninth of the device
+// most bytes of converted fields and of a converted basis: 1 GiB is 12 fields of 24^3 x 32, enough that the links
+// (0.25 GB there) count little; 32 GiB hold MINRES-DR(240, 200) on that lattice (20.9 GB) and are a ninth of
+// the device.  A basis beyond FX_BASIS_KEEP is given back at the end of the call.
 constexpr size_t FX_FIELD_MAX = (size_t)1 << 30, FX_BASIS_MAX = (size_t)32 << 30;
 constexpr size_t FX_BASIS_KEEP = (size_t)4 << 30;
 struct FxScope {
@@ -207,7 +210,7 @@ struct FxScope {
     if (--ctx->fx_depth == 0) {
       if (ctx->fx_src) fx_done(ctx);
       ctx->fx_src = nullptr;
-      if (ctx->ws_size[WS_FX_BASIS] > std::min(FX_BASIS_KEEP, ctx->fx_basis_max)) fx_release_basis(ctx);
+      if (ctx->ws_size[WS_FX_BASIS] > std::min(FX_BASIS_KEEP, ctx->fx_basis_max)) ws_free(ctx, WS_FX_BASIS);
     }
   }
   FxScope(const FxScope &) = delete;

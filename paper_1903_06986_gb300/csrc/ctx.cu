@@ -78,6 +78,8 @@ static lqcd_status timing_collect(lqcd_ctx *ctx) {
 static size_t ws_bytes(const lqcd_ctx *ctx) {
   size_t n = 0;
   for (size_t b : ctx->ws_size) n += b;
+  for (const lqcd_ctx *k : ctx->kin)
+    for (size_t b : k->ws_size) n += b;
   return n;
 }
 
@@ -86,7 +88,45 @@ static cudaError_t device_alloc(lqcd_ctx *ctx, void **p, size_t bytes) {
   // an allocation would invalidate the capture; whoever captures has sized its workspace before
   if (ctx->stream == ctx->cap_stream) return cudaErrorStreamCaptureUnsupported;
   if (ctx->memory_limit && ws_bytes(ctx) + bytes > ctx->memory_limit) return cudaErrorMemoryAllocation;
-  return cudaMalloc(p, bytes);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+  }
+  return e;
+}
+
+// Gives the integer basis of ctx and its kin back, or (all) their fields and links too; the calls that run go on
+// without them.  Returns whether there was any.
+static bool fx_give_back(lqcd_ctx *ctx, bool all) {
+  bool any = false;
+  auto one = [&](lqcd_ctx *c) {
+    if (c->ws_ptr[WS_FX_BASIS] && c->fx_hold == 0) {
+      any = true;
+      ws_free(c, WS_FX_BASIS);
+      c->fx_basis_now = 0;
+    }
+    if (all && (c->ws_ptr[WS_FX_LINKS] || c->ws_ptr[WS_FX_FIELD]) && c->fx_hold == 0) {
+      any = true;
+      ws_free(c, WS_FX_FIELD);
+      ws_free(c, WS_FX_LINKS);
+      c->fx_src = nullptr;
+      c->fx_field_now = 0;
+    }
+  };
+  one(ctx);
+  for (lqcd_ctx *k : ctx->kin) {
+    if (k->eo) k->stream = ctx->stream;   // as its loop's next call would set it
+    one(k);
+  }
+  return any;
+}
+
+cudaError_t dev_malloc(lqcd_ctx *ctx, void **p, size_t bytes) {
+  cudaError_t e = device_alloc(ctx, p, bytes);
+  for (int all = 0; all < 2 && e == cudaErrorMemoryAllocation; ++all)
+    if (fx_give_back(ctx, all != 0)) e = device_alloc(ctx, p, bytes);
+  return e;
 }
 
 lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
@@ -103,17 +143,17 @@ lqcd_status ws_get(lqcd_ctx *ctx, int slot, size_t bytes, void **ptr) {
       ctx->ws_size[slot] = 0;
     }
     void *p = nullptr;
-    cudaError_t e = device_alloc(ctx, &p, bytes);
-    if (e == cudaErrorMemoryAllocation && slot != WS_FX_BASIS && ctx->ws_ptr[WS_FX_BASIS]) {
-      // the integers of a Krylov basis are only the faster form: they make room for what a call needs
-      cudaGetLastError();
-      fx_release_basis(ctx);
+    // the integers do not push each other out, but for a basis that makes room for links and fields
+    cudaError_t e;
+    if (slot == WS_FX_BASIS || slot == WS_FX_FIELD || slot == WS_FX_LINKS) {
       e = device_alloc(ctx, &p, bytes);
+      if (e == cudaErrorMemoryAllocation && slot != WS_FX_BASIS && fx_give_back(ctx, false)) e = device_alloc(ctx, &p, bytes);
+    } else {
+      e = dev_malloc(ctx, &p, bytes);
     }
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(ctx, e == cudaErrorStreamCaptureUnsupported ? LQCD_ERR_CUDA : LQCD_ERR_OOM, "workspace slot %d: cudaMalloc(%zu) failed: %s", slot, bytes, cudaGetErrorString(e));
-    }
+    if (e != cudaSuccess)
+      return set_err(ctx, e == cudaErrorStreamCaptureUnsupported ? LQCD_ERR_CUDA : LQCD_ERR_OOM,
+                     "workspace slot %d: cudaMalloc(%zu) failed: %s", slot, bytes, cudaGetErrorString(e));
     ctx->ws_ptr[slot] = p;
     ctx->ws_size[slot] = bytes;
   }
@@ -130,7 +170,6 @@ void ws_free(lqcd_ctx *ctx, int slot) {
   ctx->ws_size[slot] = 0;
 }
 
-void fx_release_basis(lqcd_ctx *ctx) { ws_free(ctx, WS_FX_BASIS); }
 
 void graph_cache_clear(lqcd_ctx *ctx) {
   if (ctx->graph_cache.empty()) return;
@@ -253,6 +292,7 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
   c->probe_depth = 0;
   c->inner_window = 0;
   c->memory_limit = 0;
+  c->fx_hold = 0;
   c->fx_src = nullptr;
   c->fx_depth = 0;
   c->fx_field_max = c->fx_field_now = FX_FIELD_MAX;
@@ -277,6 +317,7 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
 
 lqcd_status lqcd_ctx_destroy(lqcd_ctx *ctx) {
   if (!ctx) return LQCD_ERR_INVALID_ARG;
+  for (lqcd_ctx *k : ctx->kin) k->kin.erase(std::remove(k->kin.begin(), k->kin.end(), ctx), k->kin.end());
   cudaStreamSynchronize(ctx->stream);
   graph_cache_clear(ctx);
   cudaStreamSynchronize(ctx->run_stream);
@@ -328,12 +369,19 @@ lqcd_status lqcd_set_inner_window(lqcd_ctx *ctx, int window) {
 
 lqcd_status lqcd_set_integer_workspace(lqcd_ctx *ctx, size_t field_bytes, size_t basis_bytes) {
   if (!ctx) return LQCD_ERR_INVALID_ARG;
-  graph_cache_clear(ctx);   // captured cycles hold the form that the old limits gave
-  ctx->fx_field_max = ctx->fx_field_now = field_bytes;
-  ctx->fx_basis_max = ctx->fx_basis_now = basis_bytes;
-  if (ctx->ws_size[WS_FX_BASIS] > basis_bytes) ws_free(ctx, WS_FX_BASIS);
-  if (ctx->ws_size[WS_FX_FIELD] > field_bytes) ws_free(ctx, WS_FX_FIELD);
-  if (field_bytes == 0) ws_free(ctx, WS_FX_LINKS);
+  auto set = [&](lqcd_ctx *c) {
+    graph_cache_clear(c);   // captured cycles hold the form that the old limits gave
+    c->fx_field_max = c->fx_field_now = field_bytes;
+    c->fx_basis_max = c->fx_basis_now = basis_bytes;
+    if (c->ws_size[WS_FX_BASIS] > basis_bytes) ws_free(c, WS_FX_BASIS);
+    if (c->ws_size[WS_FX_FIELD] > field_bytes) ws_free(c, WS_FX_FIELD);
+    if (field_bytes == 0) ws_free(c, WS_FX_LINKS);
+  };
+  set(ctx);
+  for (lqcd_ctx *k : ctx->kin) {   // the reduced contexts of its loop estimates
+    k->stream = ctx->stream;
+    set(k);
+  }
   return LQCD_OK;
 }
 

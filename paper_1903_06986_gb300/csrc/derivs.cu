@@ -268,7 +268,7 @@ extern "C" lqcd_status lqcd_loop_derivs(lqcd_ctx *ctx, const double *links, doub
   const int nn = o->nnoise;
   // deflation space for GMRES-Proj from the special right-hand side (GMRES-DR on M)
   double2 *bs = nullptr, *xs = nullptr;
-  LQCD_CUDA(ctx, cudaMalloc(&bs, sizeof(double2) * (size_t)N * 2));
+  LQCD_CUDA(ctx, dev_malloc(ctx, (void **)&bs, sizeof(double2) * (size_t)N * 2));
   xs = bs + N;
   lqcd_defl *dm = nullptr;
   struct Guard {
@@ -309,7 +309,7 @@ extern "C" lqcd_status lqcd_loop_derivs(lqcd_ctx *ctx, const double *links, doub
   const int bw = std::min(o->block, nn);
   const long long bn = (long long)bw * N;
   double2 *eta;
-  LQCD_CUDA(ctx, cudaMalloc(&eta, sizeof(double2) * (size_t)bn * 9));
+  LQCD_CUDA(ctx, dev_malloc(ctx, (void **)&eta, sizeof(double2) * (size_t)bn * 9));
   struct Guard2 { void *p; ~Guard2() { if (p) cudaFree(p); } } g2{eta};
   double2 *x = eta + bn, *px = x + bn, *y = px + bn, *g5e = y + bn, *w = g5e + bn, *xp = w + bn, *dxp = xp + bn;
   double2 *hy = dxp + bn;  // the Hermitian path's M' solution before gamma_5

@@ -248,6 +248,11 @@ template <typename S> struct ArnoldiLaunch {
 // every later inner product and update (fxblas.cu).  CGS2 over all vectors, as FP64 solves take it.
 inline lqcd_status arnoldi_enqueue_fx(Arnoldi &a, int j0) {
   lqcd_ctx *ctx = a.ctx;
+  struct Hold {
+    lqcd_ctx *c;
+    explicit Hold(lqcd_ctx *c_) : c(c_) { ++c->fx_hold; }
+    ~Hold() { --c->fx_hold; }
+  } hold(ctx);
   const long long N = a.N, vs = (long long)a.nrhs * N, V = ctx->V, fq = fx::blocks32(V) * 384 * a.nrhs, fe = V * a.nrhs;
   if (j0 > 0) LQCD_TRY(fx_convert(ctx, a.Vb, a.fx, V, j0 * a.nrhs));   // vectors kept by a restart
   for (int j = j0; j < a.m; ++j) {
@@ -746,11 +751,9 @@ lqcd_status gmresdr_core(lqcd_ctx *ctx, const Op &op, const double2 *b, double2 
       d->N = N;
       d->V = d->E = nullptr;
       d->Hbar_dev = nullptr;
-      // the cycles are over: a large integer basis makes room for the space
-      if (ctx->ws_size[WS_FX_BASIS] > FX_BASIS_KEEP) fx_release_basis(ctx);
-      cudaError_t e1 = cudaMalloc(&d->V, sizeof(double2) * (size_t)(k + 1) * N);
-      cudaError_t e2 = cudaMalloc(&d->E, sizeof(double2) * (size_t)k * N);
-      cudaError_t e3 = cudaMalloc(&d->Hbar_dev, sizeof(double2) * (size_t)(k + 1) * k);
+      cudaError_t e1 = dev_malloc(ctx, (void **)&d->V, sizeof(double2) * (size_t)(k + 1) * N);
+      cudaError_t e2 = dev_malloc(ctx, (void **)&d->E, sizeof(double2) * (size_t)k * N);
+      cudaError_t e3 = dev_malloc(ctx, (void **)&d->Hbar_dev, sizeof(double2) * (size_t)(k + 1) * k);
       if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
         cudaGetLastError();
         if (d->V) cudaFree(d->V);
@@ -1036,7 +1039,7 @@ lqcd_status mixed_core(lqcd_ctx *ctx, const Op &op, const lqcd_defl *defl, const
   // the FP32 copy of the deflation space is made once per space and kept with it
   lqcd_defl *dmut = const_cast<lqcd_defl *>(defl);
   if (!dmut->Vf32) {
-    if (cudaMalloc(&dmut->Vf32, sizeof(float2) * (size_t)(k + 1) * N) != cudaSuccess) {
+    if (dev_malloc(ctx, (void **)&dmut->Vf32, sizeof(float2) * (size_t)(k + 1) * N) != cudaSuccess) {
       cudaGetLastError();
       dmut->Vf32 = nullptr;
       return set_err(ctx, LQCD_ERR_OOM, "mixed solve: FP32 copy of the deflation space does not fit");
@@ -1292,7 +1295,7 @@ lqcd_status lqcd_defl_import(lqcd_ctx *ctx, int k, const double *E, const double
   d->V = nullptr;
   d->Hbar_dev = nullptr;
   d->E = nullptr;
-  if (cudaMalloc(&d->E, sizeof(double2) * (size_t)k * ctx->N) != cudaSuccess) {
+  if (dev_malloc(ctx, (void **)&d->E, sizeof(double2) * (size_t)k * ctx->N) != cudaSuccess) {
     cudaGetLastError();
     delete d;
     return set_err(ctx, LQCD_ERR_OOM, "defl_import: allocation failed");
@@ -1327,9 +1330,9 @@ lqcd_status lqcd_defl_import_space(lqcd_ctx *ctx, int k, const double *V, const 
   d->Hbar_dev = nullptr;
   d->tc = nullptr;
   std::unique_ptr<lqcd_defl, lqcd_status (*)(lqcd_defl *)> guard(d, lqcd_defl_destroy);
-  cudaError_t e1 = cudaMalloc(&d->V, sizeof(double2) * (size_t)(k + 1) * d->N);
-  cudaError_t e2 = cudaMalloc(&d->E, sizeof(double2) * (size_t)k * d->N);
-  cudaError_t e3 = cudaMalloc(&d->Hbar_dev, sizeof(double2) * (size_t)(k + 1) * k);
+  cudaError_t e1 = dev_malloc(ctx, (void **)&d->V, sizeof(double2) * (size_t)(k + 1) * d->N);
+  cudaError_t e2 = dev_malloc(ctx, (void **)&d->E, sizeof(double2) * (size_t)k * d->N);
+  cudaError_t e3 = dev_malloc(ctx, (void **)&d->Hbar_dev, sizeof(double2) * (size_t)(k + 1) * k);
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, LQCD_ERR_OOM, "defl_import_space: allocation failed");

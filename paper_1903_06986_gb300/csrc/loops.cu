@@ -1336,7 +1336,7 @@ lqcd_status es_setup(lqcd_loop *L, const double2 *U, F addES) {
     L->es_perm[q] = best;
     found[q] = dist <= 1e-8 * std::max(std::abs(lq), 1e-300);
   }
-  if (cudaMalloc(&L->g5E, sizeof(double2) * (size_t)k * N) != cudaSuccess) {
+  if (dev_malloc(ctx, (void **)&L->g5E, sizeof(double2) * (size_t)k * N) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, LQCD_ERR_OOM, "ES: allocation of the left-vector basis failed");
   }
@@ -1404,13 +1404,13 @@ lqcd_status eo_es_space(lqcd_loop *L, const double *links) {
   const int Q = (int)keep.size();
   if (Q == 0) return LQCD_OK;
   double2 *Ve = nullptr, *E = nullptr;
-  if (cudaMalloc(&Ve, sizeof(double2) * (size_t)Q * ce->N) != cudaSuccess) {
+  if (dev_malloc(ctx, (void **)&Ve, sizeof(double2) * (size_t)Q * ce->N) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, LQCD_ERR_OOM, "ES (even/odd): allocation failed");
   }
   struct G { void *p; ~G() { if (p) cudaFree(p); } } g{Ve};
   for (int i = 0; i < Q; ++i) LQCD_TRY(blas_copy(ce, d->E + (size_t)keep[i] * ce->N, Ve + (size_t)i * ce->N, ce->N));
-  if (cudaMalloc(&E, sizeof(double2) * 2 * (size_t)Q * ctx->N) != cudaSuccess) {
+  if (dev_malloc(ctx, (void **)&E, sizeof(double2) * 2 * (size_t)Q * ctx->N) != cudaSuccess) {
     cudaGetLastError();
     return set_err(ctx, LQCD_ERR_OOM, "ES (even/odd): allocation failed");
   }
@@ -1432,8 +1432,6 @@ lqcd_status eo_noise_solve(lqcd_loop *L, const double2 *U, const double2 *eta, d
                            lqcd_solve_info *info) {
   lqcd_ctx *ctx = L->ctx, *ce = L->ce;
   ce->stream = ctx->stream;
-  ce->fx_field_max = ctx->fx_field_max;
-  ce->fx_basis_max = ctx->fx_basis_max;
   FxScope scope_e(ce);
   const long long Ne = ce->N, N = ctx->N;
   double2 *be, *xe, *ye;
@@ -1726,6 +1724,9 @@ lqcd_status loop_setup(lqcd_ctx *ctx, const double *links, double kappa, const l
     L->ce->defl_engine = ctx->defl_engine;
     L->ce->fx_field_max = ctx->fx_field_max;
     L->ce->fx_basis_max = ctx->fx_basis_max;
+    L->ce->memory_limit = ctx->memory_limit;
+    ctx->kin.push_back(L->ce);
+    L->ce->kin.push_back(ctx);
     const long long Ne = L->ce->N;
     double2 *be;
     LQCD_TRY(ws_get(L->ce, WS_SPEC, sizeof(double2) * (size_t)Ne * 2, (void **)&be));

@@ -875,9 +875,9 @@ lqcd_status tc_slices_make(lqcd_ctx *ctx, const double2 *E, int k, void **out) {
   S->mtc = (int)((S->L + TC_M - 1) / TC_M);
   S->kcc = (k + TC_KCH - 1) / TC_KCH;
   const size_t bg = tc_bytes_g(k, S->L), bc = tc_bytes_c(k, S->L);
-  cudaError_t e1 = cudaMalloc(&S->Ag, bg), e2 = cudaMalloc(&S->Ac, bc);
-  cudaError_t e3 = cudaMalloc(&S->eexp, sizeof(int) * (k + 2) + sizeof(unsigned long long) * k + sizeof(int) * (k + 1));
-  cudaError_t e4 = cudaMalloc(&S->rowexp, sizeof(int) * S->L);
+  cudaError_t e1 = dev_malloc(ctx, (void **)&S->Ag, bg), e2 = dev_malloc(ctx, (void **)&S->Ac, bc);
+  cudaError_t e3 = dev_malloc(ctx, (void **)&S->eexp, sizeof(int) * (k + 2) + sizeof(unsigned long long) * k + sizeof(int) * (k + 1));
+  cudaError_t e4 = dev_malloc(ctx, (void **)&S->rowexp, sizeof(int) * S->L);
   if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess) {
     cudaGetLastError();
     if (e1 == cudaSuccess) cudaFree(S->Ag);

@@ -94,3 +94,53 @@ def test_solve_when_the_integers_do_not_fit(room, evenodd):
     assert torch_cuda().equal(again, want)
     for x in (plain, got):
         assert rel_err(host(x), host(want)) < 1e-10
+
+
+def test_another_allocation_takes_the_room_of_the_integers():
+    """Eigenvectors that fit only without the integer basis, then only without fields and links; what does not
+    fit at all is refused, and the solve gives its bits again afterwards."""
+    dims, k = (4, 4, 4, 6), 6
+    ctx = context(dims)
+    U, b = dev(synth.su3_links(dims, 0.45, 4)), dev(field(dims, 4, 5))
+    E, lam = dev(field(dims, k, 6)), np.linspace(0.1, 0.6, k).astype(complex)
+    solve = lambda: ctx.gmresdr_solve(U, KAPPA, b, 24, 6, 1e-12, max_cycles=40)[0]
+    want, need = solve(), k * 12 * 384 * 16
+    basis, fields = 25 * 4 * field_bytes(384), links_bytes(384) + 4 * field_bytes(384)
+    assert need < fields < basis
+    held = ctx.workspace_bytes
+    ctx.inject_memory_limit(held + need - 1)
+    d1 = ctx.defl_import(E, lam)
+    assert ctx.workspace_bytes <= held - basis
+    ctx.inject_memory_limit(ctx.workspace_bytes + need - 1)
+    d2 = ctx.defl_import(E, lam)
+    assert ctx.workspace_bytes <= held - basis - fields
+    ctx.inject_memory_limit(ctx.workspace_bytes + need - 1)
+    with pytest.raises(lqcd.LqcdError, match="status 6"):
+        ctx.defl_import(E, lam)
+    ctx.inject_memory_limit(0)
+    assert torch_cuda().equal(solve(), want)
+    d1.close(), d2.close()
+
+
+def test_the_full_context_takes_the_room_of_its_reduced_one():
+    """The integers that an even/odd loop's reduced context keeps make room for the full context."""
+    dims, k = (4, 4, 4, 4), 6
+    ctx = context(dims)
+    U = dev(synth.su3_links(dims, 0.45, 2))
+    E, lam = dev(field(dims, k, 6)), np.linspace(0.1, 0.6, k).astype(complex)
+    loop = ctx.loop_setup(U, KAPPA, 3, 4, 4, 30, 8, 3, 3, 1e-10, 1e-10, evenodd=1)
+    try:
+        want = loop.noises(U, 0, 4)[0]
+        ctx.set_integer_workspace(0, 0)              # of both
+        bare = ctx.workspace_bytes
+        ctx.set_integer_workspace(GIB, GIB)
+        assert np.array_equal(loop.noises(U, 0, 4)[0], want)
+        held, own = ctx.workspace_bytes, links_bytes(256) + 4 * field_bytes(256)
+        assert held - bare > own + links_bytes(256) + field_bytes(128)      # both hold some
+        ctx.inject_memory_limit(bare + k * 12 * 256 * 16 + 1000)
+        ctx.defl_import(E, lam).close()
+        assert ctx.workspace_bytes <= bare + 1000
+        ctx.inject_memory_limit(0)
+        assert np.array_equal(loop.noises(U, 0, 4)[0], want)
+    finally:
+        loop.close()
