@@ -115,6 +115,9 @@ typedef struct {
  * link_recon, LQCD_ERR_CUDA if no device is usable. */
 lqcd_status lqcd_ctx_create(lqcd_ctx **ctx, const int dims[4], int link_recon, void *stream);
 lqcd_status lqcd_ctx_destroy(lqcd_ctx *ctx);
+/* Later calls go to stream.  FP64 operator applications (full, hopping and even/odd) and contractions wait on the
+ * device for those queued on the stream before; other calls share workspace with what is still queued
+ * there, so order the new stream after the old one first. */
 lqcd_status lqcd_set_stream(lqcd_ctx *ctx, void *stream);
 /* Message of the last failure on this context ("" if none); valid until the next call. */
 const char *lqcd_last_error_string(const lqcd_ctx *ctx);

@@ -89,7 +89,7 @@ struct lqcd_ctx {
   std::vector<lqcd_ctx *> kin;   // full and reduced context of one loop estimate: used by the same calls
   size_t memory_limit;       // injected: allocations beyond it fail (lqcd_inject_memory_limit; 0: none)
   cudaEvent_t fx_event;
-  cudaStream_t fx_event_stream;
+  unsigned long long fx_event_id;   // of that stream: a handle may come back for another stream, an id does not
   int inner_window;          // Lanczos window of Hermitian mixed-precision inner cycles (0 = full Gram-Schmidt)
   // even/odd reduced context (lqcd_ctx_create_evenodd): fields hold the even sites only (V above is
   // half the lattice), the operator is hat M = 1 - kappa^2 P_eo P_oe, eo_dims the full extents

@@ -298,7 +298,7 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
   c->fx_field_max = c->fx_field_now = FX_FIELD_MAX;
   c->fx_basis_max = c->fx_basis_now = FX_BASIS_MAX;
   c->fx_event = nullptr;
-  c->fx_event_stream = nullptr;
+  c->fx_event_id = 0;
   c->eo = 0;
   for (int i = 0; i < 4; ++i) c->eo_dims[i] = dims[i];
   c->cap_stream = nullptr;

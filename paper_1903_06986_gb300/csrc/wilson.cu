@@ -319,7 +319,8 @@ lqcd_status fx_links(lqcd_ctx *ctx, const double2 *U, fx::Links *L, bool *use, b
       *use = false;
       return LQCD_OK;
     }
-    if (ctx->fx_event && ctx->fx_event_stream != ctx->stream)
+    unsigned long long id = 0;
+    if (ctx->fx_event && (cudaStreamGetId(ctx->stream, &id) != cudaSuccess || id != ctx->fx_event_id))
       LQCD_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->fx_event, 0));
   }
   char *p;
@@ -396,8 +397,11 @@ void fx_done(lqcd_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);   // no event to wait for later: the use ends here
     return;
   }
-  cudaEventRecord(ctx->fx_event, ctx->stream);
-  ctx->fx_event_stream = ctx->stream;
+  if (cudaEventRecord(ctx->fx_event, ctx->stream) != cudaSuccess ||
+      cudaStreamGetId(ctx->stream, &ctx->fx_event_id) != cudaSuccess) {
+    cudaGetLastError();
+    cudaStreamSynchronize(ctx->stream);
+  }
 }
 
 lqcd_status wilson_launch_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,
