@@ -336,6 +336,10 @@ lqcd_status lqcd_tc_slice_bytes(const int dims[4], int k, size_t *bytes);
  * LQCD_ERR_OOM if the second copy of V does not fit. */
 lqcd_status lqcd_basis_dot(lqcd_ctx *ctx, const double *V, int nvec, const double *w, int nrhs, double *h);
 lqcd_status lqcd_basis_update(lqcd_ctx *ctx, const double *V, int nvec, const double *h, double *w, int nrhs);
+/* The inner products of the reduced-precision cycles: V and w packed fields (lqcd_pack_f32, lqcd_pack_half) of
+ * storage prec, summed in FP32 over 8 products at a time at most, their sums to about one FP32 rounding per
+ * thread, then in FP64. */
+lqcd_status lqcd_basis_dot_packed(lqcd_ctx *ctx, int prec, const void *V, int nvec, const void *w, int nrhs, double *h);
 
 /* ---- perturbative and polynomial series (Sec. 5.1, 5.2) ---------------------- */
 

@@ -140,6 +140,7 @@ def load(path=None):
         "lqcd_inject_memory_limit": [vp, C.c_size_t],
         "lqcd_basis_dot": [vp, vp, i, vp, i, vp],
         "lqcd_basis_update": [vp, vp, i, vp, vp, i],
+        "lqcd_basis_dot_packed": [vp, i, vp, i, vp, i, vp],
         "lqcd_inject_tc_stall": [vp, i],
         "lqcd_tc_vdag_x": [vp, vp, i, vp, i, vp],
         "lqcd_tc_v_c": [vp, vp, i, vp, i, vp],
@@ -618,6 +619,12 @@ class Context:
         """h[i, r] = <V_i^r, w^r> as in the FP64 Krylov cycles; V (nvec, nrhs, ...) and w (nrhs, ...) fields."""
         h = _torch().empty(tuple(V.shape[:2]), dtype=_torch().complex128, device=V.device)
         self._check(self.lib.lqcd_basis_dot(self.h, _ptr(V), V.shape[0], _ptr(w), w.shape[0], _ptr(h)))
+        return h
+
+    def basis_dot_packed(self, V, w, nvec, nrhs, prec):
+        """h[i, r] = <V_i^r, w^r> of packed fields as in the reduced-precision cycles; V: nvec * nrhs packed fields."""
+        h = _torch().empty((nvec, nrhs), dtype=_torch().complex128, device=V.device)
+        self._check(self.lib.lqcd_basis_dot_packed(self.h, prec, _ptr(V, V.dtype), nvec, _ptr(w, w.dtype), nrhs, _ptr(h)))
         return h
 
     def basis_update(self, V, h, w):

@@ -153,3 +153,20 @@ def test_a_tiny_site_with_zeros_against_a_large_one():
     w[at + (2, 1)] = 1e-300 - 2e-300j
     d, _ = plain(V, w, h)
     assert np.abs(host(ctx.basis_dot(dev(V), dev(w))) - d).max() <= 1e-14 * np.abs(d).max()
+
+
+@pytest.mark.parametrize("nvec", [1, 2, 7, 8, 11])
+@pytest.mark.parametrize("prec,v,wv", [("f32", 1 + 2.0 ** -9, 1 + 2.0 ** -11), ("f16", 1 + 2.0 ** -10, 1 + 2.0 ** -10)])
+def test_packed_products_of_equal_terms(prec, v, wv, nvec):
+    """Terms 1 + 2^-9 + .. + 2^-20 of equal sign: a chain of FP32 additions drops the last part of each beyond 2^4
+    (2^-21 of the sum and more); sums of at most 8 terms are exact, and their sum is off by a rounding per thread."""
+    from paper_1903_06986_gb300 import lqcd
+    dims, nrhs = (8, 8, 8, 16), 2
+    ctx = context(dims)
+    pr = {"f32": lqcd.PREC_F32, "f16": lqcd.PREC_F16}[prec]
+    pack = (lambda x: ctx.pack_f32(x)) if prec == "f32" else (lambda x: ctx.pack_half(x, pr))
+    V = dev(np.full(L.field_shape(dims, (nvec * nrhs,)), v * (1 + 1j)))
+    w = dev(np.full(L.field_shape(dims, (nrhs,)), wv * (1 + 1j)))
+    h = host(ctx.basis_dot_packed(pack(V), pack(w), nvec, nrhs, pr))
+    want = 2 * v * wv * 12 * 8192
+    assert np.abs(h - want).max() <= 2.0 ** -23 * want
