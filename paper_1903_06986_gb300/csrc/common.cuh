@@ -176,6 +176,8 @@ lqcd_status fx_field(lqcd_ctx *ctx, long long S, int nrhs, fx::Field *f, int *ch
 lqcd_status fx_convert(lqcd_ctx *ctx, const double2 *in, const fx::Field &f, long long S, int nrhs);
 // allocates the two workspaces with the context where they are small (64 MiB at most)
 void fx_reserve_small(lqcd_ctx *ctx);
+// lqcd_ctx_create without them: the extents of a reduced context are set afterwards
+lqcd_status ctx_new(lqcd_ctx **out, const int dims[4], int link_recon, void *stream);
 // FP64 operator (flags as wilson_launch, or 4 with g5mask) on nrhs fields whose integers are f; in: the
 // same fields, canonical
 lqcd_status wilson_launch_converted(lqcd_ctx *ctx, const double2 *U, double kappa, const double2 *in, const fx::Field &f,

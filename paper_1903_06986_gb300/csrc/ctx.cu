@@ -245,11 +245,7 @@ lqcd_status host_stage(lqcd_ctx *ctx, size_t bytes, double **ptr) {
   return LQCD_OK;
 }
 
-extern "C" {
-
-const char *lqcd_version(void) { return "lqcd-gb300 0.1 (sm_103a)"; }
-
-lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, void *stream) {
+lqcd_status ctx_new(lqcd_ctx **out, const int dims[4], int link_recon, void *stream) {
   if (!out || !dims) return LQCD_ERR_INVALID_ARG;
   *out = nullptr;
   for (int i = 0; i < 4; ++i)
@@ -310,9 +306,18 @@ lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, v
     delete c;
     return LQCD_ERR_CUDA;
   }
-  fx_reserve_small(c);
   *out = c;
   return LQCD_OK;
+}
+
+extern "C" {
+
+const char *lqcd_version(void) { return "lqcd-gb300 0.1 (sm_103a)"; }
+
+lqcd_status lqcd_ctx_create(lqcd_ctx **out, const int dims[4], int link_recon, void *stream) {
+  const lqcd_status st = ctx_new(out, dims, link_recon, stream);
+  if (st == LQCD_OK) fx_reserve_small(*out);
+  return st;
 }
 
 lqcd_status lqcd_ctx_destroy(lqcd_ctx *ctx) {

@@ -330,9 +330,9 @@ extern "C" lqcd_status lqcd_ctx_create_evenodd(lqcd_ctx **out, const int dims[4]
   // the reduced context: half the sites, so every field and solver has length 12 V / 2; its dims
   // (Lx/2, Ly, Lz, Lt) describe that length, the full lattice is kept in eo_dims
   int hd[4] = {dims[0] / 2, dims[1], dims[2], dims[3]};
-  int cd[4] = {2, 2, 2, 2};  // placeholder extents accepted by the plain constructor
+  int cd[4] = {2, 2, 2, 2};  // placeholder extents accepted by ctx_new
   lqcd_ctx *c = nullptr;
-  const lqcd_status st = lqcd_ctx_create(&c, cd, link_recon, stream);
+  const lqcd_status st = ctx_new(&c, cd, link_recon, stream);
   if (st != LQCD_OK) return st;
   const long long V = (long long)hd[0] * hd[1] * hd[2] * hd[3];
   if (2 * V > (1LL << 28)) {
