@@ -869,13 +869,16 @@ lqcd_status blas_norms(lqcd_ctx *ctx, const S *x, long long n, int nrhs, double 
 }
 
 static int multidot_chunks(lqcd_ctx *ctx, long long n, int nrhs, int nvec, bool shared, int kv = 1) {
-  // element chunks of at least 8 loads (of kv elements) per thread; enough blocks (chunks x vector groups x
+  // element chunks of at least 8 loads (of kv elements) per thread, but of 8 elements while that leaves fewer
+  // blocks than SMs (two FP16 fields of 8^3 x 16: 12.0 against 9.0 us for eight vectors, 7.1 against 6.4 for two;
+  // up to two or four blocks per SM costs 20 to 60 % on several right-hand sides); enough blocks (chunks x vector groups x
   // right-hand sides) for about 16 per SM, several waves of the 4-6 resident ones, so that no SM
   // idles at the end.  With a basis shared by several right-hand
   // sides, also chunks short enough that the blocks in flight (about 8 per SM) touch at most ~32 MB
   // of L2, so that the basis chunk is read from DRAM once for all of them.
   const int ngroup = (nvec + GROUP - 1) / GROUP;
-  const long long max_chunks = std::max<long long>(1, n / (8LL * kv * BT));
+  const long long fill = ctx->sms / std::max<long long>(1, (long long)nrhs * ngroup);
+  const long long max_chunks = std::max<long long>(1, std::max(n / (8LL * kv * BT), std::min(fill, n / (8LL * BT))));
   long long want = std::max<long long>(1, (16LL * ctx->sms) / std::max<long long>(1, (long long)nrhs * ngroup));
   if (shared && nrhs > 1) {
     const long long per_chunk_blocks = (long long)nrhs * ngroup;

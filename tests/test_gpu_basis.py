@@ -170,3 +170,23 @@ def test_packed_products_of_equal_terms(prec, v, wv, nvec):
     h = host(ctx.basis_dot_packed(pack(V), pack(w), nvec, nrhs, pr))
     want = 2 * v * wv * 12 * 8192
     assert np.abs(h - want).max() <= 2.0 ** -23 * want
+
+
+@pytest.mark.parametrize("dims,nvec,nrhs", [((2, 2, 2, 2), 2, 1), ((4, 4, 4, 8), 8, 1), ((5, 3, 7, 9), 1, 2), ((5, 3, 7, 9), 9, 3),
+                                            ((8, 8, 8, 16), 2, 1), ((12, 12, 12, 24), 2, 1), ((6, 6, 6, 12), 40, 12)])
+@pytest.mark.parametrize("prec", ["f32", "f16"])
+def test_packed_products_of_short_fields(prec, dims, nvec, nrhs):
+    """Chunks of 8 elements per thread where 8 loads would leave SMs without a block, and their remainders."""
+    from paper_1903_06986_gb300 import lqcd
+    ctx = context(dims)
+    pr = {"f32": lqcd.PREC_F32, "f16": lqcd.PREC_F16}[prec]
+    pack = ctx.pack_f32 if prec == "f32" else lambda x: ctx.pack_half(x, pr)
+    unpack = ctx.unpack_f32 if prec == "f32" else lambda x: ctx.unpack_half(x, pr)
+    r = np.random.default_rng(21)
+    make = lambda n: dev(r.standard_normal(L.field_shape(dims, (n,))) + 1j * r.standard_normal(L.field_shape(dims, (n,))))
+    V, w = pack(make(nvec * nrhs)), pack(make(nrhs))
+    got = host(ctx.basis_dot_packed(V, w, nvec, nrhs, pr))
+    v, u = host(unpack(V)).reshape(nvec, nrhs, -1), host(unpack(w)).reshape(nrhs, -1)
+    # FP32 chains of at most 8 products, a rounding of their sums, and those of the stored scale
+    tol = 16 * 2.0 ** -24 * (np.abs(v) * np.abs(u)).sum(-1) * 2 ** 0.5
+    assert (np.abs(got - (v.conj() * u).sum(-1)) <= tol).all()
