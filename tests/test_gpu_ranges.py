@@ -119,3 +119,22 @@ def test_contract_keeps_small_entries_of_w():
     got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
     ref = O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
     assert rel_err(got, ref) < 1e-13
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("what", ["w", "eta", "links"])
+def test_contract_with_a_non_finite_entry(what, bad):
+    """The densities of the timeslices that the entry reaches are not finite, all others are those without it."""
+    dims = (3, 4, 5, 6)
+    ctx = context(dims)
+    U, eta, w = synth.su3_links(dims, 0.5, 1), field(dims, 3, 2), field(dims, 3, 3)
+    eta[2, 3], w[2, 0] = 0.0, 0.0                          # blocks of zeros beside it
+    dens = lambda: O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
+    at, clean = ((3, 2, 1, 0, 2, 1, 1) if what == "links" else (1, 2, 1, 0, 2, 3, 1)), dens()
+    a = {"links": U, "eta": eta, "w": w}[what]
+    a[at] += 1.0 - 2.0j
+    fin = dens() == clean                                  # the projectors of t drop half of the spins
+    a[at] = bad
+    got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
+    assert not fin.all() and np.array_equal(np.isfinite(got), fin)
+    assert np.abs(got - clean)[fin].max() <= 1e-13 * np.abs(clean).max()

@@ -90,3 +90,25 @@ def test_packed_register_forms(prec, eps):
                                                               prec=prec), prec))
             for a, b in ((pair.real, whole[r:r + 2].real), (pair.imag, whole[r:r + 2].imag)):
                 assert (np.abs(a - b) <= 2 * eps * np.abs(b) + 1e-7 * np.abs(whole).max()).all()
+
+
+def test_hop_traces_by_site_at_its_last_order():
+    """K = 9, the largest that is followed source by source: gauge-rotated unit links, whose traces are those of the
+    free field, and general links against the probing form."""
+    from tests.test_oracle_traces import free_hop_traces
+    dims, K = (10, 10, 11, 10), 9
+    ctx = context(dims)
+    r = np.random.default_rng(15)
+    g = np.linalg.qr(r.standard_normal((10, 11, 10, 10, 3, 3)) + 1j * r.standard_normal((10, 11, 10, 10, 3, 3)))[0]
+    U = np.stack([g @ np.roll(g, -1, axis=3 - mu).conj().swapaxes(-1, -2) for mu in range(4)])
+    got, ref = ctx.hop_traces(dev(U), 0.13, K).sum(axis=-1), free_hop_traces(dims, 0.13, K)
+    ref[np.abs(ref) < 1e-3] = 0.0   # zeros of the momentum sum to its rounding; the others are at least 12 V kappa
+    scale = 12.0 * np.prod(dims) * 2.0 ** np.arange(K)
+    assert (np.abs(got - ref).max(axis=-1) <= 1e-13 * np.maximum(np.abs(ref).max(axis=-1), scale)).all()
+    Ud = dev(synth.su3_links(dims, 0.5, 16))
+    got = ctx.hop_traces(Ud, 0.13, K)
+    ctx.set_probe_depth(K - 1)
+    want = ctx.hop_traces(Ud, 0.13, K)
+    for k in range(K):
+        scale = max(np.abs(want[k]).max(), 12.0 * np.prod(dims[:3]) * 2.0 ** k)
+        assert np.abs(got[k] - want[k]).max() <= 1e-13 * scale, k
