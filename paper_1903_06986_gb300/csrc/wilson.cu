@@ -740,12 +740,12 @@ __device__ __forceinline__ __nv_bfloat162 b_fromf(float2 a) { return __float22bf
 template <> struct PairIO<__half2> : PairIOHalf<__half2, h2x2, h_lo, h_hi, h_tof, h_fromf> {};
 template <> struct PairIO<__nv_bfloat162> : PairIOHalf<__nv_bfloat162, b2x2, b_lo, b_hi, b_tof, b_fromf> {};
 
-// Blocks of 64 threads fill the last wave better than 128 (12^3 x 24, 8 right-hand sides: 22.5 us with 128).
-// RES: resident blocks per SM the registers are limited for: 8 (128 registers), or 6 (168) for FP16 / BF16
+// Blocks of 64 threads (PAIR_BT) or, where pair_launch takes them, of 128.
+// RES: resident blocks of 64 per SM the registers are limited for: 8 (128 registers), or 6 (168) for FP16 / BF16
 // fields with rebuilt links where pair_launch takes it.
 constexpr int PAIR_BT = 64;
 template <typename S, int RECON, int MODE, int RES>
-__global__ void __launch_bounds__(PAIR_BT, RES) wilson_pair_kernel(const float4 *__restrict__ U,
+__global__ void __launch_bounds__(2 * PAIR_BT, RES / 2) wilson_pair_kernel(const float4 *__restrict__ U,
                                                           const typename Chunk<S>::T *__restrict__ in,
                                                           typename Chunk<S>::T *__restrict__ out, float kappa,
                                                           int Lx, int Ly, int Lz, int Lt, int V, int nrhs,
@@ -1130,8 +1130,14 @@ lqcd_status pair_launch(lqcd_ctx *ctx, const float4 *U, double kappa, const void
   using T = typename Chunk<S>::T;
   const T *in = (const T *)in_;
   T *out = (T *)out_;
-  int bs = PAIR_BT;
   const int groups = (nrhs + 1) / 2;
+  // FP32 fields of 0.6 to 2.25 waves of 128 threads: blocks of 128 take 1 to 6 % less time (13 x 11 x 15 x 17, 6 fields,
+  // general links: 15.9 against 16.6 us; 20 x 12 x 16 x 24, 2 fields: 12.6 against 13.0; 16^3 x 32, 2 fields: 18.4
+  // against 19.6).  Fewer sites spread better over blocks of 64 (12^3 x 24, 2 fields: 7.9 against 8.2 us), and more
+  // leave a shorter tail (24^3 x 32, 10 fields: 246 against 248 us); so do FP16 and BF16 fields of any size (within
+  // 1 % of blocks of 128 from half a wave on).
+  const long long n128 = (long long)ceil_div(ctx->V, 2 * PAIR_BT) * groups, wave = 4LL * ctx->sms;
+  int bs = sizeof(T) == 16 && 5 * n128 > 3 * wave && 4 * n128 <= 9 * wave ? 2 * PAIR_BT : PAIR_BT;
   while (bs > 32 && (long long)ceil_div(ctx->V, bs) * groups < 2LL * ctx->sms) bs /= 2;
   const long long nblk = (long long)ceil_div(ctx->V, bs) * groups;
   if (nblk > 0x7fffffffLL) return set_err(ctx, LQCD_ERR_INVALID_ARG, "packed wilson: grid too large");
