@@ -349,46 +349,172 @@ __device__ __forceinline__ void hop(const Field &f, int r, long long S, bool g5,
   }
 }
 
-// The same sum in FP64 (bad threads), with the factor -gamma_5 that g5 stands for
+// acc += direction d of the hopping term in FP64 at link-lattice site s, with the factor -gamma_5 that g5 stands for
 template <bool COMPACT, typename Nbr>
-__device__ __noinline__ void hop_fp64(const double2 *U, const double2 *src, long long VL, int s, bool g5, Nbr nbr,
-                                      double2 *out) {
+__device__ __forceinline__ void direction_fp64(int d, const double2 *U, const double2 *src, long long VL, int s, bool g5,
+                                               const Nbr &nbr, Cx<double> acc[4][3]) {
   using namespace spin;
-  Cx<double> acc[4][3], p[4][3], u[9];
+  Cx<double> p[4][3], u[9];
+  const int n = nbr(d);
+  load_spinor<double, false>(src + 12LL * (COMPACT ? n >> 1 : n), p);
+  if (g5) {
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const Cx<double> v = p[a][c];
+        p[a][c] = p[a + 2][c];
+        p[a + 2][c] = v;
+      }
+  }
+  load_link<double>(U, (d >> 1) * VL + ((d & 1) ? n : s), u);
+  switch (d) {
+    case 0: term_fwd<double, 0>(p, u, acc); break;
+    case 1: term_bwd<double, 0>(p, u, acc); break;
+    case 2: term_fwd<double, 1>(p, u, acc); break;
+    case 3: term_bwd<double, 1>(p, u, acc); break;
+    case 4: term_fwd<double, 2>(p, u, acc); break;
+    case 5: term_bwd<double, 2>(p, u, acc); break;
+    case 6: term_fwd<double, 3>(p, u, acc); break;
+    default: term_bwd<double, 3>(p, u, acc); break;
+  }
+}
+
+// The whole sum in FP64
+template <bool COMPACT, typename Nbr>
+__device__ __forceinline__ void hop_fp64(const double2 *U, const double2 *src, long long VL, int s, bool g5,
+                                         const Nbr &nbr, Cx<double> acc[4][3]) {
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[a][c] = mk<double>(0.0, 0.0);
 #pragma unroll 1
+  for (int d = 0; d < 8; ++d) direction_fp64<COMPACT>(d, U, src, VL, s, g5, nbr, acc);
+}
+
+// The same by four warps (run<4>): the upper pairs of directions d0 and d0 + 1 (the lower one of d = 6, whose upper pair
+// is zero), 24 reals 32 slots apart, and their sum for spin a in the order of the whole sum, with its bits.
+template <bool COMPACT, typename Nbr>
+__device__ __noinline__ void halves_fp64(const double2 *U, const double2 *src, long long VL, int s, bool g5, Nbr nbr,
+                                         int d0, double *o) {
+#pragma unroll 1
+  for (int d = d0; d < d0 + 2; ++d, o += 12 * 32) {
+    Cx<double> acc[4][3];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[a][c] = mk<double>(0.0, 0.0);
+    direction_fp64<COMPACT>(d, U, src, VL, s, g5, nbr, acc);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const Cx<double> v = d == 6 ? acc[2 + k][c] : acc[k][c];
+        o[(6 * k + 2 * c) * 32] = v.x;
+        o[(6 * k + 2 * c + 1) * 32] = v.y;
+      }
+  }
+}
+// (o: stride doubles between the reals)
+__device__ __forceinline__ Cx<double> sum_halves(const double *o, int stride, int a, int c) {
+  using namespace spin;
+  Cx<double> acc = mk<double>(0.0, 0.0);
+#pragma unroll
   for (int d = 0; d < 8; ++d) {
-    const int n = nbr(d);
-    load_spinor<double, false>(src + 12LL * (COMPACT ? n >> 1 : n), p);
-    if (g5) {
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const Cx<double> v = p[a][c];
-          p[a][c] = p[a + 2][c];
-          p[a + 2][c] = v;
-        }
+    if (a < 2 ? d == 6 : d == 7) continue;
+    const int k = a < 2 ? a : (a == 2) == (d < 4) ? 1 : 0;   // x and y exchange the pair
+    Cx<double> v = mk<double>(o[(12 * d + 6 * k + 2 * c) * stride], o[(12 * d + 6 * k + 2 * c + 1) * stride]);
+    if (a >= 2) {   // conjugate phases of the lower pair: -i, i, (-, +), (+, -), (-i, i), (i, -i)
+      if (d == 0 || d == 1 || d == 4 || d == 5) v = ti(v);
+      if (d == 0 || d == (a == 2 ? 2 : 3) || d == (a == 2 ? 4 : 5)) v = neg(v);
     }
-    load_link<double>(U, (d >> 1) * VL + ((d & 1) ? n : s), u);
-    switch (d) {
-      case 0: term_fwd<double, 0>(p, u, acc); break;
-      case 1: term_bwd<double, 0>(p, u, acc); break;
-      case 2: term_fwd<double, 1>(p, u, acc); break;
-      case 3: term_bwd<double, 1>(p, u, acc); break;
-      case 4: term_fwd<double, 2>(p, u, acc); break;
-      case 5: term_bwd<double, 2>(p, u, acc); break;
-      case 6: term_fwd<double, 3>(p, u, acc); break;
-      default: term_bwd<double, 3>(p, u, acc); break;
-    }
+    acc = acc + v;
+  }
+  return acc;
+}
+
+// Half spinor component k of direction d, multiplied by the link, for one site by one lane, without branches on d:
+// lanes of a warp take the 16 (d, k) of a site in turn where a warp has few (FEW) bad ones.  Ordinary fields have a bad
+// site in one warp of a thousand, and an FP64 instruction holds the pipe for 16 clocks however many lanes take part: the
+// whole sum by one lane was a tail of 20 us at the end of a launch.  Four fields of 12^3 x 24, conversions
+// included: M 134.7 us with it, 109.3 so (113.6 with no such sites), the even/odd hop 94.5 and 73.0.  More
+// than FEW take a lane per site (10 fields of 24^3 x 32, all sites: 7.26 ms, 6.62 in the plain FP64 kernel before the
+// integers).  n: link-lattice index of the neighbour; o as in halves_fp64.
+constexpr int FEW = 8;
+template <bool COMPACT>
+__device__ __noinline__ void half_fp64(const double2 *U, const double2 *src, long long VL, int s, int n, bool g5, int d,
+                                       int k, double *o, int stride) {
+  using namespace spin;
+  const int mu = d >> 1, bwd = d & 1;
+  const double2 *p = src + 12LL * (COMPACT ? n >> 1 : n);
+  const double2 *u = U + (mu * VL + (bwd ? n : s)) * 9;
+  // h = p_a + phase p_b (table at the head of spin.cuh); the t projection is 2 p of one pair
+  const int up = g5 ? 2 : 0;   // exchanged spins
+  const int a = mu == 3 ? (bwd ? k : 2 + k) : k, b = mu == 3 ? a : mu == 2 ? 2 + k : 3 - k;
+  const bool rot = mu == 0 || mu == 2, minus = mu != 3 && ((bwd != 0) != (mu != 0 && k == 1));
+  Cx<double> h[3], m[9], r[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const Cx<double> x = load_c<double>(p + 3 * (a ^ up) + c), y = load_c<double>(p + 3 * (b ^ up) + c);
+    const Cx<double> t = rot ? ti(y) : y;
+    h[c] = minus ? x - t : x + t;
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int e = 0; e < 3; ++e)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) out[3 * a + c] = make_double2(acc[a][c].x, acc[a][c].y);
+    for (int c = 0; c < 3; ++c) {
+      const Cx<double> v = load_c<double>(u + (bwd ? 3 * c + e : 3 * e + c));
+      m[3 * e + c] = mk<double>(v.x, bwd ? -v.y : v.y);
+    }
+  mul_u<double>(m, h, r);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    o[(12 * d + 6 * k + 2 * c) * stride] = r[c].x;
+    o[(12 * d + 6 * k + 2 * c + 1) * stride] = r[c].y;
+  }
+}
+
+// The results of the lanes in bad, self + sc * (the sum in FP64), in the place of self in their blocks of the warp's
+// buffer smp (self: 0 none; 1; 2 with gamma_5; left: gamma_5 on the result; as in run); o: 96 reals of the warp
+template <bool COMPACT, typename Nbr>
+__device__ __noinline__ void sites_fp64(char *smp, double *o, const double2 *U, const double2 *src, long long VL, int s,
+                                        bool g5, Nbr nbr, int self, bool left, double sc, unsigned bad) {
+  const int lane = threadIdx.x & 31;
+  auto get = [&](const double2 *m, int i) {
+    const double2 x = m[self == 2 ? (i + 6) % 12 : i];
+    return self == 0 ? make_double2(0.0, 0.0) : self == 1 ? x : make_double2(-x.x, -x.y);
+  };
+  auto put = [&](double2 *m, int i, double2 x, Cx<double> v) {
+    const double2 y = make_double2(fma(sc, v.x, x.x), fma(sc, v.y, x.y));
+    m[left ? (i + 6) % 12 : i] = left ? make_double2(-y.x, -y.y) : y;
+  };
+  if (__popc(bad) > FEW) {
+    if (!(bad >> lane & 1)) return;
+    Cx<double> acc[4][3];
+    hop_fp64<COMPACT>(U, src, VL, s, g5, nbr, acc);
+    double2 *m = (double2 *)(smp + lane * SITE_BYTES), x[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) x[i] = get(m, i);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) put(m, i, x[i], acc[i / 3][i % 3]);
+    return;
+  }
+  for (unsigned todo = bad; todo; todo &= todo - 1) {
+    const int b = __ffs(todo) - 1, sb = __shfl_sync(0xffffffffu, s, b);
+    int n = 0;
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+      const int nb = __shfl_sync(0xffffffffu, nbr(d), b);
+      if (d == lane >> 1) n = nb;
+    }
+    if (lane < 16) half_fp64<COMPACT>(U, src, VL, sb, n, g5, lane >> 1, lane & 1, o, 1);
+    __syncwarp();
+    double2 *m = (double2 *)(smp + b * SITE_BYTES), x = make_double2(0.0, 0.0);
+    if (lane < 12) x = get(m, lane);
+    __syncwarp();
+    if (lane < 12) put(m, lane, x, sum_halves(o, 1, lane / 3, lane % 3));
+    __syncwarp();
+  }
 }
 
 // Neighbours of a site on a periodic Lx x Ly x Lz x Lt lattice
@@ -417,7 +543,7 @@ struct Torus {
 };
 
 // Shared bytes of a block of 128 threads in run
-template <int SPLIT> constexpr int SMEM_BYTES = SPLIT == 1 ? 4 * WARP_BYTES : WARP_BYTES + 4 * 24 * 32 * 8;
+template <int SPLIT> constexpr int SMEM_BYTES = SPLIT == 1 ? 4 * (WARP_BYTES + 96 * 8) : WARP_BYTES + 4 * 24 * 32 * 8;
 
 // One application for this thread: out[out_i] = self[self_i] + coef * hopping term (self may be NULL; the
 // gamma_5 flags: on the hopping input, on self, on the result).  src: the canonical field f was
@@ -442,32 +568,44 @@ __device__ __forceinline__ void run(char *smem, const double2 *U, const Links &L
   const double k = A.E > 1080 ? sc * __hiloint2double((A.E - 2101 + 1023) << 20, 0) : 0.0;
   double2 *m = st.mine();
   if constexpr (SPLIT == 1) {
-    double2 p[12];
     wait_all();
     __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 12; ++i)
-      p[i] = !self ? make_double2(0.0, 0.0) : self_g5 ? make_double2(-m[(i + 6) % 12].x, -m[(i + 6) % 12].y) : m[i];
-    __syncwarp();
     if (!A.bad) {
+      double2 p[12];
+#pragma unroll
+      for (int i = 0; i < 12; ++i)
+        p[i] = !self ? make_double2(0.0, 0.0) : self_g5 ? make_double2(-m[(i + 6) % 12].x, -m[(i + 6) % 12].y) : m[i];
 #pragma unroll
       for (int i = 0; i < 12; ++i) {
         p[i].x = fma(k, (double)A.v[i / 3][i % 3][0], p[i].x);
         p[i].y = fma(k, (double)A.v[i / 3][i % 3][1], p[i].y);
       }
-    } else {
-      hop_fp64<COMPACT>(U, src, VL, s, g5, nbr, m);
 #pragma unroll
-      for (int i = 0; i < 12; ++i) p[i] = make_double2(fma(sc, m[i].x, p[i].x), fma(sc, m[i].y, p[i].y));
+      for (int i = 0; i < 12; ++i) m[i] = left_g5 ? make_double2(-p[(i + 6) % 12].x, -p[(i + 6) % 12].y) : p[i];
     }
-#pragma unroll
-    for (int i = 0; i < 12; ++i) m[i] = left_g5 ? make_double2(-p[(i + 6) % 12].x, -p[(i + 6) % 12].y) : p[i];
+    const unsigned bad = __ballot_sync(0xffffffffu, A.bad);
+    if (bad)
+      sites_fp64<COMPACT>(st.smp, (double *)(smem + 4 * WARP_BYTES) + 96 * warp, U, src, VL, s, g5, nbr,
+                          !self ? 0 : self_g5 ? 2 : 1, left_g5, sc, bad);
     __syncwarp();
     st.store<SPLIT>(out, out_i);
   } else {
     long long *red = (long long *)(smem + WARP_BYTES);   // [warp][real 24][lane 32]
+    if (!A.bad) {
 #pragma unroll
-    for (int i = 0; i < 24; ++i) red[(warp * 24 + i) * 32 + st.lane] = A.v[i / 6][i / 2 % 3][i & 1];
+      for (int i = 0; i < 24; ++i) red[(warp * 24 + i) * 32 + st.lane] = A.v[i / 6][i / 2 % 3][i & 1];
+    }
+    const unsigned bad = __ballot_sync(0xffffffffu, A.bad);   // the same in the four warps, and as with SPLIT = 1
+    if (__popc(bad) > FEW) {
+      if (A.bad) halves_fp64<COMPACT>(U, src, VL, s, g5, nbr, 2 * warp, (double *)red + warp * 24 * 32 + st.lane);
+    } else if (bad) {
+      // lane 4 i + j: half spinor j of the warp's four, of the i-th bad site
+      unsigned rest = bad;
+      for (int i = 0; i < st.lane >> 2; ++i) rest &= rest - 1;
+      const int b = rest ? __ffs(rest) - 1 : 0, sb = __shfl_sync(0xffffffffu, s, b), d = 2 * warp + (st.lane >> 1 & 1);
+      const int n0 = __shfl_sync(0xffffffffu, nbr(2 * warp), b), n1 = __shfl_sync(0xffffffffu, nbr(2 * warp + 1), b);
+      if (rest) half_fp64<COMPACT>(U, src, VL, sb, d & 1 ? n1 : n0, g5, d, st.lane & 1, (double *)red + b, 32);
+    }
     wait_all();
     __syncthreads();
     double2 p[3];
@@ -475,20 +613,18 @@ __device__ __forceinline__ void run(char *smem, const double2 *U, const Links &L
     for (int c = 0; c < 3; ++c) {
       const int i = 3 * warp + c;
       p[c] = !self ? make_double2(0.0, 0.0) : self_g5 ? make_double2(-m[(i + 6) % 12].x, -m[(i + 6) % 12].y) : m[i];
-      long long re = 0, im = 0;
+      if (!A.bad) {
+        long long re = 0, im = 0;
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        re += red[(w * 24 + 2 * i) * 32 + st.lane];
-        im += red[(w * 24 + 2 * i + 1) * 32 + st.lane];
+        for (int w = 0; w < 4; ++w) {
+          re += red[(w * 24 + 2 * i) * 32 + st.lane];
+          im += red[(w * 24 + 2 * i + 1) * 32 + st.lane];
+        }
+        p[c] = make_double2(fma(k, (double)re, p[c].x), fma(k, (double)im, p[c].y));
+      } else {
+        const Cx<double> h = sum_halves((const double *)red + st.lane, 32, warp, c);
+        p[c] = make_double2(fma(sc, h.x, p[c].x), fma(sc, h.y, p[c].y));
       }
-      if (!A.bad) p[c] = make_double2(fma(k, (double)re, p[c].x), fma(k, (double)im, p[c].y));
-    }
-    if (A.bad) {
-      double2 full[12];
-      hop_fp64<COMPACT>(U, src, VL, s, g5, nbr, full);
-#pragma unroll
-      for (int i = 0; i < 12; ++i)
-        if (i / 3 == warp) p[i % 3] = make_double2(fma(sc, full[i].x, p[i % 3].x), fma(sc, full[i].y, p[i % 3].y));
     }
     __syncthreads();
 #pragma unroll

@@ -115,7 +115,7 @@ __device__ __forceinline__ Cx<double> psplit(const double2 *U, const double2 *et
 template <int MU>
 __device__ __forceinline__ Cx<double> psplit_fx(const longlong2 *q, const int *ex, const fx::Links &L, const double2 *U,
                                                 const double2 *eta, const double2 *w, int s, int sp, long long V,
-                                                const Cx<double> eta_s[4][3]) {
+                                                const Cx<double> eta_s[4][3], bool &held) {
   const int Xu = __ldg(L.ex + MU * V + s), X1 = Xu + __ldg(ex + s) + 2, X2 = Xu + __ldg(ex + sp) + 2;
   if (max(X1, X2) <= 2900) {   // every entry in the integers' range
     // both exponents are above 1100 unless a block is zero
@@ -145,12 +145,65 @@ __device__ __forceinline__ Cx<double> psplit_fx(const longlong2 *q, const int *e
     const Cx<double> d = mk<double>(k1 * d1.x - k2 * d2.x, k1 * d1.y - k2 * d2.y);
     // eta above 2^960 leaves the range of FP64 times the integers (up to 2^62), which k1 and k2 take out
     // only here: an Inf or NaN in d1 or d2 stays one
-    if (isfinite(d.x) && isfinite(d.y)) return d;
+    held = isfinite(d.x) && isfinite(d.y);
+    return d;
   }
-  Cx<double> ws[4][3];
-  load_spinor<double, false>(w + 12LL * s, ws);
-  return psplit<MU>(U, eta, w, s, sp, V, eta_s, ws);
+  held = false;
+  return mk<double>(0.0, 0.0);
 }
+
+// The FP64 form of the same by one lane, where many of the warp's sites need it
+template <int MU>
+__device__ __noinline__ Cx<double> psplit_lane(const double2 *U, const double2 *eta, const double2 *w, int s, int sp,
+                                               long long V) {
+  Cx<double> es[4][3], ws[4][3];
+  load_spinor<double, false>(eta + 12LL * s, es);
+  load_spinor<double, false>(w + 12LL * s, ws);
+  return psplit<MU>(U, eta, w, s, sp, V, es, ws);
+}
+
+// The same for one site by the warp: lane (term, k, colour) of the first 12.  An FP64 instruction holds the pipe for 16
+// clocks however many lanes take part, so that the four directions of one site by one lane were a tail of 24 us
+// (4 fields of 12^3 x 24: 363 us, 336 so; 339 with no such sites).  Called after the loop over the sites: a vote
+// inside it costs 9 % (24^3 x 32, ten fields: 6.81 ms, 6.24 so).
+__device__ __noinline__ Cx<double> psplit_warp(int mu, const double2 *U, const double2 *eta, const double2 *w, int s,
+                                               int sp, long long V) {
+  const int lane = threadIdx.x & 31, second = lane / 6, k = lane / 3 % 2, c = lane % 3;
+  Cx<double> d = mk<double>(0.0, 0.0);
+  if (lane < 12) {
+    // upper pair of (1 + g) at the first term, (1 - g) at the second; see half_spinor
+    const double2 *x = w + 12LL * (second ? sp : s), *e = eta + 12LL * (second ? s : sp), *u = U + (mu * V + s) * 9;
+    const int a = mu == 3 ? (second ? 2 + k : k) : k, b = mu == 3 ? a : mu == 2 ? 2 + k : 3 - k;
+    const bool plus = (second != 0) != (mu != 0 && k == 1);
+    auto half = [&](const double2 *p, int col) {
+      const Cx<double> v = load_c<double>(p + 3 * a + col), l = load_c<double>(p + 3 * b + col);
+      const Cx<double> q = mu == 1 ? l : ti(l);
+      return mu == 3 ? v : plus ? v + q : v - q;
+    };
+    Cx<double> r = mk<double>(0.0, 0.0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const Cx<double> h = half(x, j), m = load_c<double>(u + (second ? 3 * c + j : 3 * j + c));
+      const double my = second ? m.y : -m.y;
+      r.x = fma(m.x, h.x, r.x);
+      r.x = fma(-my, h.y, r.x);
+      r.y = fma(m.x, h.y, r.y);
+      r.y = fma(my, h.x, r.y);
+    }
+    const Cx<double> h = half(e, c);
+    d = mk<double>(fma(h.x, r.x, h.y * r.y), fma(h.x, r.y, -(h.y * r.x)));
+    if (second) d = neg(d);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    d.x += __shfl_xor_sync(0xffffffffu, d.x, o);
+    d.y += __shfl_xor_sync(0xffffffffu, d.y, o);
+  }
+  d.x = __shfl_sync(0xffffffffu, d.x, 0);
+  d.y = __shfl_sync(0xffffffffu, d.y, 0);
+  return mu == 3 ? d + d : d;
+}
+
 
 // partial[((r * Lt + t) * nchunk + chunk) * 9 + op]; grid (nchunk * Lt, nrhs).
 // Bound by FP64 issue (two operations per clock and SM): 152 operations of the local densities, 924 of
@@ -176,6 +229,8 @@ __global__ void __launch_bounds__(CBT) contract_kernel(const double2 *__restrict
   KSum acc[18];
 #pragma unroll
   for (int q = 0; q < 18; ++q) acc[q].init();
+  // FX: the first site of this thread with point-split terms that are left to the warp at the end, 16 i + directions
+  unsigned rec = 0;
   for (int i = i0 + threadIdx.x; i < i1; i += CBT) {
     const int s = t * Vs + i;
     const int x = i % Lx, y = (i / Lx) % Ly, z = i / (Lx * Ly);
@@ -201,10 +256,23 @@ __global__ void __launch_bounds__(CBT) contract_kernel(const double2 *__restrict
     const int tp = (t + 1 == Lt) ? s - (Lt - 1) * Vs : s + Vs;
     auto split_term = [&](auto mu, int sp) {
       constexpr int MU = decltype(mu)::value;
-      if constexpr (FX)
-        d = psplit_fx<MU>(f.q + (long long)r * fx::blocks32(V) * 384, f.ex + (long long)r * V, L, U, er, wr, s, sp, V, es);
-      else
+      if constexpr (FX) {
+        bool held;
+        d = psplit_fx<MU>(f.q + (long long)r * fx::blocks32(V) * 384, f.ex + (long long)r * V, L, U, er, wr, s, sp, V, es,
+                          held);
+        if (!held) {
+          if (rec == 0 || rec >> 4 == (unsigned)i) {
+            rec |= (unsigned)i << 4 | 1u << MU;
+            d = mk<double>(0.0, 0.0);
+          } else {
+            Cx<double> wv[4][3];
+            load_spinor<double, false>(wr + 12LL * s, wv);
+            d = psplit<MU>(U, er, wr, s, sp, V, es, wv);
+          }
+        }
+      } else {
         d = psplit<MU>(U, er, wr, s, sp, V, es, ws);
+      }
       acc[10 + 2 * MU].add(kappa * d.x);
       acc[11 + 2 * MU].add(kappa * d.y);
     };
@@ -212,6 +280,39 @@ __global__ void __launch_bounds__(CBT) contract_kernel(const double2 *__restrict
     split_term(std::integral_constant<int, 1>{}, yp);
     split_term(std::integral_constant<int, 2>{}, zp);
     split_term(std::integral_constant<int, 3>{}, tp);
+  }
+  if constexpr (FX) {
+    const unsigned left = __ballot_sync(0xffffffffu, rec != 0);
+    if (left) {
+      const int step[4] = {1, Lx, Lx * Ly, Vs}, len[4] = {Lx, Ly, Lz, Lt};
+      auto rest = [&](auto mu) {
+        constexpr int MU = decltype(mu)::value;
+        auto next = [&](int s) { return s / step[MU] % len[MU] + 1 == len[MU] ? s - (len[MU] - 1) * step[MU] : s + step[MU]; };
+        const bool mine = (rec >> MU & 1u) != 0;
+        Cx<double> d = mk<double>(0.0, 0.0);
+        if (__popc(left) > fx::FEW) {
+          const int s = t * Vs + (int)(rec >> 4);
+          if (mine) d = psplit_lane<MU>(U, er, wr, s, next(s), V);
+        } else {
+          for (unsigned todo = left; todo; todo &= todo - 1) {
+            const int b = __ffs(todo) - 1;
+            const unsigned rb = __shfl_sync(0xffffffffu, rec, b);
+            if ((rb >> MU & 1u) == 0) continue;
+            const int s = t * Vs + (int)(rb >> 4);
+            const Cx<double> v = psplit_warp(MU, U, er, wr, s, next(s), V);
+            if ((int)(threadIdx.x & 31) == b) d = v;
+          }
+        }
+        if (mine) {
+          acc[10 + 2 * MU].add(kappa * d.x);
+          acc[11 + 2 * MU].add(kappa * d.y);
+        }
+      };
+      rest(std::integral_constant<int, 0>{});
+      rest(std::integral_constant<int, 1>{});
+      rest(std::integral_constant<int, 2>{});
+      rest(std::integral_constant<int, 3>{});
+    }
   }
   __shared__ double red[CBT / 32][18];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -138,3 +138,23 @@ def test_contract_with_a_non_finite_entry(what, bad):
     got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
     assert not fin.all() and np.array_equal(np.isfinite(got), fin)
     assert np.abs(got - clean)[fin].max() <= 1e-13 * np.abs(clean).max()
+
+
+@pytest.mark.parametrize("kind", ["within a site", "sites", "point"])
+def test_both_launch_forms_give_the_same_bits(kind):
+    """Ten fields (a thread per site) and each of them alone (four warps per 32 sites), sites in FP64 among them."""
+    from paper_1903_06986_gb300 import lqcd
+    torch = pytest.importorskip("torch")
+    dims, n = (8, 8, 8, 16), 10
+    ctx, eo = context(dims), lqcd.EvenOddContext(dims)
+    U, psi = dev(links(dims, "su3")), spread(dims, n, kind)
+    psi[:, :5] = field(dims, n, 11)[:, :5]                 # timeslices of entries that the integers hold
+    psi = dev(psi)
+    for flag in range(4):
+        whole = ctx.wilson_apply(U, KAPPA, psi, flags=flag)
+        for r in (0, 7):
+            assert torch.equal(ctx.wilson_apply(U, KAPPA, psi[r:r + 1].contiguous(), flags=flag)[0], whole[r]), (flag, r)
+    e, o = eo.split(psi)
+    for x, par in ((o, 0), (e, 1)):
+        whole = eo.hop(U, x, par)
+        assert torch.equal(eo.hop(U, x[3:4].contiguous(), par)[0], whole[3])
