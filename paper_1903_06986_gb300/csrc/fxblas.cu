@@ -8,12 +8,14 @@
 //
 // Inner products: the 12 components of a site are summed exactly as integers at the exponent X_V + X_w of
 // the site (w is converted once per group of vectors), then added to an FP64 sum per thread: four FP64
-// operations per site instead of 48.  The kept unit is 2^-56 of the largest product of the site, below
-// the rounding of one FP64 product of that size.
+// operations per site instead of 48.  The unit kept is 2^-54 to 2^-56 (by the mantissas) of
+// the product of the largest entries; a real has 24 dropped low products of at most a quarter unit (6 units; about
+// one half with random signs), where the FP64 chain rounds 24 times.
 // Updates: sum_i V_i h_i of a site is one integer per real, at an exponent that all vectors of the sum
-// share (found in a first pass over the exponents alone); V_i is shifted to it.  The kept unit is 2^-55 of
-// the largest |V_i h_i| of the site and one FP64 multiply-add per real ends the sum, where the FP64
-// chain rounds 2 nvec times.
+// share (found in a first pass over the exponents alone); V_i is shifted to it.  The unit kept is 2^-53 to
+// 2^-55 of the largest |V_i h_i| of the site, coarser where 64 and more vectors of that size need room (the exponent
+// of the sum grows with log2 of their number less 6); two low products of at most a quarter unit are dropped per
+// vector, and one FP64 multiply-add per real ends the sum, where the FP64 chain rounds 2 nvec times.
 // Sites with an entry that the integers cannot hold (FX_BAD, products near the ends of the exponent range)
 // and non-finite coefficients take the FP64 sums, from the FP64 basis beside the integers.
 #include <algorithm>

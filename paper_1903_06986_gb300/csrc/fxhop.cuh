@@ -2,8 +2,8 @@
 //
 // What bounds the plain form: an SM issues two FP64 operations per clock and the stencil needs
 // about 860 per (site, right-hand side): 430 clocks, 6.6 ms for ten fields of 24^3 x 32, against
-// 0.3 ms of HBM traffic.  The same SM issues 64 32 x 32 -> 64-bit integer multiply-adds per clock
-// (measured: 59 mad.wide.s32 against 1.7 to 2 DFMA), so the stencil runs on integers:
+// 0.3 ms of HBM traffic.  The same SM issues 32 32 x 32 -> 64-bit integer multiply-adds per clock
+// (against 1.7 to 2 DFMA measured), 1824 per site, 57 clocks, so the stencil runs on integers:
 //   * fx_convert_kernel turns a field into integers once per application: a real x of a site whose
 //     largest real has biased exponent X becomes q = x 2^(1082 - X), |q| < 2^60 (the mantissa
 //     shifted by X - exponent; all 53 bits survive down to 2^-7 of the site's largest entry).
@@ -13,13 +13,15 @@
 //   * spin projections are 64-bit additions; a half spinor is shifted right by E - X_u - X - 1 to the
 //     exponent E >= X_u + X + 2 that all eight directions of the thread share, leaving |h| < 2^60;
 //   * both factors are split as hi 2^32 + lo with signed lo: a product needs hi hi and
-//     (hi lo + lo hi) / 2^32, three mad.wide; lo lo / 2^64 is below half the unit that is kept.  Six
+//     (hi lo + lo hi) / 2^32, three mad.wide; lo lo / 2^64, a quarter of the unit that is kept at most, is dropped.  Six
 //     products are summed exactly (|hi hi| sum < 2^59, |mixed| sum < 2^63), the mixed sum enters by
 //     its high word (one mad.wide), and the eight directions are added as 64-bit integers (< 2^62).
 // FP64 arithmetic is left with the last p - kappa acc (24 conversions, 24 DFMA).
-// Error: the kept unit is 2^-56 of (largest link entry x largest half spinor entry around the site),
-// below the roundings of the FP64 chain it replaces (tests/test_gpu_fxhop.py compares both with
-// extended precision).
+// Error: with the exponent of the largest product around the site, the unit kept is 2^-53 to 2^-55 (by the
+// mantissas) of largest link entry x largest field entry.  A real of the result has 48 dropped lo lo, at most a
+// quarter of it each (12 units; random signs make it about one), 8 roundings of half a unit and the truncated
+// inputs.  Measured against extended precision the error is below that of the FP64 chain
+// (tests/test_gpu_fxhop.py).
 // Sites or links with a NaN, an Inf, or a scale near the ends of the exponent range carry the exponent
 // FX_BAD, those with entries far apart FX_WIDE; the threads that meet one run the plain FP64 stencil.
 //
@@ -550,7 +552,7 @@ template <int SPLIT> constexpr int SMEM_BYTES = SPLIT == 1 ? 4 * (WARP_BYTES + 9
 // converted from.  A lane with out_i < 0 (its site repeats another's) helps and stores nothing.
 // SPLIT = 1: one thread per site.  SPLIT = 4, for fields that leave most of the chip idle: the four
 // warps of a block share 32 sites, warp w adds the two directions of mu = w and finishes spin w; the
-// sums are integers at one exponent, so both forms give the same bits.
+// sums are integers at one exponent, so both forms give the same bits, and FP64 sites add the directions in one order.
 template <int SPLIT, bool COMPACT, typename Nbr>
 __device__ __forceinline__ void run(char *smem, const double2 *U, const Links &L, long long VL, int s, const Nbr &nbr,
                                     const Field &f, int r, long long S, const double2 *src, bool g5,

@@ -511,8 +511,8 @@ struct TcArgs {
   int nb;                  // mode 1: complex columns (column 2r real part, 2r + 1 imaginary part)
   double *out;             // mode 1: out[r * m_valid + m]
   int g5;                  // mode 1: write gamma_5 times the product (rows: 24 reals per site, pairs of spins
-                           // exchanged and negated); a pass of its own was 0.30 ms of the 3.08 ms projection
-                           // of 16 fields of 16^3 x 32 on 160 vectors
+                           // exchanged and negated); a pass of its own took 0.18 ms of the 3.07 ms projection
+                           // of 16 fields of 16^3 x 32 on 160 vectors (2.89 without)
   int *err;
   unsigned long long wait_ns;  // bound of every pipeline wait (the context's setting)
   int stop_after;          // failure injection: the loader stops after this many chunks (-1: never)

@@ -222,8 +222,9 @@ __global__ void __launch_bounds__(FX_BS) fx_links_convert_kernel(const double2 *
 
 // FP64 operator: M, M g5 (bit r of g5mask for the masked form), M^dag or P for right-hand side r =
 // blockIdx.x % nrhs (fastest, so that the links of one site block are shared through L2).
-// Four blocks per SM (128 registers): ten fields of 24^3 x 32 in 1.63 ms, 1.71 ms with three and 1.79 ms
-// with five; the integer multiply-adds alone (1824 per site, 32 per clock and SM) take 0.86 ms.
+// Four blocks per SM (128 registers; the form with a thread per site spills 124 bytes): ten fields of
+// 24^3 x 32 in 1.59 ms (1.63 with 504 bytes of spills, when three blocks took 1.71 ms and five 1.79); the integer multiply-adds alone (1824 per site, 32 per
+// clock and SM) take 0.86 ms at 1.92 GHz.
 enum { FX_G5IN = 1, FX_G5LEFT = 2, FX_HOP = 4, FX_MASK = 8 };
 template <int SPLIT>
 __global__ void __launch_bounds__(FX_BS, 4) wilson_fx_kernel(const double2 *__restrict__ U, fx::Links L, fx::Field f,
