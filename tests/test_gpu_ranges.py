@@ -158,3 +158,57 @@ def test_both_launch_forms_give_the_same_bits(kind):
     for x, par in ((o, 0), (e, 1)):
         whole = eo.hop(U, x, par)
         assert torch.equal(eo.hop(U, x[3:4].contiguous(), par)[0], whole[3])
+
+
+def few(dims, n, sites):
+    """Gaussian fields with one entry 1e-9 of the others at the listed (t, z, y, x), and the mask of their neighbours."""
+    psi, hit = field(dims, n, 12), np.zeros(field(dims, 1, 0).shape[1:5], bool)
+    for i, at in enumerate(sites):
+        psi[(slice(None),) + at + (i % 4, i % 3)] *= 1e-9
+        hit[at] = True
+    near = np.zeros_like(hit)
+    for axis in range(4):
+        near |= np.roll(hit, 1, axis) | np.roll(hit, -1, axis)
+    return psi, near
+
+
+FEW_SITES = [[(3, 2, 4, 5)], [(0, 0, 0, 0), (0, 0, 2, 1), (7, 1, 1, 1), (15, 7, 7, 7)],
+             [(5, 5, y, x) for y in (0, 2, 4) for x in (0, 3, 6)]]
+
+
+@pytest.mark.parametrize("n", [1, 6])
+@pytest.mark.parametrize("sites", FEW_SITES)
+def test_operator_with_few_sites_outside_the_integers(sites, n):
+    """One, some and many lanes of a warp in FP64, entry by entry to its roundings; all forms of the operator."""
+    from paper_1903_06986_gb300 import lqcd
+    dims = (8, 8, 8, 16)
+    ctx, eo = context(dims), lqcd.EvenOddContext(dims)
+    U = links(dims, "su3")
+    psi, near = few(dims, n, sites)
+    g5 = lambda a: -a[..., [2, 3, 0, 1], :]
+    ext = lambda a: L.wilson(U.astype(np.clongdouble), np.longdouble(KAPPA), a.astype(np.clongdouble))
+    top, _ = around(dims, psi)
+    m = np.where(near[..., None, None], 0.0, top)
+    hopped, sum_abs = L.hop(U.astype(np.clongdouble), psi.astype(np.clongdouble)), abs_hop(U, psi)
+    tol = 40 * EPS * (np.abs(psi) + KAPPA * sum_abs) + KAPPA * 8 * 6 * 2.0 ** -54 * m
+    tol5 = 40 * EPS * (np.abs(g5(psi)) + KAPPA * abs_hop(U, g5(psi))) + KAPPA * 8 * 6 * 2.0 ** -54 * m
+    for flag, ref, t in ((lqcd.APPLY_M, ext(psi), tol), (lqcd.APPLY_G5R, ext(g5(psi)), tol5),
+                         (lqcd.APPLY_DAG, g5(ext(g5(psi))), np.abs(g5(tol5))),
+                         (lqcd.APPLY_HOP, hopped, 40 * EPS * sum_abs + 8 * 6 * 2.0 ** -54 * m)):
+        got = host(ctx.wilson_apply(dev(U), KAPPA, dev(psi), flags=flag))
+        assert (np.abs(got - ref) <= t).all(), flag
+    e, o = eo.split(dev(psi))
+    want, bound = (eo.split(dev(a.astype(complex))) for a in (hopped, 41 * EPS * sum_abs + 8 * 6 * 2.0 ** -54 * m))
+    for x, par in ((o, 0), (e, 1)):
+        assert (np.abs(host(eo.hop(dev(U), x, par)) - host(want[par])) <= host(bound[par]).real).all(), par
+
+
+@pytest.mark.parametrize("n", [1, 6])
+@pytest.mark.parametrize("sites", FEW_SITES)
+def test_contract_with_few_sites_outside_the_integers(sites, n):
+    dims = (8, 8, 8, 16)
+    ctx = context(dims)
+    U, eta, (w, _) = links(dims, "su3"), field(dims, n, 13), few(dims, n, sites)
+    got = ctx.contract(dev(U), 0.14, dev(eta), dev(w))
+    ref = O.per_t(O.densities(U, 0.14, eta, w)).transpose(1, 0, 2)
+    assert rel_err(got, ref) < 1e-13
