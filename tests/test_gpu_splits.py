@@ -112,3 +112,19 @@ def test_hop_traces_by_site_at_its_last_order():
     for k in range(K):
         scale = max(np.abs(want[k]).max(), 12.0 * np.prod(dims[:3]) * 2.0 ** k)
         assert np.abs(got[k] - want[k]).max() <= 1e-13 * scale, k
+
+
+@pytest.mark.parametrize("recon", [12, 18])
+def test_packed_block_sizes(recon):
+    """FP32 fields of 12^3 x 24 in blocks of 128 threads (four fields, a wave), of 64 (two; ten) and of a ragged lattice:
+    the same bits in every block."""
+    torch = pytest.importorskip("torch")
+    for dims, sizes in (((12, 12, 12, 24), (10, 4, 2)), ((13, 11, 15, 17), (5, 2))):
+        ctx = context(dims)
+        Up = ctx.pack_links_f32(dev(synth.su3_links(dims, 0.4323, 13)), recon)
+        p = ctx.pack_f32(dev(fields(dims, sizes[0], 14)))
+        for flag in range(4):
+            whole = ctx.wilson_apply_packed(Up, recon, 0.137, p, flags=flag)
+            for n in sizes[1:]:
+                part = ctx.wilson_apply_packed(Up, recon, 0.137, p[:n].contiguous(), flags=flag)
+                assert torch.equal(part, whole[:n]), (dims, n, flag)
